@@ -529,7 +529,7 @@ int moss_selftest_bounded_wait(void* cuda_stream);
  * without waiting.
  *
  * It allocates nothing: the scan's look-back words live in one file-scope
- * static device array of 32 KiB (plus 256 bytes), held by every GPU that
+ * static device array of 8 KiB (plus 256 bytes), held by every GPU that
  * loads the library until the process exits.  Limit: n_lanes <=
  * MOSS_NOALLOC_MAX_LANES; larger sizes return MOSS_EINVAL.  The first call on
  * a device looks up that array's device address (and the SM count) with the

@@ -133,3 +133,29 @@ def test_noalloc_flags_negative_size():
 def test_noalloc_rejects_oversize():
     binding.load()
     assert binding.moss_lane_offsets_noalloc(binding.NOALLOC_MAX_LANES + 1, 1, 1, 1, 1, 1) == binding.MOSS_EINVAL
+
+
+@pytest.mark.parametrize("n_lanes", [1, 3, 4, 5, 127, 128, 4095, 4096, 4097, 8193])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_noalloc_tile_edges_and_alignment(n_lanes, shift):
+    """Sizes around a thread's four lanes and a tile's 4,096, with arrays at 16-byte boundaries (16-byte accesses)
+    and one element off (single accesses): exact, and nothing is written past the ends."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    args, want_off, want_lb = _noalloc_random(n_lanes, 29, torch)
+
+    def at(x, n):
+        out = torch.full((n + 12,), -7, dtype=torch.int32, device="cuda")
+        if x is not None:
+            out[4 + shift:4 + shift + n] = x
+        return out
+
+    ins = [at(x, len(x)) for x in args]
+    nxt, lb = at(None, n_lanes + 1), at(None, n_lanes)
+    ptr = [t.data_ptr() + 4 * (4 + shift) for t in (*ins, nxt, lb)]
+    assert binding.moss_lane_offsets_noalloc(n_lanes, *ptr, torch.cuda.current_stream().cuda_stream) == binding.MOSS_OK
+    torch.cuda.synchronize()
+    for got, want in ((nxt.cpu().numpy(), want_off), (lb.cpu().numpy(), want_lb)):
+        assert np.array_equal(got[4 + shift:4 + shift + len(want)], want)
+        assert (got[:4 + shift] == -7).all() and (got[4 + shift + len(want):] == -7).all()
