@@ -21,6 +21,14 @@ using namespace moss;
 
 constexpr int RB_WORDS = M_NFIELDS + 2;  // readback slot: metric record, step, error word
 
+// Getter outputs up to this size go through a pinned buffer of the handle and
+// a copy by the host: one wait in all, where a copy to pageable memory waits
+// for the kernel and then for itself (the queues of 1,200 bytes of lanes
+// 36.3 -> 24.7 us, of 160 KB 41.6 -> 35.2 us, waits included).  Larger ones
+// are copied straight to the caller's memory, at C2C speed (170 GB/s; the
+// host copies about 14 GB/s).
+constexpr size_t GETTER_PINNED = 192 << 10;
+
 namespace {
 
 struct SnapBufs {
@@ -121,13 +129,13 @@ struct MossHandle {
     unsigned long long* d_gap_head = nullptr;
     int n_lane_tiles = 0, max_slot_tiles = 0, n_junc_chunks = 0;
     Counters* d_cnt = nullptr;  // [2]: per parity; d_cnt[0].err holds the device error bits
-    int32_t* d_stage = nullptr;          // setter staging (2 * n_junctions)
-    int32_t* h_stage = nullptr;          // pinned host staging of setter arguments (2 * n_junctions)
-    cudaEvent_t stage_free = nullptr;    // recorded after the last copy out of h_stage
+    int32_t* h_stage = nullptr;          // pinned host staging of setter arguments (2 * n_junctions), read by the setter's kernel
+    cudaEvent_t stage_free = nullptr;    // recorded after the last kernel that reads h_stage
     // pinned readback: per slot a metric record, its step and the error word;
     // slots [0, MOSS_METRIC_SLOTS) serve moss_metrics_enqueue/read, the last
     // one moss_get_metrics
     long long* h_rb = nullptr;
+    void* h_out = nullptr;               // pinned: outputs of the getters up to GETTER_PINNED bytes
     cudaEvent_t rb_ev[MOSS_METRIC_SLOTS] = {};
     int rb_scen[MOSS_METRIC_SLOTS] = {};
     bool rb_pending[MOSS_METRIC_SLOTS] = {};
@@ -493,7 +501,7 @@ int junction_init(MossHandle* h, int j0, int j1) {
 template <typename Real>
 void enqueue_set_signal(MossHandle* h, int n, int policy) {
     Ctx<Real> c = make_ctx<Real>(h, h->parity);
-    k_set_signal<Real><<<(n + 255) / 256, 256, 0, h->stream>>>(c, n, h->d_stage, h->d_stage + n, policy);
+    k_set_signal<Real><<<(n + 255) / 256, 256, 0, h->stream>>>(c, n, h->h_stage, h->h_stage + n, policy);
 }
 
 void destroy_graphs(MossHandle* h) {
@@ -794,10 +802,10 @@ int device_setup(MossHandle* h, void* stream) {
     c0[0].tag = 1;
     TRY(upload(h, &h->d_cnt, c0));
     TRY(upload(h, &h->d_bar, std::vector<unsigned>(2, 0u)));
-    TRY(dalloc(h, &h->d_stage, 2 * std::max(NJ, 1)));
     CK(cudaHostAlloc((void**)&h->h_stage, sizeof(int32_t) * 2 * std::max(NJ, 1), cudaHostAllocDefault));
     CK(cudaHostAlloc((void**)&h->h_rb, sizeof(long long) * RB_WORDS * (MOSS_METRIC_SLOTS + 1),
                      cudaHostAllocDefault));
+    CK(cudaHostAlloc(&h->h_out, GETTER_PINNED, cudaHostAllocDefault));
     for (int k = 0; k < MOSS_METRIC_SLOTS; ++k)
         CK(cudaEventCreateWithFlags(&h->rb_ev[k], cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&h->stage_free, cudaEventDisableTiming));
@@ -1129,22 +1137,33 @@ void free_all(MossHandle* h) {
     h->h_stage = nullptr;
     if (h->h_rb) cudaFreeHost(h->h_rb);
     h->h_rb = nullptr;
+    if (h->h_out) cudaFreeHost(h->h_out);
+    h->h_out = nullptr;
     for (int k = 0; k < MOSS_METRIC_SLOTS; ++k)
         if (h->rb_ev[k]) cudaEventDestroy(h->rb_ev[k]);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     h->stream = nullptr;
 }
 
-// copies of scenario s's metric record, its step and the device error word,
-// behind the work queued so far, into readback slot `slot`
+// scenario s's metric record, its step and the device error word, as they are
+// behind the work queued so far, into readback slot `slot` (one launch that
+// stores to the pinned slot; three copies had cost 8.6 us of stream time)
 int enqueue_readback(MossHandle* h, int s, int slot) {
-    long long* M = h->h_rb + (size_t)slot * RB_WORDS;
-    CK(cudaMemcpyAsync(M, h->d_metrics + (size_t)s * M_NFIELDS, M_NFIELDS * sizeof(long long),
-                       cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(M + M_NFIELDS, h->d_step + s, sizeof(long long), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(M + M_NFIELDS + 1, &h->d_cnt->err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    k_readback<<<1, 32, 0, h->stream>>>(h->d_metrics + (size_t)s * M_NFIELDS, h->d_step + s, &h->d_cnt->err,
+                                        h->h_rb + (size_t)slot * RB_WORDS);
+    CK(cudaGetLastError());
     return MOSS_OK;
 }
+
+// the device error word that a getter's kernel stored in the last readback slot
+int getter_status(MossHandle* h) {
+    int err = 0;
+    std::memcpy(&err, h->h_rb + (size_t)MOSS_METRIC_SLOTS * RB_WORDS + M_NFIELDS + 1, sizeof(int));
+    return device_status(h, err);
+}
+
+// where a getter's kernel stores the device error word
+long long* getter_err(MossHandle* h) { return h->h_rb + (size_t)MOSS_METRIC_SLOTS * RB_WORDS + M_NFIELDS + 1; }
 
 // the metrics of scenario s from a completed readback slot
 int readback_metrics(MossHandle* h, int s, int slot, MossMetrics* out) {
@@ -1179,57 +1198,54 @@ int scen_metrics(MossHandle* h, int s, MossMetrics* out) {
 }
 
 template <typename Real>
-void unpack_a(const std::vector<char>& raw, int n, std::vector<int32_t>& lane, std::vector<int32_t>& id,
-              std::vector<double>& sv, std::vector<double>& vv) {
-    const RecA<Real>* a = (const RecA<Real>*)raw.data();
-    for (int k = 0; k < n; ++k) {
-        lane[k] = a[k].lane; id[k] = a[k].id; sv[k] = (double)a[k].s; vv[k] = (double)a[k].v;
+int scen_state_of(MossHandle* h, int s, MossState* out) {
+    const int nv = h->scen_nv[s], v0 = h->scen_veh_off[s], lo = h->scen_lane_off[s];
+    Ctx<Real> c = make_ctx<Real>(h, h->parity);
+    // the per-vehicle arrays are laid out on the device in the candidate
+    // records (96 B or more per vehicle, free between steps), then each goes
+    // to the caller's array in one copy
+    StateOut o;
+    o.s = (double*)h->d_cands;
+    o.v = o.s + nv;
+    o.status = (int32_t*)(o.v + nv);
+    o.lane = o.status + nv;
+    o.rc = o.lane + nv;
+    o.flags = o.rc + nv;
+    const int nb = std::max(1, std::min((nv + 255) / 256, h->sm_count * 8));
+    k_state_fill<Real><<<nb, 256, 0, h->stream>>>(c, s, v0, nv, o, getter_err(h));
+    if (nv > 0) {
+        k_state_gather<Real><<<nb, 256, 0, h->stream>>>(c, v0, nv, lo, h->scen_nl[s], o);
+        CK(cudaGetLastError());
+        const size_t ni = (size_t)nv * sizeof(int32_t), nd = (size_t)nv * sizeof(double);
+        if (2 * nd + 4 * ni <= GETTER_PINNED) {
+            CK(cudaMemcpyAsync(h->h_out, o.s, 2 * nd + 4 * ni, cudaMemcpyDeviceToHost, h->stream));
+            CK(cudaStreamSynchronize(h->stream));
+            const char* q = (const char*)h->h_out;
+            std::memcpy(out->s, q, nd); q += nd;
+            std::memcpy(out->v, q, nd); q += nd;
+            std::memcpy(out->status, q, ni); q += ni;
+            std::memcpy(out->lane, q, ni); q += ni;
+            std::memcpy(out->rc, q, ni); q += ni;
+            std::memcpy(out->flags, q, ni);
+            return getter_status(h);
+        }
+        CK(cudaMemcpyAsync(out->s, o.s, nd, cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaMemcpyAsync(out->v, o.v, nd, cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaMemcpyAsync(out->status, o.status, ni, cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaMemcpyAsync(out->lane, o.lane, ni, cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaMemcpyAsync(out->rc, o.rc, ni, cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaMemcpyAsync(out->flags, o.flags, ni, cudaMemcpyDeviceToHost, h->stream));
     }
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(h->stream));
+    return getter_status(h);
 }
 
 int scen_state(MossHandle* h, int s, MossState* out) {
     if (!out || !out->status || !out->lane || !out->s || !out->v || !out->rc || !out->flags)
         return fail(h, MOSS_EINVAL, "null state array");
     if (s < 0 || s >= h->n_scen) return fail(h, MOSS_EINVAL, "scenario index out of range");
-    CK(cudaStreamSynchronize(h->stream));
-    Counters c;
-    CK(cudaMemcpy(&c, h->d_cnt + h->parity, sizeof(c), cudaMemcpyDeviceToHost));
-    const int n = c.n_cur, NV = h->n_veh;
-    const SnapBufs& b = h->snap[h->parity];
-    const size_t ra = reca_size(h->precision);
-    std::vector<char> raw((size_t)n * ra);
-    std::vector<RecB> rb(n);
-    std::vector<int32_t> lane(n), id(n), status(NV), vflags(NV);
-    std::vector<double> sv(n), vv(n);
-    long long step = 0;
-    CK(cudaMemcpy(&step, h->d_step + s, sizeof(long long), cudaMemcpyDeviceToHost));
-    if (n > 0) {
-        CK(cudaMemcpy(raw.data(), b.a, raw.size(), cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(rb.data(), b.b, n * sizeof(RecB), cudaMemcpyDeviceToHost));
-        if (h->precision == 64) unpack_a<double>(raw, n, lane, id, sv, vv);
-        else unpack_a<float>(raw, n, lane, id, sv, vv);
-    }
-    CK(cudaMemcpy(status.data(), h->d_vstatus, NV * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(vflags.data(), h->d_vflags, NV * 4, cudaMemcpyDeviceToHost));
-    const int v0 = h->scen_veh_off[s], v1 = v0 + h->scen_nv[s];
-    const int lo = h->scen_lane_off[s];
-    const long long tag = (step - 1) & 0xFFFFFF;
-    for (int g = v0; g < v1; ++g) {
-        const int i = g - v0;
-        out->status[i] = status[g];
-        out->lane[i] = -1; out->s[i] = 0; out->v[i] = 0; out->rc[i] = 0;
-        out->flags[i] = ((long long)(((unsigned)vflags[g]) >> 8) == tag && step > 0) ? (vflags[g] & 255) : 0;
-    }
-    for (int k = 0; k < n; ++k) {
-        const int g = id[k];
-        if (g < v0 || g >= v1) continue;
-        const int i = g - v0;
-        out->lane[i] = lane[k] - lo;
-        out->s[i] = sv[k];
-        out->v[i] = vv[k];
-        out->rc[i] = rb[k].rptr - h->route_span[g].x;
-    }
-    return check_device(h);
+    return h->precision == 64 ? scen_state_of<double>(h, s, out) : scen_state_of<float>(h, s, out);
 }
 
 int jl_toward_host(const MossHandle* h, int l, int out_road) {
@@ -1436,25 +1452,28 @@ int reroute(MossHandle* h, int n, const int32_t* vids, const int32_t* route_off,
 template <typename Real>
 int scen_lane_metrics(MossHandle* h, int s, int32_t* queue, double* speed) {
     Ctx<Real> c = make_ctx<Real>(h, h->parity);
-    if (queue) {
-        const int l0 = h->scen_lane_off[s], l1 = l0 + h->scen_nl[s];
-        if (l1 > l0) {
-            k_lane_queue<Real><<<(l1 - l0 + 255) / 256, 256, 0, h->stream>>>(c, l0, l1, (int32_t*)h->d_mbuf);
-            CK(cudaGetLastError());
-            CK(cudaMemcpyAsync(queue, h->d_mbuf, (size_t)(l1 - l0) * 4, cudaMemcpyDeviceToHost, h->stream));
-            CK(cudaStreamSynchronize(h->stream));
-        }
+    const int l0 = h->scen_lane_off[s], nl = queue ? h->scen_nl[s] : 0;
+    const int r0 = h->scen_road_off[s], nr = speed ? h->scen_nr[s] : 0;
+    if (nl == 0 && nr == 0) {
+        CK(cudaStreamSynchronize(h->stream));
+        return check_device(h);
     }
-    if (speed) {
-        const int r0 = h->scen_road_off[s], r1 = r0 + h->scen_nr[s];
-        if (r1 > r0) {
-            k_road_speed<Real><<<(r1 - r0 + 255) / 256, 256, 0, h->stream>>>(c, r0, r1, (double*)h->d_mbuf);
-            CK(cudaGetLastError());
-            CK(cudaMemcpyAsync(speed, h->d_mbuf, (size_t)(r1 - r0) * 8, cudaMemcpyDeviceToHost, h->stream));
-            CK(cudaStreamSynchronize(h->stream));
-        }
+    const size_t nb = nl > 0 ? (size_t)nl * sizeof(int32_t) : (size_t)nr * sizeof(double);
+    void* const to = nl > 0 ? (void*)queue : (void*)speed;
+    const bool pinned = nb <= GETTER_PINNED;
+    void* const buf = pinned ? h->h_out : h->d_mbuf;
+    if (nl > 0) {
+        k_lane_queue<Real><<<(nl + 255) / 256, 256, 0, h->stream>>>(c, l0, l0 + nl, (int32_t*)buf, getter_err(h));
+    } else {
+        const int per_block = 256 / ROAD_SPEED_THREADS;
+        k_road_speed<Real><<<(nr + per_block - 1) / per_block, 256, 0, h->stream>>>(c, r0, r0 + nr, (double*)buf,
+                                                                                    getter_err(h));
     }
-    return check_device(h);
+    CK(cudaGetLastError());
+    if (!pinned) CK(cudaMemcpyAsync(to, buf, nb, cudaMemcpyDeviceToHost, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    if (pinned) std::memcpy(to, buf, nb);
+    return getter_status(h);
 }
 
 int lane_metrics(MossHandle* h, int s, int32_t* queue, double* speed) {
@@ -1559,11 +1578,10 @@ int moss_batch_set_signal_phase(moss_t h, int scenario, int n, const int32_t* ju
         sj[k] = j0 + j;
         sp[k] = p;
     }
-    CK(cudaMemcpyAsync(h->d_stage, h->h_stage, 2 * n * 4, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaEventRecord(h->stage_free, h->stream));
     if (h->precision == 64) enqueue_set_signal<double>(h, n, POL_MANUAL);
     else enqueue_set_signal<float>(h, n, POL_MANUAL);
     CK(cudaGetLastError());
+    CK(cudaEventRecord(h->stage_free, h->stream));
     return MOSS_OK;
 }
 
@@ -1586,11 +1604,10 @@ int moss_batch_set_signal_phases(moss_t h, int n, const int32_t* scenarios, cons
         sj[k] = g;
         sp[k] = p;
     }
-    CK(cudaMemcpyAsync(h->d_stage, h->h_stage, 2 * n * 4, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaEventRecord(h->stage_free, h->stream));
     if (h->precision == 64) enqueue_set_signal<double>(h, n, POL_MANUAL);
     else enqueue_set_signal<float>(h, n, POL_MANUAL);
     CK(cudaGetLastError());
+    CK(cudaEventRecord(h->stage_free, h->stream));
     return MOSS_OK;
 }
 
@@ -1608,11 +1625,10 @@ int moss_set_signal_policy(moss_t h, int n, const int32_t* junction_ids, int32_t
         h->h_stage[k] = junction_ids[k];
         h->h_stage[n + k] = 0;
     }
-    CK(cudaMemcpyAsync(h->d_stage, h->h_stage, 2 * n * 4, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaEventRecord(h->stage_free, h->stream));
     if (h->precision == 64) enqueue_set_signal<double>(h, n, policy);
     else enqueue_set_signal<float>(h, n, policy);
     CK(cudaGetLastError());
+    CK(cudaEventRecord(h->stage_free, h->stream));
     return MOSS_OK;
 }
 

@@ -167,3 +167,42 @@ def test_schedule_out_of_range_refused():
         assert sim.schedule() == before
     sim.step(5)
     assert sim.metrics()["step"] == 5
+
+
+@pytest.mark.parametrize("n", [1, 255, 257, 6143, 6144, 6145])
+@pytest.mark.parametrize("precision", [32, 64])
+def test_state_getter_returns_what_was_set(n, precision):
+    """The state getter around the size up to which it goes through pinned memory (192 KiB, 32 bytes per vehicle):
+    exactly the state that was set, by vehicle id."""
+    net = sc.grid_network(12, 300.0, 3, 13.89)
+    veh = sc.random_demand(net, n, 100, seed=n)
+    st = sc.warm_state(net, veh, 60)
+    sim = binding.Simulation(net, veh, sc.Params(), precision=precision)
+    sim.set_state(st["status"], st["lane"], st["s"], st["v"], st["rc"], 60)
+    got = sim.state()
+    for k in ("status", "lane", "s", "v", "rc"):
+        assert np.array_equal(got[k], st[k]), k
+    assert not got["flags"].any()
+
+
+@pytest.mark.parametrize("G", [4, 40])
+def test_lane_and_road_getters_match_the_state(G):
+    """Lane queues and road speeds of a small network (through pinned memory) and of one whose lanes exceed it (copied
+    to the caller's array) against the same quantities from the state: counts exact, means to FP64 rounding."""
+    net = sc.perturbed_grid_network(G, seed=1)
+    veh = sc.random_demand(net, 300 * G, 60, seed=2, dest_pool=64)
+    sim = binding.Simulation(net, veh, sc.Params())
+    sim.step(150)
+    st = sim.state()
+    act = st["status"] == 1
+    lane, s, v = st["lane"][act], st["s"][act], st["v"][act]
+    stopped = (v < 0.1) & ~(net.lane_length.astype(np.float64)[lane] - s > 50.0)
+    assert np.array_equal(sim.lane_queue(), np.bincount(lane[stopped], minlength=net.n_lanes))
+    on_road = lane < net.n_road_lanes
+    road = net.lane_road()[lane[on_road]]
+    cnt = np.bincount(road, minlength=net.n_roads)
+    total = np.bincount(road, weights=v[on_road], minlength=net.n_roads)
+    limit = np.add.reduceat(net.lane_vmax[:net.n_road_lanes].astype(np.float64), net.road_lane_off[:-1])
+    want = np.where(cnt > 0, total / np.maximum(cnt, 1), limit / np.diff(net.road_lane_off))
+    assert np.allclose(sim.road_speed(), want, rtol=1e-12, atol=0)
+    assert stopped.any()
