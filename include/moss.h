@@ -441,9 +441,10 @@ int moss_slot_set_horizon(moss_t h, int slot, int64_t stop_at);
  * Kernel timing for measurement: when enabled, every step records CUDA
  * events around each kernel on the handle's stream (graphs are not used
  * while enabled).  moss_kernel_times returns the summed milliseconds per
- * kernel since enabling, in the order (decide, lanescan, place, resolve) —
- * the launch order is decide, resolve, lanescan, place; resolve finishes the
- * lane-change candidates — and the number of timed steps.
+ * kernel since enabling, in the order (decide, lanescan, place, resolve), and
+ * the number of timed steps.  The resolution of lane-change candidates is
+ * part of decide (resolve stays 0), and up to 200,000 vehicles the lane scan
+ * is part of place (lanescan stays 0).
  */
 int moss_set_kernel_timing(moss_t h, int enable);
 int moss_kernel_times(moss_t h, double* ms4, int64_t* steps);
@@ -451,7 +452,7 @@ int moss_kernel_times(moss_t h, double* ms4, int64_t* steps);
 /*
  * Launch form of a step (no counterpart in the paper, whose step is a
  * sequence of kernels on several streams, App. B.2): mode 0 (the default)
- * replays three kernels per step from a captured CUDA graph; mode 1 runs the
+ * replays two or three kernels per step from a captured CUDA graph; mode 1 runs the
  * whole step as one cooperative launch (every block resident at once, the
  * kernels' work as phases separated by grid-wide barriers whose waits are
  * bounded: MOSS_ETIMEOUT), also graph-replayed.  Results do not depend on
@@ -461,8 +462,9 @@ int moss_kernel_times(moss_t h, double* ms4, int64_t* steps);
  */
 int moss_set_step_mode(moss_t h, int mode);
 
-/* Kernel launches of the library per step in the current mode (3 in mode 0:
- * decide, lane scan with the conflict resolution, place; 1 in mode 1). */
+/* Kernel launches of the library per step in the current mode (mode 0: 2 up to
+ * 200,000 vehicles, decide and place; 3 above: decide, lane scan, place; mode
+ * 1: 1). */
 int moss_step_launches(moss_t h, int* out);
 
 /*
@@ -472,24 +474,25 @@ int moss_step_launches(moss_t h, int* out);
  * depend on the schedule) under candidate schedules, keeps the fastest by
  * coordinate search over, in this order: k_decide blocks per SM {3,4,5}; the
  * weight of a road-lane vehicle in the split of the snapshot into k_decide's
- * block runs {0,1,2} (a junction-lane vehicle weighs 1; 0: the weight fitted each step); k_lanescan blocks
- * per SM {1,2,4}; lanes per thread of a lane-scan tile {16,8}; k_place
- * blocks per SM {4,8,16}; the step mode {0,1} (moss_set_step_mode).  Then it
- * re-captures the step graphs.  chosen3 (may be NULL) receives the chosen
- * decide/lanescan/place blocks per SM; moss_get_schedule returns the whole schedule.
+ * block runs {0,1,2} (a junction-lane vehicle weighs 1; 0: the weight fitted each step); the weight
+ * of a lane in the tiles of k_place {1,2,4} (a slot weighs 2); those tiles at
+ * full or half size {16,8}; k_place_slots blocks per SM {4,8,16}; the step
+ * mode {0,1} (moss_set_step_mode).  Then it re-captures the step graphs.
+ * chosen3 (may be NULL) receives the chosen decide blocks per SM, lane weight
+ * and place blocks per SM; moss_get_schedule returns the whole schedule.
  */
 int moss_autotune(moss_t h, int trial_steps, int* chosen3);
 
 /*
- * The launch schedule (no counterpart in the paper): out7 / in7 = k_decide,
- * k_lanescan and k_place blocks per SM, the road-lane weight of k_decide's
- * runs (0: fitted each step from the previous step's run times, the
- * default; 1..8: fixed), lanes per thread of a lane-scan tile (8 or 16), the step mode (0 or
- * 1), as moss_autotune describes, and the number of lane-change candidates
- * a k_decide block resolves itself at the end of its run (0..256, default
- * 256; the others are resolved by the first tickets of k_lanescan).
- * moss_set_schedule checks the ranges (blocks per SM 1..16 for k_decide,
- * 1..32 for the others; weight 0..8), waits for the handle's stream and
+ * The launch schedule (no counterpart in the paper): out7 / in7 = k_decide
+ * blocks per SM, the weight of a lane in k_place's tiles, k_place_slots blocks
+ * per SM, the road-lane weight of k_decide's runs (0: fitted each step from
+ * the previous step's run times, the default; 1..8: fixed), k_place's tiles at
+ * half or full size (8 or 16), the step mode (0 or 1), as moss_autotune
+ * describes, and the number of lane-change candidates that a k_decide block
+ * lists in shared memory (0..256, default 256; the others in global memory).
+ * moss_set_schedule checks the ranges (1..16 for k_decide's blocks, 1..32 for
+ * the next two; weight 0..8), waits for the handle's stream and
  * re-captures the step graphs; on an error the previous schedule stays.
  * Results never depend on the schedule.
  */

@@ -37,7 +37,13 @@ struct SnapBufs {
     int32_t* off;
 };
 
-constexpr int N_STEP_KERNELS = 4;  // decide, resolve, lanescan, place (launch order)
+constexpr int N_STEP_KERNELS = 3;  // decide, lanescan (two-kernel form of the placement only), place (launch order)
+
+// Steps per replayed graph, the longest first: between two graphs the stream
+// drains, between the steps of one graph the kernels overlap at their ends
+// (programmatic dependent launch).
+constexpr int N_GRAPHS = 3;
+constexpr int GRAPH_STEPS[N_GRAPHS] = {8, 2, 1};
 
 }  // namespace
 
@@ -124,10 +130,13 @@ struct MossHandle {
     void* d_ea = nullptr;    // RecA<Real>[cap]
     RecB* d_eb = nullptr;
     int32_t *d_enext = nullptr, *d_enter = nullptr, *d_leave = nullptr, *d_cand_late = nullptr;
-    unsigned long long *d_head = nullptr, *d_lane_tiles = nullptr;
+    unsigned long long* d_head = nullptr;
+    int32_t* d_delta[2] = {nullptr, nullptr};  // growth of k_place's tiles, per parity
+    size_t max_tiles = 0;                      // tiles of any schedule
+    int32_t* d_tiles[2] = {nullptr, nullptr};  // k_place's tile cuts, per snapshot buffer
     void* d_cands = nullptr;  // Cand<Real>[cap]
     unsigned long long* d_gap_head = nullptr;
-    int n_lane_tiles = 0, max_slot_tiles = 0, n_junc_chunks = 0;
+    int n_junc_chunks = 0;
     Counters* d_cnt = nullptr;  // [2]: per parity; d_cnt[0].err holds the device error bits
     int32_t* h_stage = nullptr;          // pinned host staging of setter arguments (2 * n_junctions), read by the setter's kernel
     cudaEvent_t stage_free = nullptr;    // recorded after the last kernel that reads h_stage
@@ -141,16 +150,17 @@ struct MossHandle {
     bool rb_pending[MOSS_METRIC_SLOTS] = {};
 
     // launch configuration (blocks per SM) of the step kernels; moss_autotune picks them
-    int cfg_decide = MOSS_DECIDE_MIN_BLOCKS, cfg_lanescan = 4, cfg_place = 8;
+    int cfg_decide = MOSS_DECIDE_MIN_BLOCKS, cfg_place = 8;
+    int cfg_lanescan = 4;  // weight of a lane in k_place's tiles, in half-slots
     int cfg_runw = 0;    // weight of a road-lane slot in k_decide's runs (0: fitted each step)
-    int cfg_lsr = 4;     // rounds of 128 lanes per warp in a lane-scan tile (4 or 2)
-    int cfg_ccap = 256;  // lane-change candidates a k_decide block resolves itself
+    int cfg_lsr = 4;     // k_place tiles of the full (4) or half (2) size
+    int cfg_ccap = 256;  // lane-change candidates a k_decide block lists in shared memory
 
     int parity = 0;  // snapshot buffer holding the current step
     int step_mode = 0;               // 0: three kernels per step; 1: one cooperative launch
     unsigned* d_bar = nullptr;       // grid barrier of the cooperative step (count, generation)
     cudaError_t launch_err = cudaSuccess;
-    cudaGraphExec_t g2[2] = {nullptr, nullptr}, g1[2] = {nullptr, nullptr};
+    cudaGraphExec_t graph[N_GRAPHS][2] = {};  // GRAPH_STEPS[k] steps from either parity
     bool timing = false;
     cudaEvent_t ev[N_STEP_KERNELS + 1] = {};
     double kms[4] = {0, 0, 0, 0};
@@ -362,10 +372,29 @@ bool same_model(const MossParams& a, const MossParams& b) {
 size_t reca_size(int precision) { return precision == 64 ? sizeof(RecA<double>) : sizeof(RecA<float>); }
 size_t sv_size(int precision) { return precision == 64 ? sizeof(SV<double>) : sizeof(SV<float>); }
 
-// lane-scan tiles of a step with `rounds` rounds of 128 lanes per warp
-int lane_tiles(const MossHandle* h, int rounds) {
-    const int tile = LANESCAN_THREADS * 4 * rounds;
-    return (h->n_lanes + tile - 1) / tile;
+// Tiles of k_place for these sizes: 1 << shift half-slots (a slot weighs 2, a
+// lane lane_w).  At least one slot per thread; above that about 4.5 tiles per
+// SM at most (the 30x30 grid of 100,000 trips: 23.0 us per step with 355
+// tiles, 23.8 with 711 and 23.4 with 178); at most 2^PLACE_LANES_LOG2 lanes a
+// tile (its shared memory).
+long long place_weight(const MossHandle* h, int lane_w) { return 2ll * h->n_veh + (long long)lane_w * h->n_lanes; }
+
+int place_shift(const MossHandle* h, int lane_w, int lsr) {
+    int shift = 9;
+    while (2 * (place_weight(h, lane_w) >> shift) > 9ll * h->sm_count && (2 << shift) <= (lane_w << PLACE_LANES_LOG2))
+        ++shift;
+    return lsr == 2 ? shift - 1 : shift;
+}
+
+// The placement as one kernel (k_place), or as k_lanescan and k_place_slots
+// for large networks: us per step 23.2 / 24.7 at 100,000 trips on the 30x30
+// grid, 45.7 / 45.0 at 350,000 in 12 slots, 55.6 / 46.9 at 500,009 in a
+// district, 170 / 142 in the city.
+constexpr int FUSED_MAX_VEH = 200000;
+bool fused_place(const MossHandle* h) { return h->step_mode == 1 || h->n_veh <= FUSED_MAX_VEH; }
+
+int place_tiles(const MossHandle* h, int lane_w, int lsr) {
+    return (int)(place_weight(h, lane_w) >> place_shift(h, lane_w, lsr)) + 1;
 }
 
 template <typename Real>
@@ -395,10 +424,14 @@ Ctx<Real> make_ctx(MossHandle* h, int cur) {
     }
     c.code = h->d_code; c.stay = (SV<Real>*)h->d_stay;
     c.ea = (RecA<Real>*)h->d_ea; c.eb = h->d_eb; c.enext = h->d_enext; c.head = h->d_head;
-    c.enter = h->d_enter; c.leave = h->d_leave; c.lane_tiles = h->d_lane_tiles;
+    c.enter = h->d_enter; c.leave = h->d_leave; c.tile_delta = h->d_delta[cur]; c.delta_nxt = h->d_delta[1 - cur];
+    c.tile_cur = h->d_tiles[cur]; c.tile_nxt = h->d_tiles[1 - cur];
+    c.tile_shift = SCAN_TILE_LOG2; c.slot_w = 0; c.lane_w = 1;
+    if (fused_place(h)) {
+        c.tile_shift = place_shift(h, h->cfg_lanescan, h->cfg_lsr); c.slot_w = 2; c.lane_w = h->cfg_lanescan;
+    }
     c.cand_late = h->d_cand_late;
     c.cands = (Cand<Real>*)h->d_cands; c.gap_head = h->d_gap_head;
-    c.n_lane_tiles = lane_tiles(h, h->cfg_lsr); c.max_slot_tiles = h->max_slot_tiles;
     c.run_w = h->cfg_runw;
     c.runstat = h->d_runstat;
     c.cand_cap = h->cfg_ccap;
@@ -414,22 +447,30 @@ Ctx<Real> make_ctx(MossHandle* h, int cur) {
 }
 
 struct Grids {
-    int decide_work, decide_ins, resolve, lanescan, place;
+    int decide_work, decide_ins, scan, place;
+    size_t place_smem;
 };
+
+// blocks of k_decide past its work blocks: one start lane per thread, and
+// enough for the phase pressures where the network has junctions
+int extra_blocks(const MossHandle* h) {
+    const int ns = (int)h->start_lanes.size();
+    return std::max((ns + TILE - 1) / TILE, std::min((h->n_jj + TILE - 1) / TILE, h->sm_count));
+}
 
 Grids grids(const MossHandle* h) {
     Grids g;
-    g.decide_work = std::max(1, std::min(h->max_slot_tiles, h->sm_count * h->cfg_decide));
-    const int ns = (int)h->start_lanes.size();
-    g.decide_ins = ns > 0 ? (ns + TILE - 1) / TILE : 0;  // one start lane per thread
-    // candidates are a few per cent of the vehicles; the kernel strides over them
-    g.resolve = std::max(1, std::min(h->max_slot_tiles, h->sm_count * 2));
-    // the lane scan's tickets, plus (MOSS_FOLD_RESOLVE) the candidate and
-    // max-pressure chunks in front of them: their number is known on the
-    // device only, so the grid takes every resident block it may need
-    const int tickets = 1 + lane_tiles(h, h->cfg_lsr) + h->n_junc_chunks + (MOSS_FOLD_RESOLVE ? (h->n_jj + TILE - 1) / TILE + 8 : 0);
-    g.lanescan = std::max(1, std::min(tickets, h->sm_count * h->cfg_lanescan));
-    g.place = std::max(1, std::min(2 * h->max_slot_tiles, h->sm_count * h->cfg_place));
+    // runs of at least a warp of vehicles, as many as the chip holds at once
+    const int resident = h->precision == 64 ? decide_min_blocks<double>() : decide_min_blocks<float>();
+    g.decide_work = std::max(1, std::min((h->n_veh + 31) / 32, h->sm_count * std::min(h->cfg_decide, resident)));
+    g.decide_ins = extra_blocks(h);
+    g.scan = 0;
+    g.place = place_tiles(h, h->cfg_lanescan, h->cfg_lsr) + h->n_junc_chunks + 1;
+    if (!fused_place(h)) {
+        g.scan = ((h->n_lanes - 1) >> SCAN_TILE_LOG2) + 1 + h->n_junc_chunks + 1;
+        g.place = std::min(2 * (h->n_veh / TILE + 1), h->sm_count * h->cfg_place);
+    }
+    g.place_smem = place_smem(place_lanes(place_shift(h, h->cfg_lanescan, h->cfg_lsr), h->cfg_lanescan));
     return g;
 }
 
@@ -438,48 +479,72 @@ Grids grids(const MossHandle* h) {
 template <typename Real, bool Groups>
 cudaError_t launch_coop(MossHandle* h, Ctx<Real>& c) {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_coop<Real, Groups>, TILE, 0);
+    const size_t smem = grids(h).place_smem;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_coop<Real, Groups>, TILE, smem);
     if (e != cudaSuccess) return e;
     int grid = std::max(1, per_sm) * h->sm_count;
-    int n_work = std::max(1, std::min(h->max_slot_tiles, grid));
-    const int ns = (int)h->start_lanes.size();
-    int n_ins = ns > 0 ? (ns + TILE - 1) / TILE : 0;
+    int n_work = std::max(1, std::min((h->n_veh + 31) / 32, grid));
+    int n_ins = extra_blocks(h), n_place = grids(h).place;
     unsigned* bar = h->d_bar;
-    void* args[] = {(void*)&c, (void*)&n_work, (void*)&n_ins, (void*)&bar};
-    return cudaLaunchCooperativeKernel((const void*)k_step_coop<Real, Groups>, grid, TILE, args, 0, h->stream);
+    void* args[] = {(void*)&c, (void*)&n_work, (void*)&n_ins, (void*)&n_place, (void*)&bar};
+    return cudaLaunchCooperativeKernel((const void*)k_step_coop<Real, Groups>, grid, TILE, args, smem,
+                                       h->stream);
 }
 
+// one launch of a step kernel; chained: it may start while the kernel before
+// it in the stream drains (it calls grid_wait before it needs its results)
+template <typename... P, typename... A>
+void launch_step_kernel(MossHandle* h, bool chained, int grid, size_t smem, void (*kernel)(P...), A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TILE); cfg.dynamicSmemBytes = smem; cfg.stream = h->stream;
+    cfg.attrs = at; cfg.numAttrs = chained ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (e != cudaSuccess) h->launch_err = e;
+}
+
+// one step from snapshot buffer `cur`; first: nothing of the handle's step
+// kernels directly before it
 template <typename Real>
-void enqueue_step(MossHandle* h, int cur, bool timed) {
+void enqueue_step(MossHandle* h, int cur, bool timed, bool first) {
     Ctx<Real> c = make_ctx<Real>(h, cur);
     const Grids g = grids(h);
     cudaStream_t s = h->stream;
     if (timed) cudaEventRecord(h->ev[0], s);
     if (h->step_mode == 1) {
-        c.n_lane_tiles = lane_tiles(h, 4);  // the single-launch step scans with the default tile
         const cudaError_t e = h->lane_groups ? launch_coop<Real, true>(h, c) : launch_coop<Real, false>(h, c);
         if (e != cudaSuccess) h->launch_err = e;
         if (timed)
             for (int q = 1; q <= N_STEP_KERNELS; ++q) cudaEventRecord(h->ev[q], s);
         return;
     }
-    if (h->lane_groups) k_decide<Real, true><<<g.decide_work + g.decide_ins, TILE, 0, s>>>(c, g.decide_work);
-    else k_decide<Real, false><<<g.decide_work + g.decide_ins, TILE, 0, s>>>(c, g.decide_work);
+    launch_step_kernel(h, !first, g.decide_work + g.decide_ins, 0,
+                       h->lane_groups ? k_decide<Real, true> : k_decide<Real, false>, c, g.decide_work);
     if (timed) cudaEventRecord(h->ev[1], s);
-#if !MOSS_FOLD_RESOLVE
-    k_resolve<Real><<<g.resolve, TILE, 0, s>>>(c);
-#endif
+    if (g.scan) launch_step_kernel(h, !timed, g.scan, 0, k_lanescan<Real>, c);
     if (timed) cudaEventRecord(h->ev[2], s);
-    if (h->cfg_lsr == 2) k_lanescan<Real, 2><<<g.lanescan, LANESCAN_THREADS, 0, s>>>(c);
-    else k_lanescan<Real, 4><<<g.lanescan, LANESCAN_THREADS, 0, s>>>(c);
+    if (g.scan) launch_step_kernel(h, !timed, g.place, 0, k_place_slots<Real>, c);
+    else launch_step_kernel(h, !timed, g.place, g.place_smem, k_place<Real>, c);
     if (timed) cudaEventRecord(h->ev[3], s);
-    k_place<Real><<<g.place, TILE, 0, s>>>(c);
-    if (timed) cudaEventRecord(h->ev[4], s);
 }
 
-void enqueue(MossHandle* h, int cur, bool timed) {
-    if (h->precision == 64) enqueue_step<double>(h, cur, timed);
-    else enqueue_step<float>(h, cur, timed);
+void enqueue(MossHandle* h, int cur, bool timed, bool first) {
+    if (h->precision == 64) enqueue_step<double>(h, cur, timed, first);
+    else enqueue_step<float>(h, cur, timed, first);
+}
+
+// tile cuts of the current snapshot (after creation, a state reset or a
+// change of the tiles)
+int tile_cuts(MossHandle* h) {
+    for (int32_t* d : h->d_delta) CK(cudaMemsetAsync(d, 0, h->max_tiles * sizeof(int32_t), h->stream));
+    if (!fused_place(h)) return MOSS_OK;
+    const int nb = (h->n_lanes + 255) / 256;
+    if (h->precision == 64) k_tile_cuts<double><<<nb, 256, 0, h->stream>>>(make_ctx<double>(h, h->parity));
+    else k_tile_cuts<float><<<nb, 256, 0, h->stream>>>(make_ctx<float>(h, h->parity));
+    CK(cudaGetLastError());
+    return MOSS_OK;
 }
 
 template <typename Real>
@@ -505,30 +570,30 @@ void enqueue_set_signal(MossHandle* h, int n, int policy) {
 }
 
 void destroy_graphs(MossHandle* h) {
-    for (int k = 0; k < 2; ++k) {
-        if (h->g2[k]) cudaGraphExecDestroy(h->g2[k]);
-        if (h->g1[k]) cudaGraphExecDestroy(h->g1[k]);
-        h->g2[k] = h->g1[k] = nullptr;
-    }
+    for (auto& g : h->graph)
+        for (cudaGraphExec_t& ex : g) {
+            if (ex) cudaGraphExecDestroy(ex);
+            ex = nullptr;
+        }
 }
 
 int build_graphs(MossHandle* h) {
     for (int p = 0; p < 2; ++p) {
-        for (int nsteps = 1; nsteps <= 2; ++nsteps) {
+        for (int q = 0; q < N_GRAPHS; ++q) {
             cudaGraph_t g = nullptr;
             CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
             h->launch_err = cudaSuccess;
-            for (int k = 0; k < nsteps; ++k) enqueue(h, (p + k) & 1, false);
+            for (int k = 0; k < GRAPH_STEPS[q]; ++k) enqueue(h, (p + k) & 1, false, k == 0);
             CK(cudaStreamEndCapture(h->stream, &g));
             if (h->launch_err != cudaSuccess) {
                 cudaGraphDestroy(g);
-                return cuda_fail(h, h->launch_err, "cooperative step launch");
+                return cuda_fail(h, h->launch_err, "step launch");
             }
             cudaGraphExec_t ex = nullptr;
             cudaError_t e = cudaGraphInstantiate(&ex, g, 0);
             cudaGraphDestroy(g);
             if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphInstantiate");
-            (nsteps == 2 ? h->g2[p] : h->g1[p]) = ex;
+            h->graph[q][p] = ex;
         }
     }
     return MOSS_OK;
@@ -794,10 +859,14 @@ int device_setup(MossHandle* h, void* stream) {
     TRY(upload(h, &h->d_head, std::vector<unsigned long long>(NL, 0ull)));
     TRY(upload(h, &h->d_enter, std::vector<int32_t>(NL, 0)));
     TRY(upload(h, &h->d_leave, std::vector<int32_t>(NL, 0)));
-    h->n_lane_tiles = lane_tiles(h, 2);  // look-back words for the smaller tile
-    h->max_slot_tiles = (NV + TILE - 1) / TILE + 1;
+    // tiles under any schedule: place_shift leaves at most 2 x 4.5 per SM, or
+    // tiles of at least the weight of 2^(PLACE_LANES_LOG2 - 2) lanes
+    h->max_tiles = 10 * (size_t)h->sm_count + ((2 * (size_t)NV + NL) >> (PLACE_LANES_LOG2 - 2)) + 4;
+    for (int k = 0; k < 2; ++k) {
+        TRY(dalloc(h, &h->d_tiles[k], h->max_tiles + 1));
+        TRY(dalloc(h, &h->d_delta[k], h->max_tiles));
+    }
     h->n_junc_chunks = (NJ + JUNC_CHUNK - 1) / JUNC_CHUNK;
-    TRY(upload(h, &h->d_lane_tiles, std::vector<unsigned long long>(h->n_lane_tiles, 0ull)));
     std::vector<Counters> c0(2, Counters{});
     c0[0].tag = 1;
     TRY(upload(h, &h->d_cnt, c0));
@@ -813,6 +882,7 @@ int device_setup(MossHandle* h, void* stream) {
     CK(cudaEventCreateWithFlags(&h->load_free, cudaEventDisableTiming));
     CK(cudaEventRecord(h->load_free, h->stream));
     for (int k = 0; k <= N_STEP_KERNELS; ++k) CK(cudaEventCreate(&h->ev[k]));
+    TRY(tile_cuts(h));
     TRY(junction_init(h, 0, NJ));
     CK(cudaStreamSynchronize(h->stream));
     TRY(build_graphs(h));
@@ -1528,27 +1598,26 @@ int moss_step(moss_t h, int n) {
     h->steps_enqueued += n;
     if (h->timing) {
         for (int k = 0; k < n; ++k) {
-            enqueue(h, h->parity, true);
+            enqueue(h, h->parity, true, true);
             h->parity ^= 1;
             CK(cudaEventSynchronize(h->ev[N_STEP_KERNELS]));
-            // reported order: decide, lanescan, place, resolve
-            static const int slot_of[N_STEP_KERNELS] = {0, 3, 1, 2};
+            // reported order: decide, lanescan, place, resolve (part of decide)
             for (int q = 0; q < N_STEP_KERNELS; ++q) {
                 float ms = 0;
+                if (q == 1 && fused_place(h)) continue;  // nothing between these events
                 CK(cudaEventElapsedTime(&ms, h->ev[q], h->ev[q + 1]));
-                h->kms[slot_of[q]] += ms;
+                h->kms[q] += ms;
             }
             h->ksteps++;
         }
         CK(cudaGetLastError());
         return MOSS_OK;
     }
-    int k = 0;
-    for (; k + 2 <= n; k += 2) CK(cudaGraphLaunch(h->g2[h->parity], h->stream));
-    if (k < n) {
-        CK(cudaGraphLaunch(h->g1[h->parity], h->stream));
-        h->parity ^= 1;
-    }
+    for (int q = 0; q < N_GRAPHS; ++q)
+        for (; n >= GRAPH_STEPS[q]; n -= GRAPH_STEPS[q]) {
+            CK(cudaGraphLaunch(h->graph[q][h->parity], h->stream));
+            h->parity ^= GRAPH_STEPS[q] & 1;
+        }
     return MOSS_OK;
 }
 
@@ -1855,8 +1924,9 @@ int moss_set_state(moss_t h, const MossState* in, int64_t step) {
     CK(cudaMemcpy(h->d_metrics + M_CUR_ACTIVE, cur, sizeof(cur), cudaMemcpyHostToDevice));
     Counters c{};
     CK(cudaMemcpy(&c, h->d_cnt + h->parity, sizeof(c), cudaMemcpyDeviceToHost));
-    c.n_cur = (int)n_act; c.n_ent = 0; c.n_cand = 0; c.n_late = 0; c.ticket_lane = 0; c.res_done = 0;
+    c.n_cur = (int)n_act; c.n_ent = 0; c.n_cand = 0; c.junc_done = 0;
     CK(cudaMemcpy(h->d_cnt + h->parity, &c, sizeof(c), cudaMemcpyHostToDevice));
+    TRY(tile_cuts(h));
     TRY(junction_init(h, 0, h->n_junctions));
     CK(cudaStreamSynchronize(h->stream));
     return MOSS_OK;
@@ -1944,11 +2014,13 @@ int moss_set_step_mode(moss_t h, int mode) {
     const int old = h->step_mode;
     h->step_mode = mode;
     destroy_graphs(h);
-    const int rc = build_graphs(h);
+    int rc = build_graphs(h);
+    if (rc == MOSS_OK) rc = tile_cuts(h);
     if (rc != MOSS_OK) {
         h->step_mode = old;
         destroy_graphs(h);
         TRY(build_graphs(h));
+        TRY(tile_cuts(h));
         return rc;
     }
     return MOSS_OK;
@@ -1956,7 +2028,7 @@ int moss_set_step_mode(moss_t h, int mode) {
 
 int moss_step_launches(moss_t h, int* out) {
     if (!h || !out) return MOSS_EINVAL;
-    *out = h->step_mode == 1 ? 1 : (MOSS_FOLD_RESOLVE ? 3 : 4);
+    *out = h->step_mode == 1 ? 1 : fused_place(h) ? 2 : 3;
     return MOSS_OK;
 }
 
@@ -1991,7 +2063,7 @@ int moss_set_kernel_timing(moss_t h, int enable) {
 static int time_steps(MossHandle* h, int steps, double* ms) {
     double tot = 0;
     for (int k = 0; k < steps; ++k) {
-        enqueue(h, h->parity, true);
+        enqueue(h, h->parity, true, true);
         h->parity ^= 1;
         CK(cudaEventSynchronize(h->ev[N_STEP_KERNELS]));
         float x = 0;
@@ -2008,8 +2080,8 @@ int moss_autotune(moss_t h, int trial_steps, int* chosen3) {
     if (trial_steps < 1) return fail(h, MOSS_EINVAL, "trial_steps must be >= 1");
     CK(cudaStreamSynchronize(h->stream));
     // coordinate search over the schedule: blocks per SM of each kernel, the
-    // road-lane weight of k_decide's runs, the lane-scan tile and the step
-    // mode; results do not depend on the schedule, only the time does
+    // road-lane weight of k_decide's runs, the lane weight and size of
+    // k_place's tiles and the step mode; results do not depend on the schedule, only the time does
     int coop = 0;
     CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
     struct Knob { int* v; int n; int c[3]; };
@@ -2023,6 +2095,7 @@ int moss_autotune(moss_t h, int trial_steps, int* chosen3) {
         for (int k = 0; k < kb.n; ++k) {
             *kb.v = kb.c[k];
             h->launch_err = cudaSuccess;
+            TRY(tile_cuts(h));
             double ms = 0;
             TRY(time_steps(h, trial_steps, &ms));
             if (h->launch_err != cudaSuccess) {  // a mode this device cannot launch
@@ -2033,6 +2106,7 @@ int moss_autotune(moss_t h, int trial_steps, int* chosen3) {
         }
         *kb.v = best;
     }
+    TRY(tile_cuts(h));
     destroy_graphs(h);
     TRY(build_graphs(h));
     if (chosen3) { chosen3[0] = h->cfg_decide; chosen3[1] = h->cfg_lanescan; chosen3[2] = h->cfg_place; }
@@ -2064,12 +2138,14 @@ int moss_set_schedule(moss_t h, const int* in7) {
     h->cfg_decide = in6[0]; h->cfg_lanescan = in6[1]; h->cfg_place = in6[2];
     h->cfg_runw = in6[3]; h->cfg_lsr = in6[4] / 4; h->step_mode = in6[5]; h->cfg_ccap = in7[6];
     destroy_graphs(h);
-    const int rc = build_graphs(h);
+    int rc = build_graphs(h);
+    if (rc == MOSS_OK) rc = tile_cuts(h);
     if (rc != MOSS_OK) {
         h->cfg_decide = old[0]; h->cfg_lanescan = old[1]; h->cfg_place = old[2];
         h->cfg_runw = old[3]; h->cfg_lsr = old[4]; h->step_mode = old[5]; h->cfg_ccap = old[6];
         destroy_graphs(h);
         TRY(build_graphs(h));
+        TRY(tile_cuts(h));
         return rc;
     }
     return MOSS_OK;

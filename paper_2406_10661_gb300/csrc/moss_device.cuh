@@ -12,7 +12,7 @@
 // search in the adjacent lane's segment (adjacent lanes of a road are
 // adjacent in memory).
 //
-// One step = three kernels:
+// One step = two kernels:
 //   k_decide    per vehicle: sensing, IDM (App. B.3 eqs. (1)-(2)), the
 //               randomized MOBIL decision (App. B.3; run from a per-warp
 //               shared-memory queue of the vehicles whose attempt draw
@@ -22,16 +22,15 @@
 //               lane-change candidates of its run (deterministic conflict
 //               rule between candidates entering the same gap from both
 //               sides); extra blocks run the departure insertion (App. B.2
-//               update stream 3);
-//   k_lanescan  first tickets: the fit of the next step's run weight, the
-//               candidates past a decide block's own list, max-pressure
-//               phase sums (§3.2); then per-lane sizes of the next snapshot
-//               -> offsets (single-pass decoupled look-back scan), signal
-//               states of the next step (§3.2 policies);
-//   k_place     writes the next snapshot: vehicles that kept their lane keep
-//               their relative order (no overtaking within a lane), vehicles
-//               that entered a lane are merged by (s, id).
-// (k_step_coop runs the same three as phases of one cooperative launch.)
+//               update stream 3) and the max-pressure phase sums (§3.2);
+//   k_place     tiles of whole lanes: the sizes of the tile's lanes in the
+//               next snapshot -> their offsets (k_decide counted how the tiles
+//               before it grow), then the next snapshot: vehicles that kept
+//               their lane keep their relative order (no overtaking within a
+//               lane), vehicles that entered a lane are merged by (s, id);
+//               other blocks: signal states of the next step (§3.2 policies),
+//               scenario clocks, the fit of the next step's run weight.
+// (k_step_coop runs the same two as phases of one cooperative launch.)
 #pragma once
 
 #include <cuda/atomic>
@@ -66,10 +65,7 @@ enum : int { ERR_TIMEOUT = 1, ERR_ROUTE = 2, ERR_TRANSFER = 4, ERR_RANGE = 8 };
 constexpr int ERR_POISON = ERR_TIMEOUT | ERR_RANGE;
 
 constexpr int TILE = 256;           // slots per tile of k_decide / k_place (= threads)
-constexpr int LANESCAN_THREADS = 256;
-constexpr int LANESCAN_ITEMS = 16;
-constexpr int LANESCAN_TILE = LANESCAN_THREADS * LANESCAN_ITEMS;
-constexpr int JUNC_CHUNK = 256;     // junctions per k_lanescan ticket (one per thread)
+constexpr int JUNC_CHUNK = 256;     // junctions per k_place block (one per thread)
 constexpr int RUNSTAT_MAX = 4096;  // k_decide work blocks whose run statistics are kept
 constexpr long long SPIN_LIMIT = 1ll << 22;  // bounded waits (~0.5 s with backoff)
 
@@ -79,22 +75,14 @@ constexpr long long SPIN_LIMIT = 1ll << 22;  // bounded waits (~0.5 s with backo
 struct Counters {
     int n_cur;       // active vehicles in the current snapshot
     int n_ent;       // entrants appended this step
-    int n_cand;      // lane-change candidates listed this step (for k_resolve)
-    int ticket_lane; // k_lanescan tickets
-    int n_late;      // candidates left to k_lanescan (past a k_decide block's own list)
+    int n_cand;      // lane-change candidates listed this step
+    int junc_done;   // k_place blocks of junctions finished (the last one advances the clocks)
     int tag;         // step tag of the per-lane lists (never 0)
     int err;         // device error bits (set 0 only)
     int n_mp;        // junctions under max pressure (set 0 only)
-    int res_done;    // k_lanescan tickets of candidate / pressure work finished
     int run_wq;      // fitted weight of a road-lane slot in k_decide's runs, x256 (0: none yet)
     int n_runs;      // k_decide work runs of this step (their statistics for the fit)
 };
-
-// the candidates past a decide block's own list are resolved in the first
-// tickets of k_lanescan instead of a kernel of their own
-#ifndef MOSS_FOLD_RESOLVE
-#define MOSS_FOLD_RESOLVE 1
-#endif
 
 // snapshot records
 template <typename Real> struct RecA;
@@ -114,7 +102,7 @@ struct alignas(16) RecB {
 };
 template <typename Real> struct alignas(2 * sizeof(Real)) SV { Real s, v; };
 
-// A lane-change candidate, finished by k_resolve.  gap = its insertion
+// A lane-change candidate, finished at the end of its block's run.  gap = its insertion
 // position in the target lane's segment plus the target lane's index: equal
 // for two candidates exactly when they enter the same lane between the same
 // target leader and follower (unique over lanes: lane l's positions span
@@ -186,7 +174,7 @@ struct Ctx {
     const int32_t* jj_from;  // the road lane each of them leaves
     const int2* road_span;   // [n_roads] (first, end) road lanes of every road (absolute ids)
     int n_jj;                // junction lanes in jj_lane
-    int32_t* mp_press;       // [n_junctions][8] phase pressures of this step, summed by k_resolve
+    int32_t* mp_press;       // [n_junctions][8] phase pressures of this step, summed by k_decide's extra blocks
     int* n_mp;               // junctions under max pressure
     // ---- vehicles (by global id)
     const int2* route_span;  // [n_veh] route of a vehicle: routes[x .. y)
@@ -219,16 +207,21 @@ struct Ctx {
     RecB* eb;
     int32_t* enext;       // per-lane singly linked list of entrants
     unsigned long long* head;  // [n_lanes] (tag << 32 | entrant) or stale
-    int32_t* enter;       // [n_lanes], zeroed by k_lanescan after use
-    int32_t* leave;       // [n_lanes], zeroed by k_lanescan after use
+    int32_t* enter;       // [n_lanes], zeroed by k_place after use
+    int32_t* leave;       // [n_lanes], zeroed by k_place after use
     Cand<Real>* cands;    // this step's lane-change candidates (cnt->n_cand of them)
-    int32_t* cand_late;   // indices of the candidates k_lanescan resolves (cnt->n_late)
+    int32_t* cand_late;   // [n_veh] candidates of a run past its block's own list, from the run's first slot on
     unsigned long long* gap_head;  // [n_veh + n_lanes + 1] (tag << 32 | candidate) or stale
-    unsigned long long* lane_tiles;
-    int n_lane_tiles, max_slot_tiles, n_junc_chunks;
+    int32_t* tile_delta;  // vehicles that enter minus vehicles that leave the lanes of a k_place tile this step
+    int32_t* delta_nxt;   // the next step's, cleared by k_place
+    int32_t* tile_cur;    // k_place tiles of this step: tile t holds the lanes [tile_cur[t], tile_cur[t+1])
+    int32_t* tile_nxt;    // the next step's, written by k_place
+    int tile_shift;       // a tile ends where slot_w * off[l] + lane_w * l passes a multiple of 1 << tile_shift
+    int slot_w, lane_w;   // weights of a slot and of a lane in the tiles
+    int n_junc_chunks;
     int run_w;           // weight of a road-lane slot in k_decide's runs (junction-lane slot: 1); 0: fitted
     int4* runstat;       // [RUNSTAT_MAX] per k_decide work block: duration (ns, lo/hi), road-lane and junction-lane slots
-    int cand_cap;        // lane-change candidates a k_decide block resolves itself (<= 256)
+    int cand_cap;        // lane-change candidates a k_decide block lists in shared memory (<= 256)
     Counters* cnt;       // this step's counters
     Counters* cnt_next;  // the next step's
     int* err;            // device error bits
@@ -310,17 +303,29 @@ __device__ __forceinline__ int junction_state(int policy, int manual, int offset
                                               const int32_t* amber, int np, long long t) {
     if (policy == POL_NONE || np <= 0) return 512;
     if (policy == POL_MANUAL) return (manual & 15) | ((np & 15) << 4);
+    // at most 8 phases: their loads go out together
+    int g[8], a[8];
     long long cyc = 0;
-    for (int p = 0; p < np; ++p) cyc += green[p] + amber[p];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        g[p] = p < np ? green[p] : 0;
+        a[p] = p < np ? amber[p] : 0;
+        cyc += (long long)g[p] + a[p];
+    }
     if (cyc <= 0) return 512;
     long long x = (t + offset) % cyc;
     if (x < 0) x += cyc;
-    for (int p = 0; p < np; ++p) {
-        const long long g = green[p], a = amber[p];
-        if (x < g + a) return p | ((np & 15) << 4) | (x >= g ? 256 | (((p + 1) % np) << 10) : 0);
-        x -= g + a;
+    int st = (np & 15) << 4;
+    bool open = true;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        if (open && p < np && x < (long long)g[p] + a[p]) {
+            st = p | ((np & 15) << 4) | (x >= g[p] ? 256 | ((p + 1 < np ? p + 1 : 0) << 10) : 0);
+            open = false;
+        }
+        x -= (long long)g[p] + a[p];
     }
-    return (np & 15) << 4;
+    return st;
 }
 
 // encoded state of a max-pressure junction (R23)

@@ -5,6 +5,15 @@
 
 namespace moss {
 
+// Programmatic dependent launch: a kernel of a step may start while the one
+// before it drains.  grid_wait returns once that kernel has finished and its
+// writes are visible (at once for an ordinary launch); grid_release lets the
+// next kernel start when every block of this one has called it or ended.  It
+// is called after grid_wait, so a kernel that runs early knows that all but
+// the kernel directly before it have finished.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // entrant list of a lane for this step's tag (-1 if empty or stale)
 __device__ __forceinline__ int list_head(const unsigned long long* head, int lane, int tag) {
     const unsigned long long h = head[lane];
@@ -19,13 +28,33 @@ __device__ __forceinline__ void list_push(unsigned long long* head, int32_t* ene
 }
 
 // ---------------------------------------------------------------------------
-// A k_decide block's lane-change candidates: their indices in the candidate
-// list, resolved by the block once its run is done; past cand_cap of them (a
-// schedule value, at most CAND_LOCAL) the rest go to the late list that
-// k_lanescan's first tickets resolve.
+// k_place's tile that holds lane l, whose segment starts at off
+template <typename Real>
+__device__ __forceinline__ int tile_key(const Ctx<Real>& c, int off, int l) {
+    return (int)(((long long)off * c.slot_w + (long long)c.lane_w * l) >> c.tile_shift);
+}
+
+// a vehicle leaves / enters lane l: counted for the lane and for its tile
+template <typename Real>
+__device__ __forceinline__ void count_leave(const Ctx<Real>& c, int l) {
+    atomicAdd(&c.leave[l], 1);
+    atomicAdd(&c.tile_delta[tile_key(c, c.slot_w ? c.cur.off[l] : 0, l)], -1);
+}
+template <typename Real>
+__device__ __forceinline__ void count_enter(const Ctx<Real>& c, int l) {
+    atomicAdd(&c.enter[l], 1);
+    atomicAdd(&c.tile_delta[tile_key(c, c.slot_w ? c.cur.off[l] : 0, l)], 1);
+}
+
+// A k_decide block's lane-change candidates: their candidates: their indices in the candidate
+// list, resolved by the block once its run is done.  The first cand_cap of
+// them (a schedule value, at most CAND_LOCAL) are listed in shared memory,
+// the rest in the run's own part of cand_late, which starts at the run's
+// first slot (a run has at most one candidate per slot).
 constexpr int CAND_LOCAL = 256;
 struct CandLocal {
     int n;
+    int run[2];  // slots of the run
     int idx[CAND_LOCAL];
 };
 
@@ -33,7 +62,7 @@ template <typename Real>
 __device__ __forceinline__ void note_candidate(const Ctx<Real>& c, CandLocal& cl, int k) {
     const int j = atomicAdd(&cl.n, 1);
     if (j < c.cand_cap) cl.idx[j] = k;
-    else c.cand_late[atomicAdd(&c.cnt->n_late, 1)] = k;
+    else c.cand_late[cl.run[0] + j - c.cand_cap] = k;
 }
 
 // ---------------------------------------------------------------------------
@@ -71,7 +100,7 @@ __device__ void insert_departure(const Ctx<Real>& c, int l, int tag) {
     B.v0f = c.v0f[vid]; B.rptr = r0; B.rlast = r1; B.nl = nl;
     c.ea[q] = A;
     c.eb[q] = B;
-    atomicAdd(&c.enter[l], 1);
+    count_enter(c, l);
     list_push(c.head, c.enext, l, q, tag);
     c.q_head[l] = h + 1;
     c.vstatus[vid] = 1;
@@ -150,7 +179,7 @@ __device__ __forceinline__ int integrate_emit(const Ctx<Real>& c, MetricAcc& acc
         c.vstatus[E.id] = 2;
         acc.arr += 1;
         acc.tt += (t + 1) - (long long)c.dep[E.id];
-        atomicAdd(&c.leave[lane], 1);
+        count_leave(c, lane);
         long long* M = c.metrics + (long long)sc * M_NFIELDS;
         atomicAdd((unsigned long long*)&M[M_CUR_ACTIVE], (unsigned long long)(-1ll));
         atomicAdd((unsigned long long*)&M[M_CUR_ARRIVED], 1ull);
@@ -164,7 +193,7 @@ __device__ __forceinline__ int integrate_emit(const Ctx<Real>& c, MetricAcc& acc
         return 0;
     }
     c.code[i] = C_MOVE;
-    atomicAdd(&c.leave[lane], 1);
+    count_leave(c, lane);
     const int q = warp_claim(&c.cnt->n_ent);
     RecA<Real> A;
     A.s = sn; A.v = vn; A.id = E.id; A.lane = nlane;
@@ -172,13 +201,13 @@ __device__ __forceinline__ int integrate_emit(const Ctx<Real>& c, MetricAcc& acc
     B.v0f = EB.v0f; B.rptr = rptr; B.rlast = rlast; B.nl = nl;
     c.ea[q] = A;
     c.eb[q] = B;
-    atomicAdd(&c.enter[nlane], 1);
+    count_enter(c, nlane);
     list_push(c.head, c.enext, nlane, q, tag);
     return 1;
 }
 
 // ---------------------------------------------------------------------------
-// A lane-change candidate leaves its decision for k_resolve: a record in the
+// A lane-change candidate leaves its decision for the end of the run: a record in the
 // candidate list, linked into the list of its target gap.
 template <typename Real>
 __device__ __forceinline__ void list_candidate(const Ctx<Real>& c, int i, const RecA<Real>& E, const RecB& EB,
@@ -321,7 +350,7 @@ __device__ __forceinline__ void mobil_finish(const Ctx<Real>& c, const MobilQueu
 // (one vehicle per thread); blocks [n_work, gridDim) run the insertion.
 // Per vehicle: the own-lane acceleration and the attempt draw, MOBIL if the
 // draw passed (from the warp's queue, above), then the update; lane-change
-// candidates are finished by k_resolve.
+// candidates are finished at the end of the block's run.
 // Groups: the network has lane groups (some road has a turn that not all of
 // its lanes serve), so the mandatory changes of R27 can occur; without them
 // that path is not compiled in.
@@ -329,6 +358,13 @@ __device__ __forceinline__ void mobil_finish(const Ctx<Real>& c, const MobilQueu
 #ifndef MOSS_DECIDE_MIN_BLOCKS
 #define MOSS_DECIDE_MIN_BLOCKS 5
 #endif
+#ifndef MOSS_DECIDE_MIN_BLOCKS_FP64
+#define MOSS_DECIDE_MIN_BLOCKS_FP64 3
+#endif
+template <typename Real>
+__host__ __device__ constexpr int decide_min_blocks() {
+    return sizeof(Real) == 8 ? MOSS_DECIDE_MIN_BLOCKS_FP64 : MOSS_DECIDE_MIN_BLOCKS;
+}
 // The run of slots [*sb, *se) of work block vb of n_work.  A vehicle on a
 // road lane costs about twice one on a junction lane (MOBIL, longer
 // neighbour searches), so the runs split the snapshot by weight: run_w (a
@@ -336,7 +372,7 @@ __device__ __forceinline__ void mobil_finish(const Ctx<Real>& c, const MobilQueu
 // slot, from the current lane offsets at the lane ranges of each scenario
 // (road lanes first, then junction lanes), when blocks take four tiles or
 // more each; then each end moves back to the start of its road.  The runs
-// are contiguous and cover every slot.
+// are contiguous and cover every slot.  s_run: shared, the run on return.
 __device__ __forceinline__ long long run_weight(int a, int b, int e, int wq) {
     return (long long)wq * (b - a) + 256ll * (e - b);
 }
@@ -363,16 +399,13 @@ __device__ __forceinline__ int road_start(const Ctx<Real>& c, int slot, int n) {
 }
 
 template <typename Real>
-__device__ __forceinline__ void decide_run(const Ctx<Real>& c, int n, int n_work, int vb, int* sb, int* se) {
-    __shared__ int s_run[2];
+__device__ __forceinline__ void decide_run(const Ctx<Real>& c, int n, int n_work, int vb, int* s_run, int* sb,
+                                           int* se) {
     const int n_tiles = (n + TILE - 1) / TILE;
     if (n_tiles < 4 * n_work) {
         // a few tiles per block: equal slot counts (weights would leave
         // blocks idle at this granularity)
-        if (threadIdx.x == 0) {
-            s_run[0] = road_start(c, (int)((long long)vb * n / n_work), n);
-            s_run[1] = road_start(c, (int)((long long)(vb + 1) * n / n_work), n);
-        }
+        if (threadIdx.x < 2) s_run[threadIdx.x] = road_start(c, (int)((long long)(vb + (int)threadIdx.x) * n / n_work), n);
     } else if (threadIdx.x < 32) {
         const int wl = threadIdx.x;
         const int wq = run_wq(c);
@@ -434,7 +467,8 @@ __device__ __forceinline__ void decide_run(const Ctx<Real>& c, int n, int n_work
 
 // The work of block vb of nvb (k_decide's grid, or a virtual block of the
 // single-launch step): vb < n_work takes a run of slot tiles, the others run
-// the insertion.
+// the insertion and add up the phase pressures of the max-pressure junctions
+// (k_place advances those).
 template <typename Real, bool Groups>
 __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int vb, int nvb) {
     const int tag = c.cnt->tag;
@@ -442,6 +476,8 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
         const int stride = (nvb - n_work) * TILE;
         for (int k = (vb - n_work) * TILE + threadIdx.x; k < c.n_start; k += stride)
             insert_departure(c, c.start_lanes[k], tag);
+        if (*c.n_mp > 0)
+            for (int k = (vb - n_work) * TILE + threadIdx.x; k < c.n_jj; k += stride) mp_accumulate(c, k);
         return;
     }
     const int n = c.cnt->n_cur;
@@ -458,16 +494,19 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
     if (vb == 0 && threadIdx.x == 0) c.cnt->n_runs = n_work;
     int n_road = 0;
     int s_beg, s_end;
-    decide_run(c, n, n_work, vb, &s_beg, &s_end);
-    const int t_beg = s_beg / TILE, t_end = s_beg < s_end ? (s_end + TILE - 1) / TILE : t_beg;
+    decide_run(c, n, n_work, vb, cl.run, &s_beg, &s_end);
+    // passes of TILE slots: from a multiple of TILE on, but a run that fits
+    // one pass takes one (its first slot rounded down to a line of records)
+    const int base = s_end - (s_beg & ~7) <= TILE ? s_beg & ~7 : s_beg / TILE * TILE;
+    const int n_pass = s_beg < s_end ? (s_end - base + TILE - 1) / TILE : 0;
     MetricAcc acc;
     macc_reset(acc, -1);
     const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31, qb = warp * 64;
     if (wl == 0) q.n[warp] = 0;
     __syncwarp();
-    for (int tile = t_beg;; ++tile) {
-        const bool last = tile >= t_end;
-        const int i = tile * TILE + threadIdx.x;
+    for (int pass = 0;; ++pass) {
+        const bool last = pass >= n_pass;
+        const int i = base + pass * TILE + threadIdx.x;
         if (!last && i >= s_beg && i < s_end) {
             const RecA<Real> E = c.cur.a[i];
             const RecB EB = c.cur.b[i];
@@ -490,7 +529,7 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
                     if (ctl & SC_RETIRE) {
                         c.code[i] = C_ARRIVE;
                         c.vstatus[E.id] = 2;
-                        atomicAdd(&c.leave[lane], 1);
+                        count_leave(c, lane);
                     } else {
                         c.code[i] = C_STAY;
                         SV<Real> w;
@@ -525,7 +564,7 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
             }
         }
         // MOBIL over the last 32 entries of the warp's queue once it holds
-        // 32, and over what is left after the last tile
+        // 32, and over what is left after the last pass
         __syncwarp();
         const int nq = q.n[warp];
         const int take = last ? nq : (nq >= 32 ? 32 : 0);
@@ -539,8 +578,8 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
     }
     // the run's lane-change candidates (their rivals are all in this run)
     __syncthreads();
-    const int ncl = min(cl.n, c.cand_cap);
-    for (int j = threadIdx.x; j < ncl; j += TILE) resolve_one(c, acc, cl.idx[j], c.n_veh, tag);
+    for (int j = threadIdx.x; j < cl.n; j += TILE)
+        resolve_one(c, acc, j < c.cand_cap ? cl.idx[j] : c.cand_late[s_beg + j - c.cand_cap], c.n_veh, tag);
     if (n_road) atomicAdd(&s_road, n_road);
     macc_flush_block<TILE>(acc, c.metrics);  // (its barriers also complete s_road)
     // the run's statistics for the next step's weight fit (run_fit)
@@ -554,184 +593,11 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
 }
 
 template <typename Real, bool Groups>
-__global__ void __launch_bounds__(TILE, MOSS_DECIDE_MIN_BLOCKS) k_decide(Ctx<Real> c, int n_work) {
-    if (*c.err & ERR_POISON) return;
+__global__ void __launch_bounds__(TILE, decide_min_blocks<Real>()) k_decide(Ctx<Real> c, int n_work) {
+    grid_wait();
+    grid_release();
+    if (__syncthreads_or(threadIdx.x == 0 ? *c.err & ERR_POISON : 0)) return;
     decide_block<Real, Groups>(c, n_work, blockIdx.x, gridDim.x);
-}
-
-template <typename Real>
-__global__ void __launch_bounds__(TILE) k_resolve(Ctx<Real> c) {
-    if (*c.err & ERR_POISON) return;
-    const int nc = c.cnt->n_late;
-    const int tag = c.cnt->tag;
-    MetricAcc acc;
-    macc_reset(acc, -1);
-    for (int k = blockIdx.x * TILE + threadIdx.x; k < nc; k += gridDim.x * TILE)
-        resolve_one(c, acc, c.cand_late[k], c.n_veh, tag);
-    // the phase pressures of the max-pressure junctions (read by k_lanescan)
-    if (*c.n_mp > 0)
-        for (int k = blockIdx.x * TILE + threadIdx.x; k < c.n_jj; k += gridDim.x * TILE) mp_accumulate(c, k);
-    macc_flush_block<TILE>(acc, c.metrics);
-}
-
-// ---------------------------------------------------------------------------
-// block-wide exclusive scan of one 64-bit value per thread (256 threads)
-__device__ __forceinline__ long long block_exclusive_scan(long long x, long long* total) {
-    __shared__ long long warp_sum[LANESCAN_THREADS / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    long long incl = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_sum[warp] = incl;
-    __syncthreads();
-    long long base = 0, tot = 0;
-#pragma unroll
-    for (int w = 0; w < LANESCAN_THREADS / 32; ++w) {
-        const long long ws = warp_sum[w];
-        if (w < warp) base += ws;
-        tot += ws;
-    }
-    __syncthreads();
-    *total = tot;
-    return base + incl - x;
-}
-
-// One lane tile of k_lanescan (LS_ROUNDS x 1024 lanes).  newsize(l) =
-// size(l) - leave(l) + enter(l); its exclusive prefix sum over lanes (the
-// next lane offsets) in one decoupled look-back pass; tile words pack
-// (flag:2 | sum:62).  Warp w takes LS_ROUNDS x 128 consecutive lanes of the
-// tile in LS_ROUNDS rounds of 128 (4 consecutive lanes per thread), so each
-// 16-byte load and store of a warp covers one contiguous 512-byte run.  The
-// tile size is a schedule choice (moss_autotune): 4 rounds (4096 lanes) or 2.
-constexpr int LS_WARPS = LANESCAN_THREADS / 32;
-static_assert(LANESCAN_TILE == LS_WARPS * 128 * 4, "the default lane tile has 4 rounds");
-static_assert(JUNC_CHUNK == LANESCAN_THREADS, "one junction per thread");
-
-template <typename Real, int LS_ROUNDS>
-__device__ __forceinline__ void lanescan_tile(const Ctx<Real>& c, int tile) {
-    constexpr int LS_TILE = LS_WARPS * 128 * LS_ROUNDS;
-    __shared__ long long s_wsum[LS_WARPS];
-    __shared__ unsigned long long s_prefix;
-    const int ln = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nl = c.n_lanes;
-    const int wbase = tile * LS_TILE + w * (LS_TILE / LS_WARPS);
-    int ns[LS_ROUNDS][4];
-    long long wpre[LS_ROUNDS];
-    long long run = 0;
-    // every load of the tile is issued before any result is used (and before
-    // the zeroing stores), so the tile costs one memory round trip
-    int o[LS_ROUNDS][4], lvv[LS_ROUNDS][4], env[LS_ROUNDS][4], o4[LS_ROUNDS];
-#pragma unroll
-    for (int r = 0; r < LS_ROUNDS; ++r) {
-        const int l0 = wbase + r * 128 + 4 * ln;
-        if (l0 + 4 <= nl) {
-            const int4 ov = *reinterpret_cast<const int4*>(c.cur.off + l0);
-            const int4 lx = *reinterpret_cast<const int4*>(c.leave + l0);
-            const int4 ex = *reinterpret_cast<const int4*>(c.enter + l0);
-            o[r][0] = ov.x; o[r][1] = ov.y; o[r][2] = ov.z; o[r][3] = ov.w;
-            lvv[r][0] = lx.x; lvv[r][1] = lx.y; lvv[r][2] = lx.z; lvv[r][3] = lx.w;
-            env[r][0] = ex.x; env[r][1] = ex.y; env[r][2] = ex.z; env[r][3] = ex.w;
-            o4[r] = ln == 31 ? c.cur.off[l0 + 4] : 0;
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int l = l0 + j;
-                const bool in = l < nl;
-                o[r][j] = in || l == nl ? c.cur.off[l] : 0;
-                lvv[r][j] = in ? c.leave[l] : 0;
-                env[r][j] = in ? c.enter[l] : 0;
-            }
-            o4[r] = 0;
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < LS_ROUNDS; ++r) {
-        const int l0 = wbase + r * 128 + 4 * ln;
-        if (l0 + 4 <= nl) {
-            *reinterpret_cast<int4*>(c.leave + l0) = make_int4(0, 0, 0, 0);
-            *reinterpret_cast<int4*>(c.enter + l0) = make_int4(0, 0, 0, 0);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (l0 + j < nl) { c.leave[l0 + j] = 0; c.enter[l0 + j] = 0; }
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < LS_ROUNDS; ++r) {
-        const int l0 = wbase + r * 128 + 4 * ln;
-        // offset after the thread's 4th lane: the next thread's first
-        int onx = __shfl_down_sync(0xffffffffu, o[r][0], 1);
-        if (ln == 31) onx = o4[r];
-        long long rs = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool valid = l0 + j < nl;
-            const int onext = j < 3 ? o[r][j + 1] : onx;
-            ns[r][j] = valid ? (onext - o[r][j]) - lvv[r][j] + env[r][j] : 0;
-            rs += ns[r][j];
-        }
-        const long long p = rs;
-        long long incl = p;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, incl, d);
-            if (ln >= d) incl += y;
-        }
-        wpre[r] = run + incl - p;
-        run += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (ln == 0) s_wsum[w] = run;
-    __syncthreads();
-    long long wb = 0, total = 0;
-#pragma unroll
-    for (int k = 0; k < LS_WARPS; ++k) {
-        const long long x = s_wsum[k];
-        if (k < w) wb += x;
-        total += x;
-    }
-    if (threadIdx.x < 32) {
-        bool timeout = false;
-        unsigned long long prefix = 0;
-        if (tile == 0) {
-            if (threadIdx.x == 0) store_release(&c.lane_tiles[0], (2ull << 62) | (unsigned long long)total);
-        } else {
-            if (threadIdx.x == 0) store_release(&c.lane_tiles[tile], (1ull << 62) | (unsigned long long)total);
-            prefix = warp_lookback(c.lane_tiles, tile, &timeout);
-            if (threadIdx.x == 0) {
-                store_release(&c.lane_tiles[tile], (2ull << 62) | (prefix + (unsigned long long)total));
-                if (timeout) atomicOr(c.err, ERR_TIMEOUT);
-            }
-        }
-        if (threadIdx.x == 0) s_prefix = prefix;
-    }
-    __syncthreads();
-    const long long base = (long long)s_prefix + wb;
-#pragma unroll
-    for (int r = 0; r < LS_ROUNDS; ++r) {
-        const int l0 = wbase + r * 128 + 4 * ln;
-        const long long ex = base + wpre[r];
-        long long en = ex;
-        int on[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            on[j] = (int)en;
-            en += ns[r][j];
-        }
-        if (l0 + 4 <= nl) {
-            *reinterpret_cast<int4*>(c.nxt.off + l0) = make_int4(on[0], on[1], on[2], on[3]);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (l0 + j < nl) c.nxt.off[l0 + j] = on[j];
-        }
-        if (l0 < nl && nl <= l0 + 4) {  // this thread holds the last lane
-            c.nxt.off[nl] = (int)en;
-            c.cnt_next->n_cur = (int)en;
-        }
-    }
 }
 
 // Fit of the cost of a road-lane and a junction-lane vehicle in k_decide
@@ -739,7 +605,7 @@ __device__ __forceinline__ void lanescan_tile(const Ctx<Real>& c, int tile) {
 // slots) + c_junction x (junction slots) over the runs; the next step splits
 // its runs with the weight c_road / c_junction (clamped to [0.5, 4]; the
 // previous weight when the fit is degenerate, e.g. no junction vehicles).
-// One block (a ticket of k_lanescan); every work run rewrites its entry each
+// One block (a ticket of k_place); every work run rewrites its entry each
 // step.
 template <typename Real>
 __device__ void run_fit(const Ctx<Real>& c) {
@@ -781,107 +647,30 @@ __device__ void run_fit(const Ctx<Real>& c) {
     }
 }
 
-// k_lanescan.  Ticket 0: the run-weight fit.  Then (the first tickets below)
-// the late candidates and max-pressure sums, the next-snapshot lane offsets
-// (lane tiles, above), and the signal states of the next step for chunks of
-// junctions.
-template <typename Real, int LS_ROUNDS = 4>
-__device__ __forceinline__ void lanescan_blocks(const Ctx<Real>& c) {
-    __shared__ int s_tile;
-#if MOSS_FOLD_RESOLVE
-    // first tickets: the lane-change candidates (k_resolve's work) and the
-    // max-pressure sums, in chunks of TILE; the later tickets wait until all
-    // of those are done (their blocks hold earlier tickets, so they are
-    // running: the wait is bounded)
-    __shared__ int s_ready;
-    const int nc = c.cnt->n_late;  // candidates past the k_decide blocks' own lists
-    const int tag = c.cnt->tag;
-    const int r_cand = (nc + TILE - 1) / TILE;
-    const int n_res = r_cand + (*c.n_mp > 0 ? (c.n_jj + TILE - 1) / TILE : 0);
-    if (threadIdx.x == 0) s_ready = n_res == 0;
-#else
-    const int n_res = 0;
-#endif
-    const int n_tickets = 1 + n_res + c.n_lane_tiles + c.n_junc_chunks;
-    for (;;) {
-        if (threadIdx.x == 0) s_tile = atomicAdd(&c.cnt->ticket_lane, 1);
-        __syncthreads();
-        int tile = s_tile;
-        __syncthreads();
-        if (tile >= n_tickets) return;
-        // ticket 0: the run-weight fit of k_decide's runs (needs nothing else)
-        if (tile == 0) {
-            run_fit(c);
-            __syncthreads();
-            continue;
-        }
-        tile -= 1;
-#if MOSS_FOLD_RESOLVE
-        if (tile < n_res) {
-            MetricAcc acc;
-            macc_reset(acc, -1);
-            if (tile < r_cand) {
-                const int k = tile * TILE + threadIdx.x;
-                if (k < nc) resolve_one(c, acc, c.cand_late[k], c.n_veh, tag);
-            } else {
-                const int k = (tile - r_cand) * TILE + threadIdx.x;
-                if (k < c.n_jj) mp_accumulate(c, k);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                __threadfence();
-                atomicAdd(&c.cnt->res_done, 1);
-            }
-            // the metric sums are read by no later ticket: after the signal
-            macc_flush_block<TILE>(acc, c.metrics);
-            continue;
-        }
-        // lane tiles read the enter / leave counts the candidates change;
-        // junction tickets read only the max-pressure sums
-        if (!s_ready && (tile - n_res < c.n_lane_tiles || *c.n_mp > 0)) {
-            if (threadIdx.x == 0) {
-                cuda::atomic_ref<int, cuda::thread_scope_device> done(c.cnt->res_done);
-                long long spins = 0;
-                while (done.load(cuda::memory_order_acquire) < n_res) {
-                    if (++spins > SPIN_LIMIT) { atomicOr(c.err, ERR_TIMEOUT); break; }
-                    if (spins > 16) __nanosleep(64);
-                }
-                s_ready = 1;
-            }
-            __syncthreads();
-        }
-        tile -= n_res;
-#endif
-        if (tile < c.n_lane_tiles) {
-            lanescan_tile<Real, LS_ROUNDS>(c, tile);
-        } else {
-            // signal states of the next step
-            const int j0 = (tile - c.n_lane_tiles) * JUNC_CHUNK;
-            const int j = j0 + threadIdx.x;
-            if (j < c.n_junctions && !c.scen_ctl[c.junc[j].scen])
-                c.junc_state[j] = c.junc_policy[j] == POL_MAXP ? mp_advance(c, j) : junction_state_at(c, j, 1);
-        }
-        __syncthreads();
-    }
-}
-
-template <typename Real, int LS_ROUNDS>
-__global__ void __launch_bounds__(LANESCAN_THREADS) k_lanescan(Ctx<Real> c) {
-    if (*c.err & ERR_POISON) return;
-    lanescan_blocks<Real, LS_ROUNDS>(c);
-}
-
 // ---------------------------------------------------------------------------
-// k_place: writes the next snapshot.  Stayer tiles (one per block iteration):
-// a vehicle that kept its lane goes to off'[lane] + (stayers ahead of it in
-// the lane) + (entrants ahead of it), its stayers ahead counted in its tile
-// (below).  Then the entrants: rank = stayers ahead + entrants ahead.  Block
-// 0 prepares the next step's counters and advances the scenarios' clocks.
+// k_place: the lane offsets of the next snapshot, then the snapshot itself.
+//
+// A tile is a run of whole lanes [tile_cur[t], tile_cur[t+1]) with their
+// vehicles, cut where slot_w * off[l] + lane_w * l passes a multiple of
+// 1 << tile_shift
+// (the previous step's tiles wrote the cuts).  newsize(l) = size(l) - leave(l)
+// + enter(l).  k_decide also counts how each tile grows (tile_delta), so the
+// next offset of a tile's first lane is its offset now plus the growth of the
+// tiles before it: every tile adds those words up for itself and no tile
+// waits for another.  The vehicles of a lane lie in the tile, so a stayer's
+// next slot is its own slot plus a per-lane shift, minus the leavers before it
+// in the tile, plus the entrants ahead of it.
+//
+// Latency-bound on small networks and bandwidth-bound on large ones, so the
+// tile size follows the network (place_shift on the host).  Everything the
+// step before wrote (cuts, offsets, records) is loaded before grid_wait, past
+// L1: the tail of k_decide covers it.
+
+// entrants of a list (from q on) that are ahead of (s, id); n_in: its length
 template <typename Real>
-__device__ __forceinline__ int entrants_ahead(const Ctx<Real>& c, int lane, Real s, int id, int tag,
-                                              int* n_in = nullptr) {
+__device__ __forceinline__ int entrants_ahead(const Ctx<Real>& c, int q, Real s, int id, int* n_in = nullptr) {
     int cnt = 0, guard = 0;
-    for (int q = list_head(c.head, lane, tag); q >= 0; q = c.enext[q]) {
+    for (; q >= 0; q = c.enext[q]) {
         const RecA<Real> Q = c.ea[q];
         if (ahead(Q.s, Q.id, s, id)) ++cnt;
         if (++guard > c.n_veh) { atomicOr(c.err, ERR_RANGE); break; }
@@ -890,33 +679,448 @@ __device__ __forceinline__ int entrants_ahead(const Ctx<Real>& c, int lane, Real
     return cnt;
 }
 
+constexpr int TW = TILE / 32;           // warps per block
+constexpr int PLACE_ROUNDS = 16;        // slot rounds whose leaver masks are held at a time
+constexpr int PLACE_LANES_LOG2 = 11;    // a tile holds at most 2^11 lanes
+// shared memory of a tile with up to `lanes` lanes: next offset (one more),
+// shift, entrants and their list per lane
+__host__ __device__ constexpr size_t place_smem(int lanes) { return sizeof(int) * (4 * (size_t)lanes + 1); }
+// lanes of the widest tile: each one adds at least lane_w
+__host__ __device__ constexpr int place_lanes(int tile_shift, int lane_w) {
+    return ((1 << tile_shift) + lane_w - 1) / lane_w;
+}
+
+// the clocks of every scenario, one step on (a frozen or retiring one stands
+// still; one that reaches its horizon freezes)
 template <typename Real>
-__device__ __forceinline__ void place_blocks(const Ctx<Real>& c, int vb, int nvb) {
+__device__ __forceinline__ void advance_clocks(const Ctx<Real>& c) {
+    for (int s = threadIdx.x; s < c.n_scen; s += TILE) {
+        if (c.scen_ctl[s]) continue;
+        const long long t = c.scen_step[s] + 1;
+        c.scen_step[s] = t;
+        if (t == c.stop_at[s]) c.scen_ctl[s] = SC_FROZEN;
+    }
+}
+
+template <typename Real, bool Pdl>
+__device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
+    extern __shared__ int s_lanes[];
+    __shared__ unsigned long long s_wsum[TW];       // per warp: leavers << 32 | next size of its lanes
+    __shared__ unsigned s_ball[PLACE_ROUNDS * TW];  // leaver mask of each 32 slots
+    __shared__ int s_lp[PLACE_ROUNDS * TW];         // leavers of the tile before them
+    __shared__ int s_sum[TW];
+    __shared__ int s_nel;                           // lanes with entrants
+    const int cap = place_lanes(c.tile_shift, c.lane_w);
+    int* const s_nx = s_lanes;            // [cap + 1] next offset of a lane
+    int* const s_sh = s_lanes + cap + 1;  // [cap] next slot - slot of a lane's first vehicle, + leavers before the lane
+    int* const s_hd = s_sh + cap;         // [cap] entrants of a lane: -1 none; >= 0 list; <= -2: one, ahead of the last
+                                          // -2 - s_hd stayers
+    int* const s_el = s_hd + cap;         // [cap] lanes with entrants
+    const int tid = threadIdx.x, ln = tid & 31, w = tid >> 5;
+    // ---- what the previous step wrote
+    const int tag = __ldcg(&c.cnt->tag);
+    const int L0 = __ldcg(&c.tile_cur[tile]), L1 = __ldcg(&c.tile_cur[tile + 1]), m = L1 - L0;
+    const int S0 = __ldcg(&c.cur.off[L0]), S1 = __ldcg(&c.cur.off[L1]);
+    const int K = (m + TILE - 1) / TILE;  // lane rounds of a warp
+    const int kw = w * 32 * K + ln;       // the thread's first lane of the tile
+    int o0 = 0, o1 = 0;
+    if (kw < m) {
+        o0 = __ldcg(&c.cur.off[L0 + kw]);
+        o1 = __ldcg(&c.cur.off[L0 + kw + 1]);
+    }
+    int2 al = make_int2(-1, -1);  // id, lane of the first round's record
+    int4 ab = make_int4(0, 0, 0, 0);
+    if (S0 + tid < S1) {
+        al = __ldcg(reinterpret_cast<const int2*>(&c.cur.a[S0 + tid].id));
+        ab = __ldcg(reinterpret_cast<const int4*>(&c.cur.b[S0 + tid]));
+    }
+    if (tid == 0) s_nel = 0;
+    __syncthreads();
+    if (Pdl) {
+        grid_wait();
+        grid_release();
+    }
+    const int poison = tid == 0 ? *c.err & ERR_POISON : 0;
+    // ---- lanes: sizes, leavers, entrant lists; prefixes within the warp
+    SV<Real> st0;
+    int8_t code0 = C_STAY;
+    if (S0 + tid < S1) {
+        code0 = c.code[S0 + tid];
+        st0 = c.stay[S0 + tid];
+    }
+    int grown = 0;
+    for (int p = tid; p < tile; p += TILE) grown += c.tile_delta[p];
+    unsigned long long run = 0;
+    for (int r = 0; r < K; ++r) {
+        const int k = kw + 32 * r, l = L0 + k;
+        unsigned long long x = 0;
+        if (k < m) {
+            if (r) { o0 = c.cur.off[l]; o1 = c.cur.off[l + 1]; }
+            const int lv = c.leave[l], en = c.enter[l];
+            const unsigned long long h = c.head[l];
+            if (lv) c.leave[l] = 0;
+            s_hd[k] = -1;
+            if (en) {
+                c.enter[l] = 0;
+                if ((int)(h >> 32) == tag) s_hd[k] = (int)(unsigned)(h & 0xffffffffull);
+                s_el[atomicAdd(&s_nel, 1)] = k;
+            }
+            x = ((unsigned long long)(unsigned)lv << 32) | (unsigned)(o1 - o0 - lv + en);
+        }
+        unsigned long long incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (ln >= o) incl += y;
+        }
+        const unsigned long long ex = run + incl - x;
+        if (k < m) {
+            s_nx[k] = (int)(unsigned)(ex & 0xffffffffull);
+            s_sh[k] = (int)(ex >> 32) - o0;
+        }
+        run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (ln == 0) s_wsum[w] = run;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) grown += __shfl_xor_sync(0xffffffffu, grown, o);
+    if (ln == 0) s_sum[w] = grown;
+    // ---- the leavers of the first slot rounds
+    const int nr = min((S1 - S0 + TILE - 1) / TILE, PLACE_ROUNDS);
+    for (int r = 0; r < nr; ++r) {
+        const int i = S0 + r * TILE + tid;
+        const int8_t code = r == 0 ? code0 : (i < S1 ? c.code[i] : (int8_t)C_STAY);
+        const unsigned b = __ballot_sync(0xffffffffu, code != C_STAY);
+        if (ln == 0) s_ball[r * TW + w] = b;
+    }
+    if (__syncthreads_or(poison)) return;
+    unsigned long long wb = 0, tot = 0;
+    int prefix = S0;
+#pragma unroll
+    for (int k = 0; k < TW; ++k) {
+        const unsigned long long x = s_wsum[k];
+        if (k < w) wb += x;
+        tot += x;
+        prefix += s_sum[k];
+    }
+    if (w == TW - 1) {  // leavers before each 32 slots
+        int carry = 0;
+        for (int k0 = 0; k0 < nr * TW; k0 += 32) {
+            const int x = k0 + ln < nr * TW ? __popc(s_ball[k0 + ln]) : 0;
+            int incl = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (ln >= o) incl += y;
+            }
+            if (k0 + ln < nr * TW) s_lp[k0 + ln] = carry + incl - x;
+            carry += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+    const int nb = prefix + (int)(unsigned)(wb & 0xffffffffull), lb = (int)(wb >> 32);
+    for (int r = 0; r < K; ++r) {
+        const int k = kw + 32 * r;
+        if (k < m) {
+            const int nx = nb + s_nx[k];
+            c.nxt.off[L0 + k] = nx;
+            s_nx[k] = nx;
+            s_sh[k] += nx + lb;
+        }
+    }
+    if (tid == 0) s_nx[m] = prefix + (int)(unsigned)(tot & 0xffffffffull);
+    __syncthreads();
+    // ---- the next step's tile cuts and the ends of the snapshot
+    for (int k = tid; k < m; k += TILE) {
+        const int l = L0 + k;
+        const int q0 = tile_key(c, s_nx[k], l), q1 = tile_key(c, s_nx[k + 1], l + 1);
+        for (int q = q0 + 1; q <= q1; ++q) c.tile_nxt[q] = l + 1;
+        if (l + 1 == c.n_lanes) {
+            c.nxt.off[l + 1] = s_nx[k + 1];
+            c.cnt_next->n_cur = s_nx[k + 1];
+            c.tile_nxt[q1 + 1] = l + 1;
+        }
+    }
+    // ---- entrants: eight threads per lane that has any, four lanes at a time
+    // in a warp.  The stayers of a lane keep their order (nobody overtakes
+    // within a lane, R13), so the stayers behind an entrant form the rear of
+    // the lane's old segment: they are counted from the segment's end, 8
+    // slots per round, up to the first round that holds a stayer ahead of the
+    // entrant (entrants join mostly at the rear of a lane: one round).
+    // Stayers ahead = the lane's stayers (its next size minus its entrants)
+    // minus those behind.
+    const int sub = ln >> 3, sl = ln & 7, nel = s_nel;
+    for (int j0 = 4 * w; j0 < nel; j0 += 4 * TW) {
+        int q = -1, k = 0, b = 0, e = 0;
+        if (j0 + sub < nel) {
+            k = s_el[j0 + sub];
+            q = s_hd[k];
+            b = c.cur.off[L0 + k];
+            e = c.cur.off[L0 + k + 1];
+        }
+        const int q0 = q;
+        int n_in = 0, bh = 0;
+        while (__any_sync(0xffffffffu, q >= 0)) {
+            RecA<Real> Q;
+            RecB QB;
+            int nq = -1;
+            if (q >= 0) {
+                Q = c.ea[q];
+                nq = c.enext[q];
+                if (sl == 0) QB = c.eb[q];
+            }
+            if (q >= 0) bh = 0;  // (a lane that is through keeps its count while others go on)
+            bool open = q >= 0;
+            for (int x0 = e - 1; __any_sync(0xffffffffu, open); x0 -= 8) {
+                const int x = x0 - sl;
+                bool st = false, ah = false;
+                if (open && x >= b && c.code[x] == C_STAY) {
+                    st = true;
+                    ah = ahead(c.stay[x].s, c.cur.a[x].id, Q.s, Q.id);
+                }
+                const unsigned mb = (__ballot_sync(0xffffffffu, st && !ah) >> (8 * sub)) & 0xffu;
+                const unsigned ma = (__ballot_sync(0xffffffffu, ah) >> (8 * sub)) & 0xffu;
+                bh += __popc(mb);
+                if (ma || x0 - 8 < b) open = false;
+            }
+            if (q >= 0) {
+                if (sl == 0) {
+                    int len = 1, ent = 0;
+                    if (nq >= 0 || q != q0) ent = entrants_ahead(c, q0, Q.s, Q.id, &len);
+                    const int pos = s_nx[k + 1] - len - bh + ent;
+                    if (pos < s_nx[k] || pos >= s_nx[k + 1] || pos >= c.n_veh) {
+                        atomicOr(c.err, ERR_RANGE);
+                    } else {
+                        c.nxt.a[pos] = Q;
+                        c.nxt.b[pos] = QB;
+                    }
+                }
+                q = nq;
+                if (++n_in > c.n_veh) { atomicOr(c.err, ERR_RANGE); q = -1; }
+            }
+        }
+        if (n_in == 1 && sl == 0) s_hd[k] = -2 - bh;
+    }
+    __syncthreads();
+    // ---- stayers
+    int lcarry = 0;  // leavers of the rounds before the held ones
+    for (int r0 = 0; S0 + r0 * TILE < S1; r0 += PLACE_ROUNDS) {
+        const int nh = min((S1 - S0 + TILE - 1) / TILE - r0, PLACE_ROUNDS);
+        if (r0) {  // (a lane of thousands of vehicles)
+            __syncthreads();
+            for (int r = 0; r < nh; ++r) {
+                const int i = S0 + (r0 + r) * TILE + tid;
+                const unsigned b = __ballot_sync(0xffffffffu, i < S1 && c.code[i] != C_STAY);
+                if (ln == 0) s_ball[r * TW + w] = b;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                int x = 0;
+                for (int k = 0; k < nh * TW; ++k) {
+                    s_lp[k] = x;
+                    x += __popc(s_ball[k]);
+                }
+            }
+            __syncthreads();
+        }
+#pragma unroll 2
+        for (int r = 0; r < nh; ++r) {
+            const int i = S0 + (r0 + r) * TILE + tid;
+            const unsigned ball = s_ball[r * TW + w];
+            if (i >= S1 || ((ball >> ln) & 1u)) continue;
+            SV<Real> sv = st0;
+            if (r0 + r > 0) {
+                al = *reinterpret_cast<const int2*>(&c.cur.a[i].id);
+                ab = *reinterpret_cast<const int4*>(&c.cur.b[i]);
+                sv = c.stay[i];
+            }
+            const int lane = al.y, k = lane - L0;
+            const int o = s_nx[k], end = s_nx[k + 1], h = s_hd[k];
+            int pos = s_sh[k] + i - (lcarry + s_lp[r * TW + w] + __popc(ball & ((1u << ln) - 1u)));
+            if (h >= 0) pos += entrants_ahead(c, h, sv.s, al.x);
+            else if (h != -1) pos += end - 2 - pos < -2 - h;  // stayers behind it: end - 2 - pos
+            if (pos < o || pos >= end || pos >= c.n_veh) {
+                atomicOr(c.err, ERR_RANGE);
+            } else {
+                RecA<Real> O;
+                O.s = sv.s; O.v = sv.v; O.id = al.x; O.lane = lane;
+                c.nxt.a[pos] = O;
+                *reinterpret_cast<int4*>(&c.nxt.b[pos]) = ab;
+            }
+        }
+        lcarry += s_lp[nh * TW - 1] + __popc(s_ball[nh * TW - 1]);
+    }
+}
+
+// Block vb of the first n_junc_chunks + 1 blocks of the kernel after k_decide:
+// the signal states of the next step (JUNC_CHUNK junctions each; with Clocks
+// the last of them to finish advances the clocks, which nothing else of the
+// kernel reads), then the run-weight fit with the next step's counters.  Pdl:
+// the kernel may have started before k_decide ended.
+template <typename Real, bool Pdl, bool Clocks>
+__device__ __forceinline__ void close_step(const Ctx<Real>& c, int vb) {
+    const int nj = c.n_junc_chunks;
+    if (Pdl) {
+        grid_wait();
+        grid_release();
+    }
+    if (__syncthreads_or(threadIdx.x == 0 ? *c.err & ERR_POISON : 0)) return;
+    if (vb < nj) {
+        __shared__ int s_clocks;
+        const int j = vb * JUNC_CHUNK + threadIdx.x;
+        if (j < c.n_junctions && !c.scen_ctl[c.junc[j].scen])
+            c.junc_state[j] = c.junc_policy[j] == POL_MAXP ? mp_advance(c, j) : junction_state_at(c, j, 1);
+        if (!Clocks) return;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_clocks = nj == 1 || atomicAdd(&c.cnt->junc_done, 1) == nj - 1;
+            __threadfence();
+        }
+        __syncthreads();
+        if (s_clocks) advance_clocks(c);
+        return;
+    }
+    if (threadIdx.x == 0) {
+        const int tag = c.cnt->tag;
+        c.cnt_next->n_ent = 0;
+        c.cnt_next->n_cand = 0;
+        c.cnt_next->junc_done = 0;
+        c.cnt_next->tag = tag >= 0x3fffffff ? 1 : tag + 1;
+    }
+    if (Clocks && nj == 0) advance_clocks(c);
+    run_fit(c);
+}
+
+// Virtual block vb of the fused form: close_step's, then the tiles.
+template <typename Real, bool Pdl>
+__device__ __forceinline__ void place_block(const Ctx<Real>& c, int vb) {
+    const int tile = vb - c.n_junc_chunks - 1;
+    if (tile < 0) {
+        close_step<Real, Pdl, true>(c, vb);
+        return;
+    }
+    if (threadIdx.x == 0) c.delta_nxt[tile] = 0;  // (last read by the step before)
+    if (tile > tile_key(c, __ldcg(&c.cnt->n_cur), c.n_lanes)) return;
+    place_tile<Real, Pdl>(c, tile);
+}
+
+#ifndef MOSS_PLACE_MIN_BLOCKS
+#define MOSS_PLACE_MIN_BLOCKS 6
+#endif
+template <typename Real>
+__global__ void __launch_bounds__(TILE, MOSS_PLACE_MIN_BLOCKS) k_place(Ctx<Real> c) {
+    place_block<Real, true>(c, blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
+// The form for large networks, where the work of a tile no longer hides behind
+// its latencies: the offsets in a kernel of their own (k_lanescan), then one
+// thread per slot and one warp per entrant, whatever their lanes
+// (k_place_slots).  Here a tile is SCAN_TILE consecutive lanes (tile_shift
+// counts lanes, slot_w is 0).
+constexpr int SCAN_TILE_LOG2 = 10;
+static_assert((1 << SCAN_TILE_LOG2) == 4 * TILE, "four lanes per thread");
+
+// Lane tiles: newsize(l) = size(l) - leave(l) + enter(l), its prefix sum
+// within the tile, and the growth of the tiles before it (tile_delta).  Four
+// consecutive lanes per thread: the 16-byte loads and stores of a warp cover
+// 512 contiguous bytes.  Bound by one memory round trip.
+template <typename Real>
+__global__ void __launch_bounds__(TILE) k_lanescan(Ctx<Real> c) {
+    const int tile = (int)blockIdx.x - c.n_junc_chunks - 1;
+    if (tile < 0) {
+        close_step<Real, true, false>(c, blockIdx.x);
+        return;
+    }
+    __shared__ int s_w[TW], s_g[TW];
+    const int ln = threadIdx.x & 31, w = threadIdx.x >> 5, nl = c.n_lanes;
+    const int l0 = (tile << SCAN_TILE_LOG2) + 4 * (int)threadIdx.x;
+    if (threadIdx.x == 0) c.delta_nxt[tile] = 0;  // (last read by the step before)
+    // offsets (written by the step before): o[4] is the end of the fourth lane
+    int o[5] = {0, 0, 0, 0, 0};
+    if (l0 + 4 <= nl) {
+        const int4 x = __ldcg(reinterpret_cast<const int4*>(c.cur.off + l0));
+        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
+        o[4] = __ldcg(c.cur.off + l0 + 4);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+            if (l0 + j <= nl) o[j] = __ldcg(c.cur.off + l0 + j);
+    }
+    const int first = __ldcg(c.cur.off + (tile << SCAN_TILE_LOG2));
+    grid_wait();
+    grid_release();
+    if (*c.err & ERR_POISON) return;  // (set by a kernel that has ended)
+    int lv[4] = {0, 0, 0, 0}, en[4] = {0, 0, 0, 0};
+    if (l0 + 4 <= nl) {
+        const int4 x = *reinterpret_cast<const int4*>(c.leave + l0), y = *reinterpret_cast<const int4*>(c.enter + l0);
+        lv[0] = x.x; lv[1] = x.y; lv[2] = x.z; lv[3] = x.w;
+        en[0] = y.x; en[1] = y.y; en[2] = y.z; en[3] = y.w;
+        *reinterpret_cast<int4*>(c.leave + l0) = make_int4(0, 0, 0, 0);
+        *reinterpret_cast<int4*>(c.enter + l0) = make_int4(0, 0, 0, 0);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (l0 + j < nl) {
+                lv[j] = c.leave[l0 + j]; en[j] = c.enter[l0 + j];
+                c.leave[l0 + j] = 0; c.enter[l0 + j] = 0;
+            }
+    }
+    int grown = 0;
+    for (int p = threadIdx.x; p < tile; p += TILE) grown += c.tile_delta[p];
+    int ns[4], sum = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        ns[j] = l0 + j < nl ? o[j + 1] - o[j] - lv[j] + en[j] : 0;
+        sum += ns[j];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (ln >= d) incl += y;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) grown += __shfl_xor_sync(0xffffffffu, grown, d);
+    if (ln == 31) { s_w[w] = incl; s_g[w] = grown; }
+    __syncthreads();
+    int at = first + incl - sum;
+#pragma unroll
+    for (int k = 0; k < TW; ++k) at += s_g[k] + (k < w ? s_w[k] : 0);
+    int on[5];
+    on[0] = at;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) on[j + 1] = on[j] + ns[j];
+    if (l0 + 4 <= nl) {
+        *reinterpret_cast<int4*>(c.nxt.off + l0) = make_int4(on[0], on[1], on[2], on[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (l0 + j < nl) c.nxt.off[l0 + j] = on[j];
+    }
+    if (l0 < nl && nl <= l0 + 4) {  // this thread holds the last lane (on[] stays at the end past it)
+        c.nxt.off[nl] = on[4];
+        c.cnt_next->n_cur = on[4];
+    }
+}
+
+// The next snapshot.  Stayer tiles (one per block iteration): a vehicle that
+// kept its lane goes to off'[lane] + (stayers ahead of it in the lane) +
+// (entrants ahead of it), its stayers ahead counted in its tile (below).
+// Then the entrants: rank = stayers ahead + entrants ahead.  Block 0 advances
+// the clocks, which k_lanescan reads and this kernel does not.
+template <typename Real>
+__global__ void __launch_bounds__(TILE) k_place_slots(Ctx<Real> c) {
+    const int vb = blockIdx.x, nvb = gridDim.x;
+    grid_wait();
+    grid_release();
+    if (__syncthreads_or(threadIdx.x == 0 ? *c.err & ERR_POISON : 0)) return;
+    if (vb == 0) advance_clocks(c);
     __shared__ int s_warp[TILE / 32];
     const int n = c.cnt->n_cur;
     const int n_ent = c.cnt->n_ent;
     const int tag = c.cnt->tag;
     const int n_tiles = (n + TILE - 1) / TILE;
     const int lane_id = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // closing the step: the next step's counters (k_lanescan already wrote
-    // its vehicle count) and every scenario's clock; no kernel of this step
-    // reads them after this point
-    if (vb == 0) {
-        if (threadIdx.x == 0) {
-            c.cnt_next->n_ent = 0;
-            c.cnt_next->n_cand = 0;
-            c.cnt_next->n_late = 0;
-            c.cnt_next->res_done = 0;
-            c.cnt_next->ticket_lane = 0;
-            c.cnt_next->tag = tag >= 0x3fffffff ? 1 : tag + 1;
-        }
-        for (int s = threadIdx.x; s < c.n_scen; s += TILE) {
-            if (c.scen_ctl[s]) continue;  // frozen or retiring: its clock stands still
-            const long long t = c.scen_step[s] + 1;
-            c.scen_step[s] = t;
-            if (t == c.stop_at[s]) c.scen_ctl[s] = SC_FROZEN;  // reached its horizon
-        }
-    }
     __shared__ int s_lpre[TILE + 1];  // leavers among the tile's slots before each slot (and in all)
     __shared__ int s_first[2];        // start and end of the lane that holds the tile's first slot
     for (int tile = vb; tile < n_tiles; tile += nvb) {
@@ -964,7 +1168,7 @@ __device__ __forceinline__ void place_blocks(const Ctx<Real>& c, int vb, int nvb
             const int ob = c.cur.off[lane], oe = c.cur.off[lane + 1];
             const int o0 = c.nxt.off[lane], o1 = c.nxt.off[lane + 1];
             int n_in = 0;
-            const int ent = entrants_ahead(c, lane, w.s, A.id, tag, &n_in);
+            const int ent = entrants_ahead(c, list_head(c.head, lane, tag), w.s, A.id, &n_in);
             const int x = threadIdx.x;
             int stay_rank;
             if (ob >= t0) {
@@ -1012,7 +1216,7 @@ __device__ __forceinline__ void place_blocks(const Ctx<Real>& c, int vb, int nvb
         }
         if (lane_id == 0) {
             int n_in = 0;
-            const int ent_ahead = entrants_ahead(c, lane, Q.s, Q.id, tag, &n_in);
+            const int ent_ahead = entrants_ahead(c, list_head(c.head, lane, tag), Q.s, Q.id, &n_in);
             const int o0 = c.nxt.off[lane], o1 = c.nxt.off[lane + 1];
             const int pos = o0 + (o1 - o0 - n_in - behind) + ent_ahead;
             if (pos < o0 || pos >= o1) {
@@ -1023,21 +1227,24 @@ __device__ __forceinline__ void place_blocks(const Ctx<Real>& c, int vb, int nvb
             }
         }
     }
-    // clear the lane look-back words for the next step (k_lanescan is done)
-    for (int k = vb * TILE + threadIdx.x; k < c.n_lane_tiles; k += nvb * TILE)
-        c.lane_tiles[k] = 0ull;
 }
 
+// tile cuts of the current snapshot's offsets (after creation, a state reset
+// or a change of the tile size; one thread per lane)
 template <typename Real>
-__global__ void __launch_bounds__(TILE) k_place(Ctx<Real> c) {
-    if (*c.err & ERR_POISON) return;
-    place_blocks(c, blockIdx.x, gridDim.x);
+__global__ void k_tile_cuts(Ctx<Real> c) {
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
+    if (l == 0) c.tile_cur[0] = c.tile_nxt[0] = 0;
+    if (l >= c.n_lanes) return;
+    const int q0 = tile_key(c, c.cur.off[l], l), q1 = tile_key(c, c.cur.off[l + 1], l + 1);
+    for (int q = q0 + 1; q <= q1; ++q) c.tile_cur[q] = l + 1;
+    if (l + 1 == c.n_lanes) c.tile_cur[q1 + 1] = l + 1;
 }
 
 // ---------------------------------------------------------------------------
 // The whole step as one cooperative launch (every block resident at once):
-// the work of k_decide, k_lanescan and k_place as three phases separated by
-// grid-wide barriers.  A barrier is a count of arrived blocks and a
+// the work of k_decide and k_place as two phases separated by a grid-wide
+// barrier.  A barrier is a count of arrived blocks and a
 // generation word; a wait that exceeds SPIN_LIMIT sets ERR_TIMEOUT and every
 // block leaves the step.
 __device__ __forceinline__ bool grid_sync(unsigned* bar, int* err) {
@@ -1069,15 +1276,16 @@ __device__ __forceinline__ bool grid_sync(unsigned* bar, int* err) {
 #endif
 template <typename Real, bool Groups>
 __global__ void __launch_bounds__(TILE, MOSS_COOP_MIN_BLOCKS) k_step_coop(Ctx<Real> c, int n_work, int n_ins,
-                                                                          unsigned* bar) {
+                                                                          int n_place, unsigned* bar) {
     if (*c.err & ERR_POISON) return;
     // decide: n_work tile runs, then n_ins insertion blocks, as virtual blocks
     for (int vb = blockIdx.x; vb < n_work + n_ins; vb += gridDim.x)
         decide_block<Real, Groups>(c, n_work, vb, n_work + n_ins);
     if (!grid_sync(bar, c.err)) return;
-    lanescan_blocks(c);
-    if (!grid_sync(bar, c.err)) return;
-    place_blocks(c, blockIdx.x, gridDim.x);
+    for (int vb = blockIdx.x; vb < n_place; vb += gridDim.x) {
+        place_block<Real, false>(c, vb);
+        __syncthreads();  // shared memory serves the next one
+    }
 }
 
 // signal states for the current step of every junction (after creation or
