@@ -440,8 +440,10 @@ Ctx<Real> make_ctx(MossHandle* h, int cur) {
     const MossParams& p = h->prm;
     c.dt = Real(p.dt); c.a_max = Real(p.a_max); c.b_comf = Real(p.b_comf); c.T = Real(p.T);
     c.s0 = Real(p.s0); c.len = Real(p.veh_len); c.pol = Real(p.politeness); c.a_th = Real(p.a_th);
-    c.b_safe = Real(p.b_safe); c.p_att = Real(p.p_attempt); c.p_hi = Real(p.p_hi); c.p_lo = Real(p.p_lo);
+    c.b_safe = Real(p.b_safe); c.p_hi = Real(p.p_hi); c.p_lo = Real(p.p_lo);
     c.band = Real(p.flag_band);
+    const double att = std::ceil((double)Real(p.p_attempt) * 16777216.0);
+    c.att24 = att > 0.0 ? (uint32_t)std::min(att, 16777216.0) : 0u;
     c.inv_2sqrt_ab = Real(1.0 / (2.0 * std::sqrt(p.a_max * p.b_comf)));
     return c;
 }
@@ -480,7 +482,11 @@ template <typename Real, bool Groups>
 cudaError_t launch_coop(MossHandle* h, Ctx<Real>& c) {
     int per_sm = 0;
     const size_t smem = grids(h).place_smem;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_coop<Real, Groups>, TILE, smem);
+    // (its static part and a wide tile's lanes pass 48 KB together in FP64)
+    cudaError_t e = cudaFuncSetAttribute(k_step_coop<Real, Groups>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)place_smem(1 << PLACE_LANES_LOG2));
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_coop<Real, Groups>, TILE, smem);
     if (e != cudaSuccess) return e;
     int grid = std::max(1, per_sm) * h->sm_count;
     int n_work = std::max(1, std::min((h->n_veh + 31) / 32, grid));

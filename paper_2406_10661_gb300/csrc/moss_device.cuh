@@ -226,8 +226,9 @@ struct Ctx {
     Counters* cnt_next;  // the next step's
     int* err;            // device error bits
     // ---- parameters
-    Real dt, a_max, b_comf, T, s0, len, pol, a_th, b_safe, p_att, p_hi, p_lo, band;
+    Real dt, a_max, b_comf, T, s0, len, pol, a_th, b_safe, p_hi, p_lo, band;
     Real inv_2sqrt_ab;  // 1 / (2 sqrt(a b)), computed in double on the host
+    uint32_t att24;     // the attempt draw passes when its 24 bits are below this (ceil(p_attempt 2^24))
 };
 
 // ---------------------------------------------------------------------------
@@ -254,7 +255,34 @@ __device__ __forceinline__ Real unit24(uint32_t w) {
     return Real(w >> 8) * Real(5.9604644775390625e-08);  // 2^-24, exact
 }
 
-template <typename Real> __device__ __forceinline__ Real rabs(Real x) { return x < Real(0) ? -x : x; }
+__device__ __forceinline__ float rabs(float x) { return fabsf(x); }
+__device__ __forceinline__ double rabs(double x) { return fabs(x); }
+
+// An FP64 instruction takes an SM of this part 16 cycles per warp (two lanes a
+// cycle), an integer one a fraction of that, so in FP64 the comparisons that
+// decide nothing by rounding are made on the bit patterns: doubles >= 0 are
+// ordered like their bits.
+
+// x > t for t >= +0 (false for NaN)
+__device__ __forceinline__ bool gt(float x, float t) { return x > t; }
+__device__ __forceinline__ bool gt(double x, double t) {
+    const long long tb = __double_as_longlong(t);
+    return (unsigned long long)(__double_as_longlong(x) - tb - 1) < (unsigned long long)(0x7ff0000000000000ll - tb);
+}
+
+// |x| < band * scale (an uncertain discrete decision, R22); in FP64 the
+// product is formed only when the exponents leave it open
+__device__ __forceinline__ bool within(float x, float band, float scale) { return rabs(x) < band * scale; }
+__device__ __forceinline__ bool within(double x, double band, double scale) {
+    // |x| >= 2^ex, band * scale <= 2^(eb + es + 2) (exponents biased by 1023)
+    const int ex = (__double2hiint(x) >> 20) & 0x7ff, eb = (__double2hiint(band) >> 20) & 0x7ff,
+              es = (__double2hiint(scale) >> 20) & 0x7ff;
+    if (ex + 1023 >= eb + es + 2) return false;
+    return rabs(x) < band * scale;
+}
+// max(x, 1)
+__device__ __forceinline__ float at_least_1(float x) { return x > 1.0f ? x : 1.0f; }
+__device__ __forceinline__ double at_least_1(double x) { return gt(x, 1.0) ? x : 1.0; }
 
 // speed in units of 2^-24 m/s, rounded to nearest (for the speed metric).  In
 // FP32 the product by 2^24 is exact and fits a 32-bit integer below 128 m/s,
@@ -274,21 +302,30 @@ template <> __device__ __forceinline__ float qdiv<float>(float x, float y) { ret
 #endif
 
 // ---------------------------------------------------------------------------
-// IDM, App. B.3 eqs. (1)-(2), delta = 4 as ((v/v0)^2)^2.
+// IDM, App. B.3 eqs. (1)-(2), delta = 4 as ((v/v0)^2)^2.  free_term is the
+// part that depends on the vehicle's own speed, shared by every IDM value of
+// a vehicle on lanes of one speed limit.
 template <typename Real>
-__device__ __forceinline__ Real idm_free(const Ctx<Real>& c, Real v, Real v0) {
+__device__ __forceinline__ Real free_term(Real v, Real v0) {
     const Real r = qdiv(v, v0), r2 = r * r;
-    return c.a_max * (Real(1) - r2 * r2);
+    return Real(1) - r2 * r2;
 }
 
+__device__ __forceinline__ float fma_rn(float a, float b, float x) { return __fmaf_rn(a, b, x); }
+__device__ __forceinline__ double fma_rn(double a, double b, double x) { return __fma_rn(a, b, x); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// f: the vehicle's free term.  The sum of s* is written as the fused
+// multiply-add it is, so that every use rounds alike whatever the compiler
+// shares between uses.
 template <typename Real>
-__device__ __forceinline__ Real idm(const Ctx<Real>& c, Real v, Real v0, Real gap, Real dv) {
-    const Real r = qdiv(v, v0), r2 = r * r;
-    const Real dyn = v * c.T + v * dv * c.inv_2sqrt_ab;
-    const Real sstar = c.s0 + (dyn > Real(0) ? dyn : Real(0));
-    const Real g = gap > Real(1e-3) ? gap : Real(1e-3);
+__device__ __forceinline__ Real idm(const Ctx<Real>& c, Real v, Real f, Real gap, Real dv) {
+    const Real dyn = fma_rn(v, c.T, mul_rn(mul_rn(v, dv), c.inv_2sqrt_ab));
+    const Real sstar = c.s0 + (gt(dyn, Real(0)) ? dyn : Real(0));
+    const Real g = gt(gap, Real(1e-3)) ? gap : Real(1e-3);
     const Real q = qdiv(sstar, g);
-    return c.a_max * (Real(1) - r2 * r2 - q * q);
+    return c.a_max * (f - q * q);
 }
 
 template <typename Real>
@@ -445,6 +482,12 @@ template <typename Real>
 __device__ __forceinline__ bool ahead(Real sa, int ia, Real sb, int ib) {
     return sa > sb || (sa == sb && ia < ib);
 }
+// (positions are >= 0; -0 counts as 0)
+template <>
+__device__ __forceinline__ bool ahead<double>(double sa, int ia, double sb, int ib) {
+    const long long a = max(__double_as_longlong(sa), 0ll), b = max(__double_as_longlong(sb), 0ll);
+    return a > b || (a == b && ia < ib);
+}
 
 // first slot in [b, e) of the current snapshot that is NOT ahead of (s, id)
 template <typename Real>
@@ -459,27 +502,45 @@ __device__ __forceinline__ int partition_point(const Ctx<Real>& c, int b, int e,
     return lo;
 }
 
+// the same with three records per round, in flight together: half the rounds
+// for twice the loads, for kernels bound by the latency of a round
+template <typename Real>
+__device__ __forceinline__ int partition_point4(const Ctx<Real>& c, int b, int e, Real s, int id) {
+    int lo = b, hi = e;
+    while (lo < hi) {
+        const int len = hi - lo, q1 = lo + len / 4, q2 = lo + len / 2, q3 = lo + (int)(3u * (unsigned)len / 4u);
+        const RecA<Real> m1 = c.cur.a[q1], m2 = c.cur.a[q2], m3 = c.cur.a[q3];
+        const bool a1 = ahead(m1.s, m1.id, s, id), a2 = ahead(m2.s, m2.id, s, id), a3 = ahead(m3.s, m3.id, s, id);
+        if (!a1) hi = q1;
+        else if (!a2) { lo = q1 + 1; hi = q2; }
+        else if (!a3) { lo = q2 + 1; hi = q3; }
+        else lo = q3 + 1;
+    }
+    return lo;
+}
+
 template <typename Real>
 struct LaneAcc {
     Real a, gap, stop_gap;
     int has_leader, stop, overlap, nl;  // nl: the next lane from this lane on the route
 };
 
-// Ego acceleration on a lane (record li) at (s, v): min over the leader (the
-// vehicle at (ld_s, ld_v) in this lane if has_ld, else lookahead over at
-// most two lanes, R11) and the stop line (R12).  nl: next lane from this
-// lane on the ego's route (-1 none).
-template <typename Real, bool Groups = true>
-__device__ __forceinline__ LaneAcc<Real> accel_on_lane(const Ctx<Real>& c, const LaneInfo& li, Real s,
-                                                       Real v, Real v0, bool has_ld, Real ld_s, Real ld_v,
-                                                       int nl, int rptr, int rlast) {
+// Ego acceleration on a lane (record li) at (s, v), f its free term there:
+// min over the leader (the vehicle at (ld_s, ld_v) in this lane if has_ld,
+// else lookahead over at most two lanes, R11) and the stop line (R12).  nl:
+// next lane from this lane on the ego's route (-1 none).  The leader is found
+// first, in the lane or beyond it, and IDM evaluated once for both: a warp
+// nearly always holds both kinds.
+template <typename Real, bool Groups>
+__device__ __forceinline__ LaneAcc<Real> accel_on_lane(const Ctx<Real>& c, const LaneInfo& li, Real s, Real v, Real f,
+                                                       bool has_ld, Real ld_s, Real ld_v, int nl, int rptr,
+                                                       int rlast) {
     LaneAcc<Real> r;
     r.has_leader = 0; r.stop = 0; r.overlap = 0; r.gap = Real(0); r.stop_gap = Real(0); r.nl = nl;
-    Real a = idm_free(c, v, v0);
     if (has_ld) {
-        const Real gap = ld_s - c.len - s;
-        a = idm(c, v, v0, gap, v - ld_v);
-        r.has_leader = 1; r.gap = gap; r.overlap = gap < Real(0);
+        r.gap = ld_s - c.len - s;
+        r.has_leader = 1;
+        r.overlap = r.gap < Real(0);
     }
     if (nl >= 0) {
         const LaneInfo ni = c.lane[nl];
@@ -491,9 +552,9 @@ __device__ __forceinline__ LaneAcc<Real> accel_on_lane(const Ctx<Real>& c, const
                 const int b = c.cur.off[x], e = c.cur.off[x + 1];
                 if (e > b) {
                     const RecA<Real> R = c.cur.a[e - 1];  // rearmost vehicle of lane x
-                    const Real gap = base + R.s - c.len;
-                    a = idm(c, v, v0, gap, v - R.v);
-                    r.has_leader = 1; r.gap = gap;
+                    r.gap = base + R.s - c.len;
+                    ld_v = R.v;
+                    r.has_leader = 1;
                     break;
                 }
                 if (k == 1) break;
@@ -512,49 +573,37 @@ __device__ __forceinline__ LaneAcc<Real> accel_on_lane(const Ctx<Real>& c, const
         }
         // stop line: a red or amber junction lane ahead (R12), or a next lane
         // restricted from passing (R25)
-        if ((li.lo >= 0 && light_of(c, ni) != LIGHT_GREEN) || (ni.flags & LF_RESTRICTED)) {
-            const Real gs = Real(li.L) - s;
-            const Real as = idm(c, v, v0, gs, v);
-            if (as < a) a = as;
-            r.stop = 1; r.stop_gap = gs;
-        }
+        r.stop = (li.lo >= 0 && light_of(c, ni) != LIGHT_GREEN) || (ni.flags & LF_RESTRICTED);
+    } else if (Groups && li.lo >= 0 && rptr < rlast) {
+        // no junction lane from this road lane to the next road of the route
+        // (lane groups, R27): stop at the lane end as before a red light
+        r.stop = 1;
     }
-    // no junction lane from this road lane to the next road of the route
-    // (lane groups, R27): stop at the lane end as before a red light
-    if (Groups && nl < 0 && li.lo >= 0 && rptr < rlast) {
-        const Real gs = Real(li.L) - s;
-        const Real as = idm(c, v, v0, gs, v);
-        if (as < a) a = as;
-        r.stop = 1; r.stop_gap = gs;
+    r.a = c.a_max * f;
+    if (r.has_leader) r.a = idm(c, v, f, r.gap, v - ld_v);
+    if (r.stop) {
+        r.stop_gap = Real(li.L) - s;
+        const Real as = idm(c, v, f, r.stop_gap, v);
+        if (as < r.a) r.a = as;
     }
-    r.a = a;
     return r;
-}
-
-// in-lane acceleration of a follower F (desired-speed factor f_v0f, lane limit
-// vmax) towards a leader at (s_ld, v_ld), or on free road (politeness terms, R2)
-template <typename Real>
-__device__ __forceinline__ Real acc_pair(const Ctx<Real>& c, const RecA<Real>& F, float f_v0f, float vmax,
-                                         bool has_ld, Real s_ld, Real v_ld) {
-    const Real v0 = Real(f_v0f) * Real(vmax);
-    if (!has_ld) return idm_free(c, F.v, v0);
-    return idm(c, F.v, v0, s_ld - c.len - F.s, F.v - v_ld);
 }
 
 template <typename Real>
 struct Decision {
     LaneAcc<Real> own;
     Real u, scale;
-    int cand, dir, tl, TL, TF, flag;  // TL/TF: slots in the target lane or -1
-    int nlt;                          // next lane on the route from the target lane
-    int att;                          // MOBIL was evaluated (the attempt draw passed)
+    int cand, dir, tl, gp, flag;  // gp: insertion slot in the target lane
+    int nlt;                      // next lane on the route from the target lane
 };
 
 // The per-vehicle decision before conflict resolution (App. B.3), in two
 // parts.  decide_own: the acceleration on the own lane and, on a road with
-// two or more lanes, the MOBIL attempt draw (R4, R6).  decide_mobil: for a
-// vehicle whose attempt draw passed, the MOBIL utilities of the sides, p_LC
-// and the direction (R1-R5).  Both are pure functions of the snapshot.
+// two or more lanes, the MOBIL attempt draw (R4, R6).  Then, for a vehicle
+// whose attempt draw passed, MOBIL: the terms of the old follower
+// (mobil_old) and of each side (mobil_side), and the choice by p_LC and the
+// direction draw (mobil_choose; R1-R5).  All are pure functions of the
+// snapshot.
 template <typename Real>
 struct OwnPart {
     LaneAcc<Real> own;
@@ -572,104 +621,101 @@ __device__ __forceinline__ OwnPart<Real> decide_own(const Ctx<Real>& c, const Re
                                                     uint32_t k0, uint32_t k1, int vbase) {
     OwnPart<Real> P;
     P.att = 0; P.mand = 0; P.u_lc = 0.0f; P.u_dir = 0.0f;
-    P.own = accel_on_lane<Real, Groups>(c, li, E.s, E.v, Real(EB.v0f) * Real(li.vmax), OLr.lane == E.lane, OLr.s,
-                                        OLr.v, EB.nl, EB.rptr, EB.rlast);
+    P.own = accel_on_lane<Real, Groups>(c, li, E.s, E.v, free_term(E.v, Real(EB.v0f) * Real(li.vmax)),
+                                                OLr.lane == E.lane, OLr.s, OLr.v, EB.nl, EB.rptr, EB.rlast);
     if (li.lo < 0 || li.hi - li.lo < 2) return P;  // junction lane or single-lane road
     // no access to the next road from this lane: a mandatory change, no draw (R27)
     if (Groups && EB.nl < 0 && EB.rptr < EB.rlast) { P.mand = 1; return P; }
     uint32_t w[4];
     philox4x32_10(k0, k1, uint32_t(E.id - vbase), uint32_t(t), 0u, 0u, w);
-    const Real u_att = unit24<Real>(w[0]);
-    if (!(u_att < c.p_att)) return P;
+    if (!((w[0] >> 8) < c.att24)) return P;
     P.att = 1;
     P.u_lc = unit24<float>(w[1]);
     P.u_dir = unit24<float>(w[2]);
     return P;
 }
 
-template <typename Real, bool Groups = true>
-__device__ __forceinline__ Decision<Real> decide_mobil(const Ctx<Real>& c, const RecA<Real>& E, const RecB& EB,
-                                                       const LaneInfo& li, const RecA<Real>& OLr,
-                                                       const RecA<Real>& OFr, float of_v0f,
-                                                       const LaneAcc<Real>& own, float f_lc, float f_dir) {
-    Decision<Real> D;
-    D.cand = 0; D.dir = 0; D.tl = -1; D.TL = -1; D.TF = -1; D.flag = 0; D.nlt = -1; D.att = 1;
-    D.u = Real(0); D.scale = Real(1);
-    D.own = own;
-    const int lane = E.lane;
-    const Real v0f = Real(EB.v0f);
-    const Real u_lc = Real(f_lc), u_dir = Real(f_dir);
+// the old follower's acceleration now (a_old) and without the ego (at_old)
+// (politeness terms, R2); OLr, OFr: records of the ego's neighbour slots
+template <typename Real>
+__device__ __forceinline__ void mobil_old(const Ctx<Real>& c, const RecA<Real>& E, float vmax, const RecA<Real>& OLr,
+                                          const RecA<Real>& OFr, float of_v0f, Real* a_old, Real* at_old) {
+    *a_old = Real(0); *at_old = Real(0);
+    if (OFr.lane != E.lane) return;
+    const Real f = free_term(OFr.v, Real(of_v0f) * Real(vmax));
+    *a_old = idm(c, OFr.v, f, E.s - c.len - OFr.s, OFr.v - E.v);
+    *at_old = c.a_max * f;
+    if (OLr.lane == E.lane) *at_old = idm(c, OFr.v, f, OLr.s - c.len - OFr.s, OFr.v - OLr.v);
+}
 
-    Real a_old = Real(0), at_old = Real(0);
-    if (OFr.lane == lane) {
-        a_old = acc_pair(c, OFr, of_v0f, li.vmax, true, E.s, E.v);
-        if (OLr.lane == lane) {
-            at_old = acc_pair(c, OFr, of_v0f, li.vmax, true, OLr.s, OLr.v);
-        } else {
-            at_old = acc_pair(c, OFr, of_v0f, li.vmax, false, Real(0), Real(0));
-        }
+// One side (target lane tl) of a MOBIL evaluation.
+template <typename Real>
+struct SideTerms {
+    Real at_ego, at_new, a_new;  // the ego's acceleration there; the new follower's with and without it
+    int valid, feas, flag;       // it is a side; the safety conditions hold; an uncertain decision
+    int gp, nlt;                 // insertion slot; next lane on the route
+};
+
+// next_road: the next road of the route (-1: none)
+template <typename Real, bool Groups, bool Wide>
+__device__ __forceinline__ SideTerms<Real> mobil_side(const Ctx<Real>& c, const RecA<Real>& E, const RecB& EB, int jb,
+                                                      const LaneInfo& ti, int tl, int next_road) {
+    SideTerms<Real> S;
+    S.at_ego = Real(0); S.at_new = Real(0); S.a_new = Real(0);
+    S.valid = 0; S.feas = 0; S.flag = 0; S.gp = 0;
+    // next lane from the target lane; a lane without access to the next road
+    // is outside the vehicle's group: not a side (R27)
+    S.nlt = (next_road >= 0) ? jl_toward(c, ti, next_road, EB.nl - jb) : -1;
+    if (Groups && next_road >= 0 && S.nlt < 0) return S;
+    S.valid = 1;
+    const int tb = c.cur.off[tl], te = c.cur.off[tl + 1];
+    const int p = Wide ? partition_point4(c, tb, te, E.s, E.id) : partition_point(c, tb, te, E.s, E.id);
+    S.gp = p;
+    const bool lead = p > tb, fol = p < te;
+    int ok = 1;
+    const Real pos_scale = at_least_1(E.s);
+    RecA<Real> TLr, TFr;
+    TLr.s = Real(0); TLr.v = Real(0); TFr.s = Real(0); TFr.v = Real(0);
+    if (lead) {
+        TLr = c.cur.a[p - 1];
+        const Real g = TLr.s - c.len - E.s;
+        if (!gt(g, Real(0))) ok = 0;
+        if (within(g, c.band, pos_scale)) S.flag = 1;
     }
-    // next road of the route (for the target lane's junction lane)
-    const int next_road = (EB.nl >= 0) ? c.lane[EB.nl].road : -1;
-    // The sides that exist are visited in order, so every vehicle with one
-    // side (an edge lane) runs the first pass together with its warp
-    // neighbours, whichever side that is; results go to the left/right
-    // variables by select.  Same arithmetic per side as a fixed left/right
-    // loop: the decision does not depend on the visiting order.
-    Real u0 = Real(0), u1 = Real(0), scl0 = Real(0), scl1 = Real(0);
-    int feas0 = 0, feas1 = 0, TL0 = -1, TL1 = -1, TF0 = -1, TF1 = -1, NL0 = -1, NL1 = -1;
-    const Real pos_scale = E.s > Real(1) ? E.s : Real(1);
-    // a side is a lane of the road that is not restricted from passing (R25)
-    const int has_l = lane - 1 >= li.lo && !(c.lane[lane - 1].flags & LF_RESTRICTED);
-    const int has_r = lane + 1 < li.hi && !(c.lane[lane + 1].flags & LF_RESTRICTED);
-    const int n_sides = has_l + has_r;
-#pragma unroll 1
-    for (int k = 0; k < n_sides; ++k) {
-        const int side = (k == 0 && has_l) ? 0 : 1;
-        const int tl = side == 0 ? lane - 1 : lane + 1;
-        const LaneInfo ti = c.lane[tl];
-        // next lane from the target lane; a lane without access to the next
-        // road is outside the vehicle's group: not a side (R27)
-        const int nlt = (next_road >= 0) ? jl_toward(c, ti, next_road, EB.nl - li.jb) : -1;
-        if (Groups && next_road >= 0 && nlt < 0) continue;
-        const int tb = c.cur.off[tl], te = c.cur.off[tl + 1];
-        const int p = partition_point(c, tb, te, E.s, E.id);
-        const int TL = (p > tb) ? p - 1 : -1, TF = (p < te) ? p : -1;
-        int ok = 1;
-        RecA<Real> TLr, TFr;
-        TLr.s = Real(0); TLr.v = Real(0); TFr.s = Real(0); TFr.v = Real(0);
-        if (TL >= 0) {
-            TLr = c.cur.a[TL];
-            const Real g = TLr.s - c.len - E.s;
-            if (!(g > Real(0))) ok = 0;
-            if (rabs(g) < c.band * pos_scale) D.flag = 1;
-        }
-        if (TF >= 0) {
-            TFr = c.cur.a[TF];
-            const Real g = E.s - c.len - TFr.s;
-            if (!(g > Real(0))) ok = 0;
-            if (rabs(g) < c.band * pos_scale) D.flag = 1;
-        }
-        const Real at_ego =
-            accel_on_lane<Real, Groups>(c, ti, E.s, E.v, v0f * Real(ti.vmax), TL >= 0, TLr.s, TLr.v, nlt, EB.rptr,
-                                        EB.rlast).a;
-        Real a_new = Real(0), at_new = Real(0);
-        if (TF >= 0) {
-            const float fv0f = c.cur.b[TF].v0f;
-            a_new = acc_pair(c, TFr, fv0f, ti.vmax, TL >= 0, TLr.s, TLr.v);
-            at_new = acc_pair(c, TFr, fv0f, ti.vmax, true, E.s, E.v);
-            if (!(at_new >= -c.b_safe)) ok = 0;
-            const Real sc = rabs(at_new) > Real(1) ? rabs(at_new) : Real(1);
-            if (rabs(at_new + c.b_safe) < c.band * sc) D.flag = 1;
-        }
-        const Real us = (at_ego - D.own.a) + c.pol * ((at_new - a_new) + (at_old - a_old)) - c.a_th;
-        const Real ss = rabs(at_ego) + rabs(D.own.a) +
-                        c.pol * (rabs(at_new) + rabs(a_new) + rabs(at_old) + rabs(a_old)) + c.a_th;
-        if (side == 0) { u0 = us; scl0 = ss; feas0 = ok; TL0 = TL; TF0 = TF; NL0 = nlt; }
-        else           { u1 = us; scl1 = ss; feas1 = ok; TL1 = TL; TF1 = TF; NL1 = nlt; }
+    if (fol) {
+        TFr = c.cur.a[p];
+        const Real g = E.s - c.len - TFr.s;
+        if (!gt(g, Real(0))) ok = 0;
+        if (within(g, c.band, pos_scale)) S.flag = 1;
     }
-    const Real u[2] = {u0, u1}, scl[2] = {scl0, scl1};
-    const int feas[2] = {feas0, feas1}, TLs[2] = {TL0, TL1}, TFs[2] = {TF0, TF1}, NLs[2] = {NL0, NL1};
+    S.at_ego = accel_on_lane<Real, Groups>(c, ti, E.s, E.v, free_term(E.v, Real(EB.v0f) * Real(ti.vmax)), lead,
+                                                     TLr.s, TLr.v, S.nlt, EB.rptr, EB.rlast).a;
+    if (fol) {
+        const Real f = free_term(TFr.v, Real(c.cur.b[p].v0f) * Real(ti.vmax));
+        S.a_new = c.a_max * f;
+        if (lead) S.a_new = idm(c, TFr.v, f, TLr.s - c.len - TFr.s, TFr.v - TLr.v);
+        S.at_new = idm(c, TFr.v, f, E.s - c.len - TFr.s, TFr.v - E.v);
+        if (!(S.at_new >= -c.b_safe)) ok = 0;
+        if (within(S.at_new + c.b_safe, c.band, at_least_1(rabs(S.at_new)))) S.flag = 1;
+    }
+    S.feas = ok;
+    return S;
+}
+
+// utility of a side and its flag scale (R22)
+template <typename Real>
+__device__ __forceinline__ void side_utility(const Ctx<Real>& c, Real at_ego, Real at_new, Real a_new, Real own_a,
+                                             Real a_old, Real at_old, Real* u, Real* scl) {
+    *u = (at_ego - own_a) + c.pol * ((at_new - a_new) + (at_old - a_old)) - c.a_th;
+    *scl = rabs(at_ego) + rabs(own_a) + c.pol * (rabs(at_new) + rabs(a_new) + rabs(at_old) + rabs(a_old)) + c.a_th;
+}
+
+// The choice between the sides (0 left, 1 right) from their utilities: fills
+// u, scale, cand, dir and flag of D; returns the side (-1: none).
+template <typename Real>
+__device__ __forceinline__ int mobil_choose(const Ctx<Real>& c, const Real u[2], const Real scl[2], const int feas[2],
+                                            float f_lc, float f_dir, Decision<Real>& D) {
+    const Real u_lc = Real(f_lc), u_dir = Real(f_dir);
     Real scale = Real(1);
     for (int sd = 0; sd < 2; ++sd)
         if (feas[sd] && scl[sd] > scale) scale = scl[sd];
@@ -680,7 +726,7 @@ __device__ __forceinline__ Decision<Real> decide_mobil(const Ctx<Real>& c, const
     const Real pl = p_lc(c, uT);
     const Real band_p = (uT < Real(1) + c.band * scale) ? c.band * scale : c.band;
     if (rabs(u_lc - pl) < band_p) D.flag = 1;
-    if (!(u_lc < pl)) return D;
+    if (!(u_lc < pl)) return -1;
     int side = -1;
     if (uT > Real(0)) {
         const Real q = uLp - u_dir * uT;
@@ -693,12 +739,65 @@ __device__ __forceinline__ Decision<Real> decide_mobil(const Ctx<Real>& c, const
         else if (feas[1]) side = 1;
         if (side >= 0 && uT < c.band * scale) D.flag = 1;
     }
-    if (side < 0) return D;
+    if (side < 0) return -1;
     D.cand = 1;
     D.dir = side == 0 ? -1 : 1;
-    D.tl = side == 0 ? lane - 1 : lane + 1;
-    D.TL = TLs[side]; D.TF = TFs[side]; D.nlt = NLs[side];
     D.u = u[side];
+    return side;
+}
+
+template <typename Real>
+__device__ __forceinline__ Decision<Real> no_decision(const LaneAcc<Real>& own) {
+    Decision<Real> D;
+    D.cand = 0; D.dir = 0; D.tl = -1; D.gp = 0; D.flag = 0; D.nlt = -1;
+    D.u = Real(0); D.scale = Real(1);
+    D.own = own;
+    return D;
+}
+
+// MOBIL of one vehicle in one thread
+template <typename Real, bool Groups = true>
+__device__ __forceinline__ Decision<Real> decide_mobil(const Ctx<Real>& c, const RecA<Real>& E, const RecB& EB,
+                                                       const LaneInfo& li, const RecA<Real>& OLr,
+                                                       const RecA<Real>& OFr, float of_v0f,
+                                                       const LaneAcc<Real>& own, float f_lc, float f_dir) {
+    Decision<Real> D = no_decision(own);
+    const int lane = E.lane;
+    Real a_old, at_old;
+    mobil_old(c, E, li.vmax, OLr, OFr, of_v0f, &a_old, &at_old);
+    // next road of the route (for the target lane's junction lane)
+    const int next_road = (EB.nl >= 0) ? c.lane[EB.nl].road : -1;
+    // The sides that exist are visited in order, so every vehicle with one
+    // side (an edge lane) runs the first pass together with its warp
+    // neighbours, whichever side that is; results go to the left/right
+    // variables by select.  Same arithmetic per side as a fixed left/right
+    // loop: the decision does not depend on the visiting order.
+    Real u0 = Real(0), u1 = Real(0), scl0 = Real(0), scl1 = Real(0);
+    int feas0 = 0, feas1 = 0, GP0 = 0, GP1 = 0, NL0 = -1, NL1 = -1;
+    // a side is a lane of the road that is not restricted from passing (R25)
+    const int has_l = lane - 1 >= li.lo && !(c.lane[lane - 1].flags & LF_RESTRICTED);
+    const int has_r = lane + 1 < li.hi && !(c.lane[lane + 1].flags & LF_RESTRICTED);
+    const int n_sides = has_l + has_r;
+#pragma unroll 1
+    for (int k = 0; k < n_sides; ++k) {
+        const int side = (k == 0 && has_l) ? 0 : 1;
+        const int tl = side == 0 ? lane - 1 : lane + 1;
+        const LaneInfo ti = c.lane[tl];
+        const SideTerms<Real> S = mobil_side<Real, Groups, false>(c, E, EB, li.jb, ti, tl, next_road);
+        if (Groups && !S.valid) continue;
+        if (S.flag) D.flag = 1;
+        Real us, ss;
+        side_utility(c, S.at_ego, S.at_new, S.a_new, D.own.a, a_old, at_old, &us, &ss);
+        if (side == 0) { u0 = us; scl0 = ss; feas0 = S.feas; GP0 = S.gp; NL0 = S.nlt; }
+        else           { u1 = us; scl1 = ss; feas1 = S.feas; GP1 = S.gp; NL1 = S.nlt; }
+    }
+    const Real u[2] = {u0, u1}, scl[2] = {scl0, scl1};
+    const int feas[2] = {feas0, feas1};
+    const int side = mobil_choose(c, u, scl, feas, f_lc, f_dir, D);
+    if (side < 0) return D;
+    D.tl = side == 0 ? lane - 1 : lane + 1;
+    D.gp = side == 0 ? GP0 : GP1;
+    D.nlt = side == 0 ? NL0 : NL1;
     return D;
 }
 
@@ -712,10 +811,7 @@ template <typename Real>
 __device__ __forceinline__ Decision<Real> decide_mandatory(const Ctx<Real>& c, int i, const RecA<Real>& E,
                                                            const RecB& EB, const LaneInfo& li,
                                                            const LaneAcc<Real>& own) {
-    Decision<Real> D;
-    D.cand = 0; D.dir = 0; D.tl = -1; D.TL = -1; D.TF = -1; D.flag = 0; D.nlt = -1; D.att = 0;
-    D.u = Real(0); D.scale = Real(1);
-    D.own = own;
+    Decision<Real> D = no_decision(own);
     const int lane = E.lane;
     const int next_road = c.routes[EB.rptr + 1];
     int best = -1;
@@ -730,27 +826,26 @@ __device__ __forceinline__ Decision<Real> decide_mandatory(const Ctx<Real>& c, i
     if (ti.flags & LF_RESTRICTED) return D;
     const int tb = c.cur.off[tl], te = c.cur.off[tl + 1];
     const int p = partition_point(c, tb, te, E.s, E.id);
-    const int TL = (p > tb) ? p - 1 : -1, TF = (p < te) ? p : -1;
-    const Real pos_scale = E.s > Real(1) ? E.s : Real(1);
+    const Real pos_scale = at_least_1(E.s);
     int ok = 1;
-    if (TL >= 0) {
-        const RecA<Real> T = c.cur.a[TL];
+    if (p > tb) {
+        const RecA<Real> T = c.cur.a[p - 1];
         const Real g = T.s - c.len - E.s;
-        if (!(g > Real(0))) ok = 0;
-        if (rabs(g) < c.band * pos_scale) D.flag = 1;
+        if (!gt(g, Real(0))) ok = 0;
+        if (within(g, c.band, pos_scale)) D.flag = 1;
     }
-    if (TF >= 0) {
-        const RecA<Real> F = c.cur.a[TF];
+    if (p < te) {
+        const RecA<Real> F = c.cur.a[p];
         const Real g = E.s - c.len - F.s;
-        if (!(g > Real(0))) ok = 0;
-        if (rabs(g) < c.band * pos_scale) D.flag = 1;
-        const Real at_new = acc_pair(c, F, c.cur.b[TF].v0f, ti.vmax, true, E.s, E.v);
+        if (!gt(g, Real(0))) ok = 0;
+        if (within(g, c.band, pos_scale)) D.flag = 1;
+        const Real f = free_term(F.v, Real(c.cur.b[p].v0f) * Real(ti.vmax));
+        const Real at_new = idm(c, F.v, f, g, F.v - E.v);
         if (!(at_new >= -c.b_safe)) ok = 0;
-        const Real sc = rabs(at_new) > Real(1) ? rabs(at_new) : Real(1);
-        if (rabs(at_new + c.b_safe) < c.band * sc) D.flag = 1;
+        if (within(at_new + c.b_safe, c.band, at_least_1(rabs(at_new)))) D.flag = 1;
     }
     if (!ok) return D;
-    D.cand = 1; D.dir = dir; D.tl = tl; D.TL = TL; D.TF = TF;
+    D.cand = 1; D.dir = dir; D.tl = tl; D.gp = p;
     D.nlt = jl_toward(c, ti, next_road);
     D.u = Real(MAND_U);
     D.scale = Real(1);

@@ -1,6 +1,8 @@
 // Kernels of one simulation step (see moss_device.cuh for the layout).
 #pragma once
 
+#include <type_traits>
+
 #include "moss_device.cuh"
 
 namespace moss {
@@ -128,8 +130,8 @@ __device__ __forceinline__ int integrate_emit(const Ctx<Real>& c, MetricAcc& acc
         disp = -v * v / (Real(2) * a);
         vn = Real(0);
     }
-    if (la.has_leader) { const Real cl = la.gap > Real(0) ? la.gap : Real(0); if (disp > cl) disp = cl; }
-    if (la.stop) { const Real cl = la.stop_gap > Real(0) ? la.stop_gap : Real(0); if (disp > cl) disp = cl; }
+    if (la.has_leader) { const Real cl = gt(la.gap, Real(0)) ? la.gap : Real(0); if (gt(disp, cl)) disp = cl; }
+    if (la.stop) { const Real cl = gt(la.stop_gap, Real(0)) ? la.stop_gap : Real(0); if (gt(disp, cl)) disp = cl; }
     LaneInfo ni = c.lane[nlane];
     Real sn = s + disp;
     if (la.stop && sn > Real(ni.L)) sn = Real(ni.L);
@@ -144,9 +146,8 @@ __device__ __forceinline__ int integrate_emit(const Ctx<Real>& c, MetricAcc& acc
     if (!la.stop) {
         for (int iter = 0;;) {
             const Real Ll = Real(ni.L);
-            const Real scl = Ll > Real(1) ? Ll : Real(1);
             const bool road = ni.lo >= 0;
-            if (rabs(ex) < c.band * scl) fl |= F_FLAGGED;
+            if (within(ex, c.band, at_least_1(Ll))) fl |= F_FLAGGED;
             if (road && rptr == rlast) {
                 if (ex >= Real(0)) arrived = true;
                 break;
@@ -206,25 +207,29 @@ __device__ __forceinline__ int integrate_emit(const Ctx<Real>& c, MetricAcc& acc
     return 1;
 }
 
+// a candidate's kinematics on its target lane
+template <typename Real>
+__device__ __forceinline__ LaneAcc<Real> target_acc(const Ctx<Real>& c, const RecA<Real>& E, const RecB& EB,
+                                                    const Decision<Real>& D) {
+    const LaneInfo ti = c.lane[D.tl];
+    RecA<Real> TLr;
+    TLr.s = Real(0); TLr.v = Real(0);
+    const bool lead = D.gp > c.cur.off[D.tl];
+    if (lead) TLr = c.cur.a[D.gp - 1];
+    return accel_on_lane<Real, true>(c, ti, E.s, E.v, free_term(E.v, Real(EB.v0f) * Real(ti.vmax)), lead,
+                                               TLr.s, TLr.v, D.nlt, EB.rptr, EB.rlast);
+}
+
 // ---------------------------------------------------------------------------
 // A lane-change candidate leaves its decision for the end of the run: a record in the
 // candidate list, linked into the list of its target gap.
 template <typename Real>
 __device__ __forceinline__ void list_candidate(const Ctx<Real>& c, int i, const RecA<Real>& E, const RecB& EB,
                                                int sc, const Decision<Real>& D, int tag, CandLocal& cl) {
-    int gp;
-    if (D.TF >= 0) gp = D.TF;
-    else if (D.TL >= 0) gp = D.TL + 1;
-    else gp = c.cur.off[D.tl];
-    const LaneInfo ti = c.lane[D.tl];
-    RecA<Real> TLr;
-    TLr.s = Real(0); TLr.v = Real(0);
-    if (D.TL >= 0) TLr = c.cur.a[D.TL];
-    const LaneAcc<Real> T = accel_on_lane(c, ti, E.s, E.v, Real(EB.v0f) * Real(ti.vmax), D.TL >= 0, TLr.s, TLr.v,
-                                          D.nlt, EB.rptr, EB.rlast);
+    const LaneAcc<Real> T = target_acc(c, E, EB, D);
     Cand<Real> C;
     C.E = E; C.EB = EB;
-    C.slot = i; C.gap = gp + D.tl;
+    C.slot = i; C.gap = D.gp + D.tl;
     C.bits = (D.dir > 0 ? CB_RIGHT : 0) | (D.flag ? CB_FLAG : 0) | (D.own.has_leader ? CB_LEADER : 0) |
              (D.own.stop ? CB_STOP : 0) | (D.own.overlap ? CB_OVERLAP : 0) | (T.has_leader ? CB_TLEADER : 0) |
              (T.stop ? CB_TSTOP : 0) | (T.overlap ? CB_TOVERLAP : 0);
@@ -346,6 +351,169 @@ __device__ __forceinline__ void mobil_finish(const Ctx<Real>& c, const MobilQueu
 }
 
 // ---------------------------------------------------------------------------
+// The wide form of the decision, taken in FP64: a pass over up to TILE slots
+// in three phases of the whole block.  (1) Each vehicle: own lane and attempt
+// draw; those that go on enter one queue of the block.  (2) A thread for each
+// side of each queued vehicle and one for its old follower.  (3) A thread per
+// queued vehicle: the choice, the conflicts and the update.  A run whose
+// vehicles pass through the queue in one round settles its conflicts here, in
+// shared memory; longer runs leave their candidates for the end of the run.
+//
+// An FP64 instruction occupies an SM for 16 cycles whether one thread of the
+// warp is active or all are, so what counts is the number of warps that run
+// each part: against a queue per warp and one thread for the whole of a
+// vehicle's MOBIL, the vehicles of all warps are packed and the second side
+// costs only those that have one.  30x30 grid in FP64: k_decide 132 -> 62 us
+// a step.  In FP32, where latency or instruction issue bounds the kernel, the
+// exchange and the three barriers cost more than that saves (30x30 grid under
+// an agent's phases 32.0 -> 33.5 us a step, city 110 -> 165 us): the form above.
+template <typename Real>
+struct WideQueue {
+    Real a[TILE], gap[TILE], sgap[TILE];          // own-lane kinematics (LaneAcc)
+    Real a_old[TILE], at_old[TILE];               // mobil_old
+    Real t_ego[2 * TILE], t_new[2 * TILE], t_anew[2 * TILE];  // mobil_side of the left (2k) and right (2k + 1) side
+    Real cu[TILE], cscale[TILE];                  // candidates: utility, flag scale
+    int gp[2 * TILE], tnl[2 * TILE], tbits[2 * TILE];  // tbits: 1 valid, 2 feasible, 4 flag
+    int i[TILE], lane[TILE], bits[TILE], nl[TILE];     // bits: 1 leader, 2 stop, 4 overlap, 8 mandatory change
+    int ckey[TILE], cid[TILE];                    // candidates: gap key, id (right: ~id)
+    float u_lc[TILE], u_dir[TILE];
+    short item[2 * TILE];                         // sides to evaluate
+    int n, n_items;
+};
+
+// phase 1: vehicle i enters the queue
+template <typename Real>
+__device__ __forceinline__ void wide_push(WideQueue<Real>& q, int i, int lane, const LaneInfo& li,
+                                          const OwnPart<Real>& P) {
+    const int k = warp_claim(&q.n);
+    q.i[k] = i; q.lane[k] = lane;
+    q.a[k] = P.own.a; q.gap[k] = P.own.gap; q.sgap[k] = P.own.stop_gap;
+    q.bits[k] = (P.own.has_leader ? 1 : 0) | (P.own.stop ? 2 : 0) | (P.own.overlap ? 4 : 0) | (P.mand ? 8 : 0);
+    q.nl[k] = P.own.nl;
+    q.u_lc[k] = P.u_lc; q.u_dir[k] = P.u_dir;
+    q.tbits[2 * k] = 0; q.tbits[2 * k + 1] = 0;
+    if (P.mand) return;
+    if (lane - 1 >= li.lo) q.item[warp_claim(&q.n_items)] = (short)(2 * k);
+    if (lane + 1 < li.hi) q.item[warp_claim(&q.n_items)] = (short)(2 * k + 1);
+}
+
+// phase 2: side x & 1 of queued vehicle x >> 1
+template <typename Real, bool Groups>
+__device__ __forceinline__ void wide_side(const Ctx<Real>& c, WideQueue<Real>& q, int x) {
+    const int k = x >> 1, i = q.i[k], lane = q.lane[k], tl = lane + ((x & 1) ? 1 : -1);
+    const RecA<Real> E = c.cur.a[i];
+    const RecB EB = c.cur.b[i];
+    const LaneInfo ti = c.lane[tl];
+    // a side is a lane of the road that is not restricted from passing (R25)
+    if (ti.flags & LF_RESTRICTED) return;
+    const int next_road = EB.nl >= 0 ? c.lane[EB.nl].road : -1;
+    const SideTerms<Real> S = mobil_side<Real, Groups, true>(c, E, EB, c.lane[lane].jb, ti, tl, next_road);
+    q.t_ego[x] = S.at_ego; q.t_new[x] = S.at_new; q.t_anew[x] = S.a_new;
+    q.gp[x] = S.gp; q.tnl[x] = S.nlt;
+    q.tbits[x] = (S.valid ? 1 : 0) | (S.feas ? 2 : 0) | (S.flag ? 4 : 0);
+}
+
+// phase 2: the old follower of queued vehicle k
+template <typename Real>
+__device__ __forceinline__ void wide_old(const Ctx<Real>& c, WideQueue<Real>& q, int k, int n) {
+    if (q.bits[k] & 8) return;
+    const int i = q.i[k];
+    const RecA<Real> E = c.cur.a[i];
+    RecA<Real> OLr = no_rec<Real>(), OFr = no_rec<Real>();
+    float of_v0f = 0.0f;
+    if (i > 0) OLr = c.cur.a[i - 1];
+    if (i + 1 < n) {
+        OFr = c.cur.a[i + 1];
+        of_v0f = c.cur.b[i + 1].v0f;
+    }
+    Real a_old, at_old;
+    mobil_old(c, E, c.lane[q.lane[k]].vmax, OLr, OFr, of_v0f, &a_old, &at_old);
+    q.a_old[k] = a_old; q.at_old[k] = at_old;
+}
+
+// phase 3: queued vehicle k (k < 0: none; every thread of the block calls it)
+template <typename Real, bool Groups>
+__device__ __forceinline__ void wide_finish(const Ctx<Real>& c, WideQueue<Real>& q, int k, bool local, MetricAcc& acc,
+                                            int tag, CandLocal& cl) {
+    Decision<Real> D;
+    D.cand = 0; D.flag = 0;
+    RecA<Real> E;
+    RecB EB;
+    LaneAcc<Real> T;
+    int sc = 0, i = 0, lane = 0;
+    if (k >= 0) {
+        i = q.i[k]; lane = q.lane[k];
+        E = c.cur.a[i];
+        EB = c.cur.b[i];
+        const LaneInfo li = c.lane[lane];
+        sc = li.scen;
+        LaneAcc<Real> own;
+        const int bits = q.bits[k];
+        own.a = q.a[k]; own.gap = q.gap[k]; own.stop_gap = q.sgap[k]; own.nl = q.nl[k];
+        own.has_leader = bits & 1; own.stop = (bits >> 1) & 1; own.overlap = (bits >> 2) & 1;
+        if (sc != acc.scen) {
+            macc_flush_thread(acc, c.metrics);
+            macc_reset(acc, sc);
+        }
+        if (Groups && (bits & 8)) {
+            D = decide_mandatory(c, i, E, EB, li, own);
+        } else {
+            D = no_decision(own);
+            Real u[2] = {Real(0), Real(0)}, scl[2] = {Real(0), Real(0)};
+            int feas[2] = {0, 0};
+#pragma unroll
+            for (int sd = 0; sd < 2; ++sd) {
+                const int x = 2 * k + sd, tb = q.tbits[x];
+                if (!(tb & 1)) continue;
+                if (tb & 4) D.flag = 1;
+                feas[sd] = (tb >> 1) & 1;
+                side_utility(c, q.t_ego[x], q.t_new[x], q.t_anew[x], own.a, q.a_old[k], q.at_old[k], &u[sd], &scl[sd]);
+            }
+            const int sd = mobil_choose(c, u, scl, feas, q.u_lc[k], q.u_dir[k], D);
+            if (sd >= 0) {
+                D.tl = lane + (sd ? 1 : -1);
+                D.gp = q.gp[2 * k + sd];
+                D.nlt = q.tnl[2 * k + sd];
+            }
+        }
+        if (D.cand) {
+            if (local) {
+                cl.idx[atomicAdd(&cl.n, 1)] = k;
+                q.ckey[k] = D.gp + D.tl;
+                q.cid[k] = D.dir > 0 ? ~E.id : E.id;
+                q.cu[k] = D.u; q.cscale[k] = D.scale;
+                T = target_acc(c, E, EB, D);
+            } else {
+                list_candidate(c, i, E, EB, sc, D, tag, cl);
+            }
+        } else {
+            integrate_emit(c, acc, i, E, EB, own, lane, D.flag ? F_FLAGGED : 0, own.overlap != 0, c.scen_step[sc], sc,
+                           tag);
+        }
+    }
+    if (!local) return;
+    __syncthreads();
+    if (k < 0 || !D.cand) return;
+    // the conflict rule R9, as in resolve_one
+    int fl = F_CANDIDATE | (D.flag ? F_FLAGGED : 0);
+    bool granted = true;
+    const int key = D.gp + D.tl;
+    for (int j = 0; j < cl.n; ++j) {
+        const int r = cl.idx[j];
+        if (r == k || q.ckey[r] != key) continue;
+        const int rid = q.cid[r];
+        if ((rid < 0) == (D.dir > 0)) continue;  // same side: no conflict
+        const Real ru = q.cu[r], rs = q.cscale[r];
+        const Real sc2 = D.scale > rs ? D.scale : rs;
+        if (rabs(D.u - ru) < c.band * sc2) fl |= F_FLAGGED;
+        if (!(D.u > ru || (D.u == ru && E.id < (rid < 0 ? ~rid : rid)))) granted = false;
+    }
+    fl |= granted ? F_CHANGED : F_CONFLICT_LOST;
+    integrate_emit(c, acc, i, E, EB, granted ? T : D.own, granted ? D.tl : lane, fl, D.own.overlap != 0, c.scen_step[sc],
+                   sc, tag);
+}
+
+// ---------------------------------------------------------------------------
 // k_decide: blocks [0, n_work) take 256-slot tiles of the current snapshot
 // (one vehicle per thread); blocks [n_work, gridDim) run the insertion.
 // Per vehicle: the own-lane acceleration and the attempt draw, MOBIL if the
@@ -361,6 +529,8 @@ __device__ __forceinline__ void mobil_finish(const Ctx<Real>& c, const MobilQueu
 #ifndef MOSS_DECIDE_MIN_BLOCKS_FP64
 #define MOSS_DECIDE_MIN_BLOCKS_FP64 3
 #endif
+template <typename Real>
+__host__ __device__ constexpr bool wide_form() { return sizeof(Real) == 8; }
 template <typename Real>
 __host__ __device__ constexpr int decide_min_blocks() {
     return sizeof(Real) == 8 ? MOSS_DECIDE_MIN_BLOCKS_FP64 : MOSS_DECIDE_MIN_BLOCKS;
@@ -471,6 +641,7 @@ __device__ __forceinline__ void decide_run(const Ctx<Real>& c, int n, int n_work
 // (k_place advances those).
 template <typename Real, bool Groups>
 __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int vb, int nvb) {
+    constexpr bool Wide = wide_form<Real>();
     const int tag = c.cnt->tag;
     if (vb >= n_work) {
         const int stride = (nvb - n_work) * TILE;
@@ -486,7 +657,7 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
     // the run holds whole roads, so the block resolves its own lane-change
     // candidates once its run is done (rule R9: rivals share the road)
     __shared__ CandLocal cl;
-    __shared__ MobilQueue<Real> q;
+    __shared__ typename std::conditional<Wide, WideQueue<Real>, MobilQueue<Real>>::type q;
     __shared__ int s_road;  // road-lane vehicles of the run (for the run-weight fit)
     unsigned long long t_start = 0;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_start));
@@ -502,8 +673,15 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
     MetricAcc acc;
     macc_reset(acc, -1);
     const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31, qb = warp * 64;
-    if (wl == 0) q.n[warp] = 0;
-    __syncwarp();
+    if constexpr (Wide) {
+        if (threadIdx.x == 0) q.n = q.n_items = 0;
+        __syncthreads();
+    } else {
+        if (wl == 0) q.n[warp] = 0;
+        __syncwarp();
+    }
+    bool local = false;  // (wide) the run's conflicts were settled in its only round of the queue
+    int rounds = 0;
     for (int pass = 0;; ++pass) {
         const bool last = pass >= n_pass;
         const int i = base + pass * TILE + threadIdx.x;
@@ -542,7 +720,13 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
                         decide_own<Real, Groups>(c, E, EB, li, OLr, t, c.key0[sc], c.key1[sc], c.veh_base[sc]);
                     int fl = 0;
                     bool cand = false;
-                    if (P.att) {
+                    if constexpr (Wide) {
+                        if (P.att) acc.mob += 1;
+                        if (P.att || (Groups && P.mand)) {
+                            wide_push(q, i, lane, li, P);
+                            cand = true;  // finished from the queue
+                        }
+                    } else if (P.att) {
                         acc.mob += 1;
                         const int k = qb + warp_claim(&q.n[warp]);
                         q.i[k] = i; q.lane[k] = lane;
@@ -563,6 +747,29 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
                 }
             }
         }
+        if constexpr (Wide) {
+            if (last) break;
+            __syncthreads();
+            // phases 2 and 3 once the queue might not hold the next pass
+            const int nq = q.n, ni = q.n_items, ni32 = (ni + 31) & ~31;
+            const bool end = pass + 1 == n_pass;
+            if (!end && nq + min(TILE, s_end - (base + (pass + 1) * TILE)) <= TILE) {
+                __syncthreads();
+                continue;
+            }
+            local = end && rounds == 0;
+            ++rounds;
+            for (int x = threadIdx.x; x < ni32 + nq; x += TILE) {
+                if (x < ni) wide_side<Real, Groups>(c, q, q.item[x]);
+                else if (x >= ni32) wide_old(c, q, x - ni32, n);
+            }
+            __syncthreads();
+            wide_finish<Real, Groups>(c, q, (int)threadIdx.x < nq ? (int)threadIdx.x : -1, local, acc, tag, cl);
+            __syncthreads();
+            if (threadIdx.x == 0) q.n = q.n_items = 0;
+            __syncthreads();
+            continue;
+        } else {
         // MOBIL over the last 32 entries of the warp's queue once it holds
         // 32, and over what is left after the last pass
         __syncwarp();
@@ -575,10 +782,12 @@ __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int
             __syncwarp();
         }
         if (last) break;
+        }
     }
     // the run's lane-change candidates (their rivals are all in this run)
     __syncthreads();
-    for (int j = threadIdx.x; j < cl.n; j += TILE)
+    const int ncl = local ? 0 : cl.n;
+    for (int j = threadIdx.x; j < ncl; j += TILE)
         resolve_one(c, acc, j < c.cand_cap ? cl.idx[j] : c.cand_late[s_beg + j - c.cand_cap], c.n_veh, tag);
     if (n_road) atomicAdd(&s_road, n_road);
     macc_flush_block<TILE>(acc, c.metrics);  // (its barriers also complete s_road)
