@@ -19,7 +19,7 @@
 
 using namespace moss;
 
-constexpr int RB_WORDS = M_NFIELDS + 2;  // readback slot: metric record, step, error word
+constexpr int RB_WORDS = M_NFIELDS + 3;  // readback slot: metric record, step, error word, ticket
 
 // Getter outputs up to this size go through a pinned buffer of the handle and
 // a copy by the host: one wait in all, where a copy to pageable memory waits
@@ -145,7 +145,7 @@ struct MossHandle {
     // one moss_get_metrics
     long long* h_rb = nullptr;
     void* h_out = nullptr;               // pinned: outputs of the getters up to GETTER_PINNED bytes
-    cudaEvent_t rb_ev[MOSS_METRIC_SLOTS] = {};
+    long long rb_ticket[MOSS_METRIC_SLOTS + 1] = {};  // the slot's last readback (its kernel stores it after the rest)
     int rb_scen[MOSS_METRIC_SLOTS] = {};
     bool rb_pending[MOSS_METRIC_SLOTS] = {};
 
@@ -497,15 +497,15 @@ cudaError_t launch_coop(MossHandle* h, Ctx<Real>& c) {
                                        h->stream);
 }
 
-// one launch of a step kernel; chained: it may start while the kernel before
-// it in the stream drains (it calls grid_wait before it needs its results)
+// one launch; chained: it may start while the kernel before it in the stream
+// drains (it calls grid_wait before it needs its results)
 template <typename... P, typename... A>
-void launch_step_kernel(MossHandle* h, bool chained, int grid, size_t smem, void (*kernel)(P...), A... args) {
+void launch_chained(MossHandle* h, bool chained, int grid, int threads, size_t smem, void (*kernel)(P...), A... args) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(TILE); cfg.dynamicSmemBytes = smem; cfg.stream = h->stream;
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = h->stream;
     cfg.attrs = at; cfg.numAttrs = chained ? 1 : 0;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
     if (e != cudaSuccess) h->launch_err = e;
@@ -526,13 +526,13 @@ void enqueue_step(MossHandle* h, int cur, bool timed, bool first) {
             for (int q = 1; q <= N_STEP_KERNELS; ++q) cudaEventRecord(h->ev[q], s);
         return;
     }
-    launch_step_kernel(h, !first, g.decide_work + g.decide_ins, 0,
-                       h->lane_groups ? k_decide<Real, true> : k_decide<Real, false>, c, g.decide_work);
+    launch_chained(h, !first, g.decide_work + g.decide_ins, TILE, 0,
+                   h->lane_groups ? k_decide<Real, true> : k_decide<Real, false>, c, g.decide_work);
     if (timed) cudaEventRecord(h->ev[1], s);
-    if (g.scan) launch_step_kernel(h, !timed, g.scan, 0, k_lanescan<Real>, c);
+    if (g.scan) launch_chained(h, !timed, g.scan, TILE, 0, k_lanescan<Real>, c);
     if (timed) cudaEventRecord(h->ev[2], s);
-    if (g.scan) launch_step_kernel(h, !timed, g.place, 0, k_place_slots<Real>, c);
-    else launch_step_kernel(h, !timed, g.place, g.place_smem, k_place<Real>, c);
+    if (g.scan) launch_chained(h, !timed, g.place, TILE, 0, k_place_slots<Real>, c);
+    else launch_chained(h, !timed, g.place, TILE, g.place_smem, k_place<Real>, c);
     if (timed) cudaEventRecord(h->ev[3], s);
 }
 
@@ -881,8 +881,7 @@ int device_setup(MossHandle* h, void* stream) {
     CK(cudaHostAlloc((void**)&h->h_rb, sizeof(long long) * RB_WORDS * (MOSS_METRIC_SLOTS + 1),
                      cudaHostAllocDefault));
     CK(cudaHostAlloc(&h->h_out, GETTER_PINNED, cudaHostAllocDefault));
-    for (int k = 0; k < MOSS_METRIC_SLOTS; ++k)
-        CK(cudaEventCreateWithFlags(&h->rb_ev[k], cudaEventDisableTiming));
+    std::memset(h->h_rb, 0, sizeof(long long) * RB_WORDS * (MOSS_METRIC_SLOTS + 1));
     CK(cudaEventCreateWithFlags(&h->stage_free, cudaEventDisableTiming));
     CK(cudaEventRecord(h->stage_free, h->stream));
     CK(cudaEventCreateWithFlags(&h->load_free, cudaEventDisableTiming));
@@ -1215,19 +1214,42 @@ void free_all(MossHandle* h) {
     h->h_rb = nullptr;
     if (h->h_out) cudaFreeHost(h->h_out);
     h->h_out = nullptr;
-    for (int k = 0; k < MOSS_METRIC_SLOTS; ++k)
-        if (h->rb_ev[k]) cudaEventDestroy(h->rb_ev[k]);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     h->stream = nullptr;
 }
 
 // scenario s's metric record, its step and the device error word, as they are
-// behind the work queued so far, into readback slot `slot` (one launch that
-// stores to the pinned slot; three copies had cost 8.6 us of stream time)
+// behind the work queued so far, into readback slot `slot`: one launch that
+// stores to the pinned slot and, last, the slot's ticket.  The launches of
+// several readbacks overlap (they only wait for the work before them), and no
+// event stands between them (10 steps and the queues and metrics of 12 slots
+// 818 -> 776 us, 30 steps and the metrics of 64 scenarios 4224 -> 4157 us).
 int enqueue_readback(MossHandle* h, int s, int slot) {
-    k_readback<<<1, 32, 0, h->stream>>>(h->d_metrics + (size_t)s * M_NFIELDS, h->d_step + s, &h->d_cnt->err,
-                                        h->h_rb + (size_t)slot * RB_WORDS);
-    CK(cudaGetLastError());
+    const long long ticket = ++h->rb_ticket[slot];
+    h->launch_err = cudaSuccess;
+    launch_chained(h, true, 1, 32, 0, k_readback, (const long long*)(h->d_metrics + (size_t)s * M_NFIELDS),
+                   (const long long*)(h->d_step + s), (const int*)&h->d_cnt->err, h->h_rb + (size_t)slot * RB_WORDS,
+                   ticket);
+    if (h->launch_err != cudaSuccess) {
+        --h->rb_ticket[slot];
+        return cuda_fail(h, h->launch_err, "metric readback");
+    }
+    return MOSS_OK;
+}
+
+// waits until the slot's last readback has arrived; an error of the stream
+// ends the wait, and so does the end of its work
+int wait_readback(MossHandle* h, int slot) {
+    const long long* word = h->h_rb + (size_t)slot * RB_WORDS + M_NFIELDS + 2;
+    const long long ticket = h->rb_ticket[slot];
+    for (unsigned spins = 1; __atomic_load_n(word, __ATOMIC_ACQUIRE) != ticket; ++spins) {
+        if (spins % 4096) continue;
+        const cudaError_t e = cudaStreamQuery(h->stream);
+        if (e == cudaErrorNotReady) continue;
+        CK(e);
+        CK(cudaStreamSynchronize(h->stream));
+        if (__atomic_load_n(word, __ATOMIC_ACQUIRE) != ticket) return fail(h, MOSS_ECUDA, "a metric readback is missing");
+    }
     return MOSS_OK;
 }
 
@@ -1267,9 +1289,8 @@ int readback_metrics(MossHandle* h, int s, int slot, MossMetrics* out) {
 int scen_metrics(MossHandle* h, int s, MossMetrics* out) {
     if (!out) return fail(h, MOSS_EINVAL, "null output");
     if (s < 0 || s >= h->n_scen) return fail(h, MOSS_EINVAL, "scenario index out of range");
-    // one stream round trip: the copies go behind the queued work, one wait
     TRY(enqueue_readback(h, s, MOSS_METRIC_SLOTS));
-    CK(cudaStreamSynchronize(h->stream));
+    TRY(wait_readback(h, MOSS_METRIC_SLOTS));
     return readback_metrics(h, s, MOSS_METRIC_SLOTS, out);
 }
 
@@ -1835,9 +1856,8 @@ int moss_metrics_enqueue(moss_t h, int scenario, int slot) {
     if (scenario < 0 || scenario >= h->n_scen) return fail(h, MOSS_EINVAL, "scenario index out of range");
     if (slot < 0 || slot >= MOSS_METRIC_SLOTS) return fail(h, MOSS_EINVAL, "metric slot out of range");
     // a slot still in flight is waited for before its memory is reused
-    if (h->rb_pending[slot]) CK(cudaEventSynchronize(h->rb_ev[slot]));
+    if (h->rb_pending[slot]) TRY(wait_readback(h, slot));
     TRY(enqueue_readback(h, scenario, slot));
-    CK(cudaEventRecord(h->rb_ev[slot], h->stream));
     h->rb_pending[slot] = true;
     h->rb_scen[slot] = scenario;
     return MOSS_OK;
@@ -1848,7 +1868,7 @@ int moss_metrics_read(moss_t h, int slot, MossMetrics* out) {
     if (!out) return fail(h, MOSS_EINVAL, "null output");
     if (slot < 0 || slot >= MOSS_METRIC_SLOTS) return fail(h, MOSS_EINVAL, "metric slot out of range");
     if (!h->rb_pending[slot]) return fail(h, MOSS_EINVAL, "nothing enqueued in this metric slot");
-    CK(cudaEventSynchronize(h->rb_ev[slot]));
+    TRY(wait_readback(h, slot));
     h->rb_pending[slot] = false;
     return readback_metrics(h, h->rb_scen[slot], slot, out);
 }

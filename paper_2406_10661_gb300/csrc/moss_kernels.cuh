@@ -1588,12 +1588,22 @@ __global__ void k_road_speed(Ctx<Real> c, int r0, int r1, double* out, long long
     }
 }
 
-// metric record, step and error word of a scenario into pinned host memory
-__global__ void k_readback(const long long* metrics, const long long* step, const int* err, long long* out) {
+// metric record, step and error word of a scenario into pinned host memory,
+// then the ticket that the host waits for
+__global__ void k_readback(const long long* metrics, const long long* step, const int* err, long long* out,
+                           long long ticket) {
+    grid_wait();
+    grid_release();
     const int k = threadIdx.x;
     if (k < M_NFIELDS) out[k] = metrics[k];
     else if (k == M_NFIELDS) out[k] = *step;
     else if (k == M_NFIELDS + 1) *(int*)(out + k) = *err;
+    __threadfence_system();
+    __syncwarp();
+    if (k == 0) {
+        cuda::atomic_ref<long long, cuda::thread_scope_system> word(out[M_NFIELDS + 2]);
+        word.store(ticket, cuda::memory_order_release);
+    }
 }
 
 // The per-vehicle state of a scenario (vehicles [v0, v0 + nv)) by id, for the
