@@ -1559,17 +1559,26 @@ int scen_lane_metrics(MossHandle* h, int s, int32_t* queue, double* speed) {
     void* const to = nl > 0 ? (void*)queue : (void*)speed;
     const bool pinned = nb <= GETTER_PINNED;
     void* const buf = pinned ? h->h_out : h->d_mbuf;
+    // pinned outputs: the last block to finish stores the slot's ticket
+    Ticket tk = {nullptr, nullptr, 0};
+    if (pinned)
+        tk = {&h->d_cnt[0].out_done, h->h_rb + (size_t)MOSS_METRIC_SLOTS * RB_WORDS + M_NFIELDS + 2,
+              ++h->rb_ticket[MOSS_METRIC_SLOTS]};
     if (nl > 0) {
-        k_lane_queue<Real><<<(nl + 255) / 256, 256, 0, h->stream>>>(c, l0, l0 + nl, (int32_t*)buf, getter_err(h));
+        k_lane_queue<Real><<<(nl + 255) / 256, 256, 0, h->stream>>>(c, l0, l0 + nl, (int32_t*)buf, getter_err(h), tk);
     } else {
         const int per_block = 256 / ROAD_SPEED_THREADS;
         k_road_speed<Real><<<(nr + per_block - 1) / per_block, 256, 0, h->stream>>>(c, r0, r0 + nr, (double*)buf,
-                                                                                    getter_err(h));
+                                                                                    getter_err(h), tk);
     }
     CK(cudaGetLastError());
-    if (!pinned) CK(cudaMemcpyAsync(to, buf, nb, cudaMemcpyDeviceToHost, h->stream));
+    if (pinned) {
+        TRY(wait_readback(h, MOSS_METRIC_SLOTS));
+        std::memcpy(to, buf, nb);
+        return getter_status(h);
+    }
+    CK(cudaMemcpyAsync(to, buf, nb, cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
-    if (pinned) std::memcpy(to, buf, nb);
     return getter_status(h);
 }
 

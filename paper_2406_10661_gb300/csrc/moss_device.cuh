@@ -81,6 +81,7 @@ struct Counters {
     int err;         // device error bits (set 0 only)
     int n_mp;        // junctions under max pressure (set 0 only)
     int run_wq;      // fitted weight of a road-lane slot in k_decide's runs, x256 (0: none yet)
+    int out_done;    // blocks of a getter that have stored their outputs (set 0 only)
     int n_runs;      // k_decide work runs of this step (their statistics for the fit)
 };
 

@@ -1535,24 +1535,45 @@ __global__ void k_set_lane(Ctx<Real> c, int n, const int32_t* ids, const int32_t
     else li->flags = vals[k] ? (li->flags | LF_RESTRICTED) : (li->flags & ~LF_RESTRICTED);
 }
 
+// The end of a getter whose outputs lie in pinned host memory: the last block
+// to have stored its own stores the ticket that the host waits for.
+struct Ticket {
+    int* done;
+    long long* word;  // null: no ticket
+    long long value;
+};
+__device__ __forceinline__ void give_ticket(const Ticket& tk) {
+    if (!tk.word) return;
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(tk.done, 1) == (int)gridDim.x - 1) {
+        *tk.done = 0;
+        __threadfence_system();
+        cuda::atomic_ref<long long, cuda::thread_scope_system> word(*tk.word);
+        word.store(tk.value, cuda::memory_order_release);
+    }
+}
+
 // metrics of the current snapshot (R24): queue length of lanes [l0, l1) —
 // vehicles with v < 0.1 m/s within the last 50 m (the lane's segment is
 // ordered from its end, so the scan stops at the first vehicle farther away).
 // err_out (pinned host memory): the device error word, so that the getter
 // needs no copy of its own for it.
 template <typename Real>
-__global__ void k_lane_queue(Ctx<Real> c, int l0, int l1, int32_t* out, long long* err_out) {
+__global__ void k_lane_queue(Ctx<Real> c, int l0, int l1, int32_t* out, long long* err_out, Ticket tk) {
     const int l = l0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (l == l0) *(int*)err_out = *c.err;
-    if (l >= l1) return;
-    const double L = (double)c.lane[l].L;
-    int q = 0;
-    for (int k = c.cur.off[l]; k < c.cur.off[l + 1]; ++k) {
-        const RecA<Real> a = c.cur.a[k];
-        if (L - (double)a.s > 50.0) break;
-        if ((double)a.v < 0.1) ++q;
+    if (l < l1) {
+        const double L = (double)c.lane[l].L;
+        int q = 0;
+        for (int k = c.cur.off[l]; k < c.cur.off[l + 1]; ++k) {
+            const RecA<Real> a = c.cur.a[k];
+            if (L - (double)a.s > 50.0) break;
+            if ((double)a.v < 0.1) ++q;
+        }
+        out[l - l0] = q;
     }
-    out[l - l0] = q;
+    give_ticket(tk);
 }
 
 // average vehicle speed of roads [r0, r1) (R24): mean speed of the vehicles
@@ -1563,7 +1584,7 @@ __global__ void k_lane_queue(Ctx<Real> c, int l0, int l1, int32_t* out, long lon
 // 105 -> 69 us, on the grid's 3,480 62 -> 26 us, with its waits).
 constexpr int ROAD_SPEED_THREADS = 8;
 template <typename Real>
-__global__ void k_road_speed(Ctx<Real> c, int r0, int r1, double* out, long long* err_out) {
+__global__ void k_road_speed(Ctx<Real> c, int r0, int r1, double* out, long long* err_out, Ticket tk) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) *(int*)err_out = *c.err;
     const int r = r0 + t / ROAD_SPEED_THREADS, p = t % ROAD_SPEED_THREADS;
@@ -1578,14 +1599,16 @@ __global__ void k_road_speed(Ctx<Real> c, int r0, int r1, double* out, long long
     }
 #pragma unroll
     for (int o = ROAD_SPEED_THREADS / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (r >= r1 || p != 0) return;
-    if (cnt > 0) {
-        out[r - r0] = sum / (double)cnt;
-    } else {
-        double lim = 0.0;
-        for (int l = sp.x; l < sp.y; ++l) lim += (double)c.lane[l].vmax;
-        out[r - r0] = lim / (double)(sp.y - sp.x);
+    if (r < r1 && p == 0) {
+        if (cnt > 0) {
+            out[r - r0] = sum / (double)cnt;
+        } else {
+            double lim = 0.0;
+            for (int l = sp.x; l < sp.y; ++l) lim += (double)c.lane[l].vmax;
+            out[r - r0] = lim / (double)(sp.y - sp.x);
+        }
     }
+    give_ticket(tk);
 }
 
 // metric record, step and error word of a scenario into pinned host memory,
