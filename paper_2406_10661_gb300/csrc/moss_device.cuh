@@ -608,6 +608,7 @@ struct Decision {
 template <typename Real>
 struct OwnPart {
     LaneAcc<Real> own;
+    Real f;             // the ego's free term on its lane
     float u_lc, u_dir;  // the draws for p_LC and the direction (exact in FP32)
     int att;            // the attempt draw passed: MOBIL is evaluated
     int mand;           // outside the lane group of the next road: mandatory change (R27)
@@ -622,8 +623,8 @@ __device__ __forceinline__ OwnPart<Real> decide_own(const Ctx<Real>& c, const Re
                                                     uint32_t k0, uint32_t k1, int vbase) {
     OwnPart<Real> P;
     P.att = 0; P.mand = 0; P.u_lc = 0.0f; P.u_dir = 0.0f;
-    P.own = accel_on_lane<Real, Groups>(c, li, E.s, E.v, free_term(E.v, Real(EB.v0f) * Real(li.vmax)),
-                                                OLr.lane == E.lane, OLr.s, OLr.v, EB.nl, EB.rptr, EB.rlast);
+    P.f = free_term(E.v, Real(EB.v0f) * Real(li.vmax));
+    P.own = accel_on_lane<Real, Groups>(c, li, E.s, E.v, P.f, OLr.lane == E.lane, OLr.s, OLr.v, EB.nl, EB.rptr, EB.rlast);
     if (li.lo < 0 || li.hi - li.lo < 2) return P;  // junction lane or single-lane road
     // no access to the next road from this lane: a mandatory change, no draw (R27)
     if (Groups && EB.nl < 0 && EB.rptr < EB.rlast) { P.mand = 1; return P; }
@@ -657,10 +658,12 @@ struct SideTerms {
     int gp, nlt;                 // insertion slot; next lane on the route
 };
 
-// next_road: the next road of the route (-1: none)
+// next_road: the next road of the route (-1: none).  Wide: f_own is the ego's
+// free term on its lane, whose limit is vmax_own.
 template <typename Real, bool Groups, bool Wide>
 __device__ __forceinline__ SideTerms<Real> mobil_side(const Ctx<Real>& c, const RecA<Real>& E, const RecB& EB, int jb,
-                                                      const LaneInfo& ti, int tl, int next_road) {
+                                                      const LaneInfo& ti, int tl, int next_road,
+                                                      Real f_own = Real(0), float vmax_own = -1.0f) {
     SideTerms<Real> S;
     S.at_ego = Real(0); S.at_new = Real(0); S.a_new = Real(0);
     S.valid = 0; S.feas = 0; S.flag = 0; S.gp = 0;
@@ -689,8 +692,8 @@ __device__ __forceinline__ SideTerms<Real> mobil_side(const Ctx<Real>& c, const 
         if (!gt(g, Real(0))) ok = 0;
         if (within(g, c.band, pos_scale)) S.flag = 1;
     }
-    S.at_ego = accel_on_lane<Real, Groups>(c, ti, E.s, E.v, free_term(E.v, Real(EB.v0f) * Real(ti.vmax)), lead,
-                                                     TLr.s, TLr.v, S.nlt, EB.rptr, EB.rlast).a;
+    const Real f_ego = Wide && ti.vmax == vmax_own ? f_own : free_term(E.v, Real(EB.v0f) * Real(ti.vmax));
+    S.at_ego = accel_on_lane<Real, Groups>(c, ti, E.s, E.v, f_ego, lead, TLr.s, TLr.v, S.nlt, EB.rptr, EB.rlast).a;
     if (fol) {
         const Real f = free_term(TFr.v, Real(c.cur.b[p].v0f) * Real(ti.vmax));
         S.a_new = c.a_max * f;

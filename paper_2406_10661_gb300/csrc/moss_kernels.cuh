@@ -370,6 +370,7 @@ __device__ __forceinline__ void mobil_finish(const Ctx<Real>& c, const MobilQueu
 template <typename Real>
 struct WideQueue {
     Real a[TILE], gap[TILE], sgap[TILE];          // own-lane kinematics (LaneAcc)
+    Real f[TILE];                                 // the ego's free term on its lane
     Real a_old[TILE], at_old[TILE];               // mobil_old
     Real t_ego[2 * TILE], t_new[2 * TILE], t_anew[2 * TILE];  // mobil_side of the left (2k) and right (2k + 1) side
     Real cu[TILE], cscale[TILE];                  // candidates: utility, flag scale
@@ -389,6 +390,7 @@ __device__ __forceinline__ void wide_push(WideQueue<Real>& q, int i, int lane, c
     q.i[k] = i; q.lane[k] = lane;
     q.a[k] = P.own.a; q.gap[k] = P.own.gap; q.sgap[k] = P.own.stop_gap;
     q.bits[k] = (P.own.has_leader ? 1 : 0) | (P.own.stop ? 2 : 0) | (P.own.overlap ? 4 : 0) | (P.mand ? 8 : 0);
+    q.f[k] = P.f;
     q.nl[k] = P.own.nl;
     q.u_lc[k] = P.u_lc; q.u_dir[k] = P.u_dir;
     q.tbits[2 * k] = 0; q.tbits[2 * k + 1] = 0;
@@ -407,7 +409,8 @@ __device__ __forceinline__ void wide_side(const Ctx<Real>& c, WideQueue<Real>& q
     // a side is a lane of the road that is not restricted from passing (R25)
     if (ti.flags & LF_RESTRICTED) return;
     const int next_road = EB.nl >= 0 ? c.lane[EB.nl].road : -1;
-    const SideTerms<Real> S = mobil_side<Real, Groups, true>(c, E, EB, c.lane[lane].jb, ti, tl, next_road);
+    const LaneInfo li = c.lane[lane];
+    const SideTerms<Real> S = mobil_side<Real, Groups, true>(c, E, EB, li.jb, ti, tl, next_road, q.f[k], li.vmax);
     q.t_ego[x] = S.at_ego; q.t_new[x] = S.at_new; q.t_anew[x] = S.a_new;
     q.gp[x] = S.gp; q.tnl[x] = S.nlt;
     q.tbits[x] = (S.valid ? 1 : 0) | (S.feas ? 2 : 0) | (S.flag ? 4 : 0);
