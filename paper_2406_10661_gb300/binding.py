@@ -273,7 +273,7 @@ class _Handle:
         return int(out.value)
 
     def set_step_mode(self, mode: int) -> None:
-        """0: three kernels per step (graph); 1: one cooperative launch per step."""
+        """0: two or three kernels per step (graph); 1: one cooperative launch per step."""
         _check(self.lib.moss_set_step_mode(self.h, int(mode)), self.h)
 
     def set_kernel_timing(self, on: bool) -> None:

@@ -157,7 +157,7 @@ struct MossHandle {
     int cfg_ccap = 256;  // lane-change candidates a k_decide block lists in shared memory
 
     int parity = 0;  // snapshot buffer holding the current step
-    int step_mode = 0;               // 0: three kernels per step; 1: one cooperative launch
+    int step_mode = 0;               // 0: two or three kernels per step; 1: one cooperative launch
     unsigned* d_bar = nullptr;       // grid barrier of the cooperative step (count, generation)
     cudaError_t launch_err = cudaSuccess;
     cudaGraphExec_t graph[N_GRAPHS][2] = {};  // GRAPH_STEPS[k] steps from either parity
@@ -1221,13 +1221,14 @@ void free_all(MossHandle* h) {
 // scenario s's metric record, its step and the device error word, as they are
 // behind the work queued so far, into readback slot `slot`: one launch that
 // stores to the pinned slot and, last, the slot's ticket.  The launches of
-// several readbacks overlap (they only wait for the work before them), and no
-// event stands between them (10 steps and the queues and metrics of 12 slots
+// several readbacks overlap on the handle's own stream (on a caller's stream
+// the launch before may be the caller's, chained in its own way), and no event
+// stands between them (10 steps and the queues and metrics of 12 slots
 // 818 -> 776 us, 30 steps and the metrics of 64 scenarios 4224 -> 4157 us).
 int enqueue_readback(MossHandle* h, int s, int slot) {
     const long long ticket = ++h->rb_ticket[slot];
     h->launch_err = cudaSuccess;
-    launch_chained(h, true, 1, 32, 0, k_readback, (const long long*)(h->d_metrics + (size_t)s * M_NFIELDS),
+    launch_chained(h, h->own_stream, 1, 32, 0, k_readback, (const long long*)(h->d_metrics + (size_t)s * M_NFIELDS),
                    (const long long*)(h->d_step + s), (const int*)&h->d_cnt->err, h->h_rb + (size_t)slot * RB_WORDS,
                    ticket);
     if (h->launch_err != cudaSuccess) {

@@ -857,10 +857,6 @@ __device__ __forceinline__ Decision<Real> decide_mandatory(const Ctx<Real>& c, i
 }
 
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long load_acquire(unsigned long long* p) {
-    cuda::atomic_ref<unsigned long long, cuda::thread_scope_device> a(*p);
-    return a.load(cuda::memory_order_acquire);
-}
 // look-back words carry flag and value in one 64-bit word, so a relaxed
 // (single-copy atomic) load that sees the flag also sees the value
 __device__ __forceinline__ unsigned long long load_relaxed(unsigned long long* p) {
