@@ -501,8 +501,8 @@ int moss_set_schedule(moss_t h, const int* in7);
 
 /*
  * Failure-detection self-test (no counterpart in the paper).  Launches one
- * warp that runs the step's look-back wait (the decoupled scan of the lane
- * offsets) against a tile word that nothing ever publishes, so the bounded
+ * warp that runs the look-back wait of moss_lane_offsets_noalloc's scan
+ * against a tile word that nothing ever publishes, so the bounded
  * wait must give up after its iteration limit (about a second) instead of
  * hanging.  Uses a 64-byte device buffer it allocates and frees itself, on
  * cuda_stream (NULL = legacy default stream), and waits for the stream.
