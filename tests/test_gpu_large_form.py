@@ -1,0 +1,253 @@
+"""The step's kernels for large handles (the lane scan and the placement by
+slots), reached at small sizes: a handle takes that form by its number of
+trips, so trips that never depart within the test are added behind the others.
+A vehicle's results depend on its own id and on the vehicles near it only, so
+they have to be what the handle without the added trips gives (the placement
+by tiles), bit for bit, and what the FP64 oracle gives."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+import oracle
+from handmade import one_road
+from paper_2406_10661_gb300 import binding, scenario as sc
+
+pytestmark = pytest.mark.gpu
+
+ADDED = 200_001  # trips that reach the form by themselves
+NEVER = 1 << 30
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    binding.load()
+
+
+def _more(veh, lane=0):
+    """The trips and ADDED more on a lane (of road 0) that never depart."""
+    off = veh.route_off[-1] + 1 + np.arange(ADDED, dtype=np.int64)
+    return sc.Vehicles(n=veh.n + ADDED, route_off=np.concatenate([veh.route_off, off]).astype(np.int32),
+                       routes=np.concatenate([veh.routes, np.zeros(ADDED)]).astype(np.int32),
+                       start_lane=np.concatenate([veh.start_lane, np.full(ADDED, lane)]).astype(np.int32),
+                       dep=np.concatenate([veh.dep, np.full(ADDED, NEVER)]).astype(np.int32),
+                       v0f=np.concatenate([veh.v0f, np.ones(ADDED)]).astype(np.float32))
+
+
+def _large(scen):
+    return dataclasses.replace(scen, veh=_more(scen.veh))
+
+
+def _set(sim, st, n):
+    """The state with the vehicles past it (to n of them) waiting."""
+    k = n - len(st["status"])
+    rest = {"status": 0, "lane": -1, "s": 0, "v": 0, "rc": 0}
+    sim.set_state(*(np.concatenate([st[x], np.full(k, rest[x], st[x].dtype)]) for x in rest), 0)
+
+
+def _pair(scen, precision, st=None):
+    large = _large(scen)
+    a = binding.Simulation(scen.net, scen.veh, scen.params, precision=precision)
+    b = binding.Simulation(large.net, large.veh, large.params, precision=precision)
+    assert a.step_launches() == 2 and b.step_launches() == 3
+    if st is not None:
+        _set(a, st, scen.veh.n); _set(b, st, large.veh.n)
+    return a, b
+
+
+def _same_state(x, y, n):
+    for k in ("status", "lane", "rc", "s", "v", "flags"):
+        assert np.array_equal(x[k][:n], y[k][:n]), k
+
+
+def _same(a, b, n, waiting=ADDED):
+    _same_state(a.state(), b.state(), n)
+    am, bm = a.metrics(), b.metrics()
+    bm["n_waiting"] -= waiting
+    assert am == bm and am["errors"] == 0
+
+
+def _as_oracle(sim, ora, n):
+    g, r = sim.state(), ora.state()
+    act = r["status"] == 1
+    assert np.array_equal(g["status"][:n], r["status"]) and np.array_equal(g["flags"][:n], r["flags"])
+    for k in ("lane", "rc"):
+        assert np.array_equal(g[k][:n][act], r[k][act]), k
+    # FP64 on both sides: a step's rounding (1e-16 relative) grows by a few digits over the rollout
+    for k in ("s", "v"):
+        assert np.abs(g[k][:n][act] - r[k][act]).max(initial=0) < 1e-6, k
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("n,lanes", [(1, 1), (255, 1), (256, 1), (257, 1), (513, 2), (1800, 1), (2600, 2)])
+def test_long_segments(n, lanes, precision):
+    """Segments at the edges of a 256-slot tile and over many tiles, every
+    vehicle attempting lane changes."""
+    rng = np.random.RandomState(n)
+    length = 9.0 * -(-n // lanes) + 50.0
+    scen, st = one_road(lanes, length, [(k % lanes, length - 1.0 - 9.0 * (k // lanes) - rng.uniform(0, 0.3),
+                                         rng.uniform(0.0, 10.0), rng.uniform(0.8, 1.2)) for k in range(n)],
+                        params=sc.Params(seed=3, p_attempt=1.0))
+    if precision == 32:
+        st = {k: v.astype(np.float32).astype(v.dtype) for k, v in st.items()}
+    a, b = _pair(scen, precision, st)
+    ora = oracle.Oracle(scen.net, scen.veh, scen.params)
+    _set(ora, st, n)
+    for _ in range(3):
+        a.step(9); b.step(9); ora.step(9)
+        _same(a, b, n)
+        if precision == 64:
+            _as_oracle(b, ora, n)
+
+
+# lanes in all: 1023, 1024, 1025, 2047, 2048, 4094 .. 4099: the remainders of a 4-lane load and of a scan tile
+@pytest.mark.parametrize("n_lanes", [1, 1023, 1024, 1025, 2047, 2048, 4094, 4095, 4096, 4097, 4099, 8193])
+def test_lane_counts(n_lanes):
+    """A corridor of one-lane roads, with a second one to make up the number of
+    lanes, as a batch: transfers over the whole scan."""
+    parts = [n_lanes] if n_lanes % 2 else [n_lanes - 1, 1]
+    scens = []
+    for i, k in enumerate(parts):  # k lanes: (k + 1) / 2 roads, the others join them
+        roads = (k + 1) // 2
+        net = sc.corridor_network(1, (60.0,) * roads)
+        cars = np.arange(0, roads, 2)
+        veh = sc.Vehicles(n=len(cars), route_off=np.concatenate([[0], np.cumsum(roads - cars)]).astype(np.int32),
+                          routes=np.concatenate([np.arange(c, roads) for c in cars]).astype(np.int32),
+                          start_lane=cars.astype(np.int32), dep=(cars % 7).astype(np.int32),
+                          v0f=np.ones(len(cars), np.float32))
+        assert net.n_lanes == k
+        scens.append(sc.Scenario(net, veh, sc.Params(scenario=i), f"corridor{k}"))
+    a = binding.Batch(scens, precision=64)
+    b = binding.Batch([_large(scens[0]), *scens[1:]], precision=64)
+    assert b.step_launches() == 3
+    for _ in range(3):
+        a.step(13); b.step(13)
+        for i, s in enumerate(scens):
+            _same_state(a.state(i), b.state(i), s.veh.n)
+            am, bm = a.metrics(i), b.metrics(i)
+            bm["n_waiting"] -= ADDED if i == 0 else 0
+            assert am == bm and am["errors"] == 0
+    for i, s in enumerate(scens):
+        ora = oracle.Oracle(s.net, s.veh, s.params)
+        ora.step(39)
+        g, r = b.state(i), ora.state()
+        assert np.array_equal(g["status"][:s.veh.n], r["status"])
+        assert np.array_equal(g["lane"][:s.veh.n], r["lane"])
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("groups,p_attempt", [(False, 0.3), (True, 0.3), (True, 1.0)])
+def test_lane_changes_and_groups(groups, p_attempt, precision):
+    """Optional and mandatory changes: many entrants per lane."""
+    scen = sc.small_groups_scenario() if groups else sc.small_scenario()
+    scen.params.p_attempt = p_attempt
+    a, b = _pair(scen, precision)
+    ora = oracle.Oracle(scen.net, scen.veh, scen.params)
+    for _ in range(3):
+        a.step(90); b.step(90); ora.step(90)
+        _same(a, b, scen.veh.n)
+        if precision == 64:
+            _as_oracle(b, ora, scen.veh.n)
+    assert b.metrics()["lane_changes"] > 0
+
+
+def test_max_pressure_and_closures():
+    """Adaptive signals (their sums and their phases belong to two kernels of
+    the step) and lanes closed and slowed on the way."""
+    scen = sc.small_scenario()
+    a, b = _pair(scen, 64)
+    ora = oracle.Oracle(scen.net, scen.veh, scen.params)
+    J = np.arange(scen.net.n_junctions, dtype=np.int32)
+    for k in range(4):
+        for sim in (a, b):
+            if k == 1:
+                sim.set_signal_policy(J, binding.POLICY_MAX_PRESSURE)
+            if k == 2:
+                sim.set_lane_restriction([3, 8], [1, 1]); sim.set_lane_max_speed([5], [6.0])
+        if k == 1:
+            ora.set_signal(list(J), oracle.POLICY_MAX_PRESSURE)
+        a.step(70); b.step(70)
+        _same(a, b, scen.veh.n)
+        for x, y in zip(a.signal_state(J), b.signal_state(J)):
+            assert np.array_equal(x, y)
+        if k < 2:
+            ora.step(70)
+            _as_oracle(b, ora, scen.veh.n)
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_batch(precision):
+    """Uneven members, one without vehicles or junctions: each as alone."""
+    net = sc.corridor_network(2, (500.0,))
+    none = sc.Vehicles(n=0, route_off=np.zeros(1, np.int32), routes=np.zeros(0, np.int32),
+                       start_lane=np.zeros(0, np.int32), dep=np.zeros(0, np.int32), v0f=np.zeros(0, np.float32))
+    scens = [sc.small_scenario(seed=4), sc.Scenario(net, none, sc.Params(), "empty"), sc.small_groups_scenario(seed=5),
+             sc.small_scenario(seed=6)]
+    for i, s in enumerate(scens):
+        s.params.scenario = i
+    batch = binding.Batch([*scens[:3], _large(scens[3])], precision=precision)
+    assert batch.step_launches() == 3
+    for n in (1, 8, 141):
+        batch.step(n)
+    for i, s in enumerate(scens):
+        alone = binding.Simulation(s.net, s.veh, s.params, precision=precision)
+        assert alone.step_launches() == 2
+        alone.step(150)
+        _same_state(alone.state(), batch.state(i), s.veh.n)
+        am, bm = alone.metrics(), batch.metrics(i)
+        bm["n_waiting"] -= ADDED if i == 3 else 0
+        assert am == bm, i
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_slots_freeze_retire_and_reuse(precision):
+    """Slots whose capacity reaches the form: scenarios frozen at horizons
+    within and at the end of the steps launched together, retired and replaced
+    while others run."""
+    scens = [sc.small_scenario(seed=k + 1) for k in range(4)]
+    need = [binding.slot_caps(s) for s in scens]
+    caps = [{k: max(c[k] for c in need) for k in need[0]} for _ in range(2)]
+    caps[1]["n_vehicles"] = ADDED
+    slots = binding.Slots(caps, scens[0].params, precision=precision)
+    assert slots.step_launches() == 3
+
+    def check(slot, scen, steps):
+        alone = binding.Simulation(scen.net, scen.veh, scen.params, precision=precision)
+        assert alone.step_launches() == 2
+        alone.step(steps)
+        assert slots.metrics(slot) == alone.metrics()
+        _same_state(alone.state(), slots.state(slot), scen.veh.n)
+
+    slots.load(0, scens[0]); slots.set_horizon(0, 93)
+    slots.step(40)
+    slots.load(1, scens[1]); slots.set_horizon(1, 80)
+    slots.step(80)
+    check(0, scens[0], 93)
+    check(1, scens[1], 80)
+    slots.retire(0)
+    slots.step(1)
+    slots.load(0, scens[2])
+    slots.step(7)
+    slots.retire(1)
+    slots.step(1)
+    slots.load(1, scens[3])
+    slots.step(60)
+    check(0, scens[2], 68)
+    check(1, scens[3], 60)
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_single_launch(precision):
+    """The step as one cooperative launch, entered and left on the way."""
+    scen = sc.small_groups_scenario()
+    a, b = _pair(scen, precision)
+    a.step(121)
+    b.step(40)
+    b.set_step_mode(1)
+    b.step(41)
+    b.set_step_mode(0)
+    b.step(40)
+    _same(a, b, scen.veh.n)
