@@ -45,7 +45,7 @@ STEP_BYTES = 64.0      # whole step: read and write one 8x4 B state record per v
 
 PROFILES = os.path.join(ROOT, "profiles")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2406_10661_gb300", "csrc", f)
-                  for f in ("moss_device.cuh", "moss_kernels.cuh")]
+                  for f in ("moss_bits.h", "moss_device.cuh", "moss_kernels.cuh")]
 
 
 def kernel_source_hash() -> str:

@@ -27,7 +27,7 @@ def _stale(out, srcs):
 def build_cuda(force=False, extra=()):
     out = os.path.join(HERE, "libmoss.so")
     units = ("moss_api.cu", "moss_noalloc.cu")
-    srcs = [os.path.join(CSRC, f) for f in units + ("moss_device.cuh", "moss_kernels.cuh")]
+    srcs = [os.path.join(CSRC, f) for f in units + ("moss_bits.h", "moss_device.cuh", "moss_kernels.cuh")]
     srcs.append(os.path.join(ROOT, "include", "moss.h"))
     if force or _stale(out, srcs):
         tmp = out + f".{os.getpid()}.tmp"

@@ -36,6 +36,8 @@
 #include <cuda/atomic>
 #include <stdint.h>
 
+#include "moss_bits.h"
+
 namespace moss {
 
 enum : int { LIGHT_GREEN = 0, LIGHT_AMBER = 1, LIGHT_RED = 2 };
@@ -261,24 +263,19 @@ __device__ __forceinline__ double rabs(double x) { return fabs(x); }
 
 // An FP64 instruction takes an SM of this part 16 cycles per warp (two lanes a
 // cycle), an integer one a fraction of that, so in FP64 the comparisons that
-// decide nothing by rounding are made on the bit patterns: doubles >= 0 are
-// ordered like their bits.
+// decide nothing by rounding are made on the bit patterns (moss_bits.h).
 
 // x > t for t >= +0 (false for NaN)
 __device__ __forceinline__ bool gt(float x, float t) { return x > t; }
 __device__ __forceinline__ bool gt(double x, double t) {
-    const long long tb = __double_as_longlong(t);
-    return (unsigned long long)(__double_as_longlong(x) - tb - 1) < (unsigned long long)(0x7ff0000000000000ll - tb);
+    return bits_gt((unsigned long long)__double_as_longlong(x), (unsigned long long)__double_as_longlong(t));
 }
 
 // |x| < band * scale (an uncertain discrete decision, R22); in FP64 the
 // product is formed only when the exponents leave it open
 __device__ __forceinline__ bool within(float x, float band, float scale) { return rabs(x) < band * scale; }
 __device__ __forceinline__ bool within(double x, double band, double scale) {
-    // |x| >= 2^ex, band * scale <= 2^(eb + es + 2) (exponents biased by 1023)
-    const int ex = (__double2hiint(x) >> 20) & 0x7ff, eb = (__double2hiint(band) >> 20) & 0x7ff,
-              es = (__double2hiint(scale) >> 20) & 0x7ff;
-    if (ex + 1023 >= eb + es + 2) return false;
+    if (bits_not_within(__double2hiint(x), __double2hiint(band), __double2hiint(scale))) return false;
     return rabs(x) < band * scale;
 }
 // max(x, 1)
