@@ -393,6 +393,13 @@ int place_shift(const MossHandle* h, int lane_w, int lsr) {
 constexpr int FUSED_MAX_VEH = 200000;
 bool fused_place(const MossHandle* h) { return h->step_mode == 1 || h->n_veh <= FUSED_MAX_VEH; }
 
+// log2 of the lanes of a scan tile
+int scan_shift(const MossHandle* h) {
+    int shift = SCAN_ROUND_LOG2;
+    while (((h->n_lanes - 1) >> shift) + 1 > SCAN_MAX_TILES) ++shift;
+    return shift;
+}
+
 int place_tiles(const MossHandle* h, int lane_w, int lsr) {
     return (int)(place_weight(h, lane_w) >> place_shift(h, lane_w, lsr)) + 1;
 }
@@ -426,7 +433,7 @@ Ctx<Real> make_ctx(MossHandle* h, int cur) {
     c.ea = (RecA<Real>*)h->d_ea; c.eb = h->d_eb; c.enext = h->d_enext; c.head = h->d_head;
     c.enter = h->d_enter; c.leave = h->d_leave; c.tile_delta = h->d_delta[cur]; c.delta_nxt = h->d_delta[1 - cur];
     c.tile_cur = h->d_tiles[cur]; c.tile_nxt = h->d_tiles[1 - cur];
-    c.tile_shift = SCAN_TILE_LOG2; c.slot_w = 0; c.lane_w = 1;
+    c.tile_shift = scan_shift(h); c.slot_w = 0; c.lane_w = 1;
     if (fused_place(h)) {
         c.tile_shift = place_shift(h, h->cfg_lanescan, h->cfg_lsr); c.slot_w = 2; c.lane_w = h->cfg_lanescan;
     }
@@ -469,7 +476,7 @@ Grids grids(const MossHandle* h) {
     g.scan = 0;
     g.place = place_tiles(h, h->cfg_lanescan, h->cfg_lsr) + h->n_junc_chunks + 1;
     if (!fused_place(h)) {
-        g.scan = ((h->n_lanes - 1) >> SCAN_TILE_LOG2) + 1 + h->n_junc_chunks + 1;
+        g.scan = ((h->n_lanes - 1) >> scan_shift(h)) + 1 + h->n_junc_chunks + 1;
         g.place = std::min(2 * (h->n_veh / TILE + 1), h->sm_count * h->cfg_place);
     }
     g.place_smem = place_smem(place_lanes(place_shift(h, h->cfg_lanescan, h->cfg_lsr), h->cfg_lanescan));
@@ -529,7 +536,7 @@ void enqueue_step(MossHandle* h, int cur, bool timed, bool first) {
     launch_chained(h, !first, g.decide_work + g.decide_ins, TILE, 0,
                    h->lane_groups ? k_decide<Real, true> : k_decide<Real, false>, c, g.decide_work);
     if (timed) cudaEventRecord(h->ev[1], s);
-    if (g.scan) launch_chained(h, !timed, g.scan, TILE, 0, k_lanescan<Real>, c);
+    if (g.scan) launch_chained(h, !timed, g.scan, TILE, 0, k_lanescan<Real, SCAN_Q>, c);
     if (timed) cudaEventRecord(h->ev[2], s);
     if (g.scan) launch_chained(h, !timed, g.place, TILE, 0, k_place_slots<Real>, c);
     else launch_chained(h, !timed, g.place, TILE, g.place_smem, k_place<Real>, c);

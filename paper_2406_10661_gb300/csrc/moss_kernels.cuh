@@ -1229,94 +1229,158 @@ __global__ void __launch_bounds__(TILE, MOSS_PLACE_MIN_BLOCKS) k_place(Ctx<Real>
 // The form for large networks, where the work of a tile no longer hides behind
 // its latencies: the offsets in a kernel of their own (k_lanescan), then one
 // thread per slot and one warp per entrant, whatever their lanes
-// (k_place_slots).  Here a tile is SCAN_TILE consecutive lanes (tile_shift
-// counts lanes, slot_w is 0).
-constexpr int SCAN_TILE_LOG2 = 10;
-static_assert((1 << SCAN_TILE_LOG2) == 4 * TILE, "four lanes per thread");
+// (k_place_slots).  Here a tile is 1 << tile_shift consecutive lanes (slot_w
+// is 0): one round of SCAN_ROUND lanes, more rounds where the handle has so
+// many lanes that there would be more than SCAN_MAX_TILES tiles, each of
+// which adds up the growth of those before it.
+constexpr int SCAN_Q = 4;                          // a thread takes 4 consecutive lanes SCAN_Q times per round
+constexpr int SCAN_ROUND_LOG2 = 12;
+constexpr int SCAN_MAX_TILES = 1024;
+static_assert((1 << SCAN_ROUND_LOG2) == 4 * SCAN_Q * TILE, "the threads cover a round");
 
-// Lane tiles: newsize(l) = size(l) - leave(l) + enter(l), its prefix sum
-// within the tile, and the growth of the tiles before it (tile_delta).  Four
-// consecutive lanes per thread: the 16-byte loads and stores of a warp cover
-// 512 contiguous bytes.  Bound by one memory round trip behind k_decide: the
-// city's scan ends 5 to 7 us after it (with look-back the whole step took 146
-// us, so 141).
-template <typename Real>
-__global__ void __launch_bounds__(TILE) k_lanescan(Ctx<Real> c) {
-    const int tile = (int)blockIdx.x - c.n_junc_chunks - 1;
-    if (tile < 0) {
-        close_step<Real, true, false>(c, blockIdx.x);
-        return;
-    }
-    __shared__ int s_w[TW], s_g[TW];
+// One lane tile: newsize(l) = size(l) - leave(l) + enter(l), its prefix sum
+// within the tile, and the growth of the tiles before it (tile_delta).  A warp
+// takes 128 Q consecutive lanes of a round, 4 per thread and Q times, so that
+// its 16-byte accesses cover 512 contiguous bytes and all loads of a round are
+// in flight together.
+//
+// Bound by one memory round trip behind k_decide, by HBM (24 B a lane) for the
+// millions of lanes of a pool of slots.  The growth words are loaded before
+// the counts are cleared: loads issued behind the clearing stores wait for
+// them.  A pool of 1,673,184 lanes, 627,900 of them in use by 32 scenarios:
+// 12 us (40 MB), where tiles of 4 lanes per thread that cleared first took 37
+// and the scan with look-back 20; the same order with 4 / 8 lanes per thread:
+// 14 / 12, 16 lanes that clear first: 17.  The city's step 139.3 -> 136.2 us.
+template <typename Real, int Q, bool Pdl>
+__device__ __forceinline__ void scan_tile(const Ctx<Real>& c, int tile) {
+    constexpr int ROUND = 4 * TILE * Q;
+    __shared__ int s_w[2][TW], s_g[TW];
     const int ln = threadIdx.x & 31, w = threadIdx.x >> 5, nl = c.n_lanes;
-    const int l0 = (tile << SCAN_TILE_LOG2) + 4 * (int)threadIdx.x;
+    const int t0 = tile << c.tile_shift;
+    const int rounds = ((min(nl - t0, 1 << c.tile_shift)) + ROUND - 1) / ROUND;
     if (threadIdx.x == 0) c.delta_nxt[tile] = 0;  // (last read by the step before)
-    // offsets (written by the step before): o[4] is the end of the fourth lane
-    int o[5] = {0, 0, 0, 0, 0};
-    if (l0 + 4 <= nl) {
-        const int4 x = __ldcg(reinterpret_cast<const int4*>(c.cur.off + l0));
-        o[0] = x.x; o[1] = x.y; o[2] = x.z; o[3] = x.w;
-        o[4] = __ldcg(c.cur.off + l0 + 4);
-    } else {
+    // offsets (written by the step before): o[q][4] is the end of the fourth lane
+    int o[Q][5];
+    const auto load_offsets = [&](int r0) {
 #pragma unroll
-        for (int j = 0; j < 5; ++j)
-            if (l0 + j <= nl) o[j] = __ldcg(c.cur.off + l0 + j);
-    }
-    const int first = __ldcg(c.cur.off + (tile << SCAN_TILE_LOG2));
-    grid_wait();
-    grid_release();
-    if (*c.err & ERR_POISON) return;  // (set by a kernel that has ended)
-    int lv[4] = {0, 0, 0, 0}, en[4] = {0, 0, 0, 0};
-    if (l0 + 4 <= nl) {
-        const int4 x = *reinterpret_cast<const int4*>(c.leave + l0), y = *reinterpret_cast<const int4*>(c.enter + l0);
-        lv[0] = x.x; lv[1] = x.y; lv[2] = x.z; lv[3] = x.w;
-        en[0] = y.x; en[1] = y.y; en[2] = y.z; en[3] = y.w;
-        *reinterpret_cast<int4*>(c.leave + l0) = make_int4(0, 0, 0, 0);
-        *reinterpret_cast<int4*>(c.enter + l0) = make_int4(0, 0, 0, 0);
-    } else {
+        for (int q = 0; q < Q; ++q) {
+            const int l0 = r0 + 128 * q;
+            if (l0 + 4 <= nl) {
+                const int4 x = __ldcg(reinterpret_cast<const int4*>(c.cur.off + l0));
+                o[q][0] = x.x; o[q][1] = x.y; o[q][2] = x.z; o[q][3] = x.w;
+                o[q][4] = __ldcg(c.cur.off + l0 + 4);
+            } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (l0 + j < nl) {
-                lv[j] = c.leave[l0 + j]; en[j] = c.enter[l0 + j];
-                c.leave[l0 + j] = 0; c.enter[l0 + j] = 0;
+                for (int j = 0; j < 5; ++j) o[q][j] = l0 + j <= nl ? __ldcg(c.cur.off + l0 + j) : 0;
             }
+        }
+    };
+    int r0 = t0 + w * (128 * Q) + 4 * ln;  // the thread's first lane of the round
+    load_offsets(r0);
+    int at = __ldcg(c.cur.off + t0);  // next offset of the round's first lane
+    if (Pdl) {
+        grid_wait();
+        grid_release();
+        if (*c.err & ERR_POISON) return;  // (set by a kernel that has ended)
     }
     int grown = 0;
-    for (int p = threadIdx.x; p < tile; p += TILE) grown += c.tile_delta[p];
-    int ns[4], sum = 0;
+    for (int r = 0; r < rounds; ++r, r0 += ROUND) {
+        if (r) load_offsets(r0);
+        int lv[Q][4], en[Q][4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        ns[j] = l0 + j < nl ? o[j + 1] - o[j] - lv[j] + en[j] : 0;
-        sum += ns[j];
+        for (int q = 0; q < Q; ++q) {
+            const int l0 = r0 + 128 * q;
+            if (l0 + 4 <= nl) {
+                const int4 x = *reinterpret_cast<const int4*>(c.leave + l0), y = *reinterpret_cast<const int4*>(c.enter + l0);
+                lv[q][0] = x.x; lv[q][1] = x.y; lv[q][2] = x.z; lv[q][3] = x.w;
+                en[q][0] = y.x; en[q][1] = y.y; en[q][2] = y.z; en[q][3] = y.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    lv[q][j] = l0 + j < nl ? c.leave[l0 + j] : 0;
+                    en[q][j] = l0 + j < nl ? c.enter[l0 + j] : 0;
+                }
+            }
+        }
+        if (r == 0)
+            for (int p = threadIdx.x; p < tile; p += TILE) grown += c.tile_delta[p];
+        int pre[Q], run = 0;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int l0 = r0 + 128 * q;
+            int sum = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int ns = l0 + j < nl ? o[q][j + 1] - o[q][j] - lv[q][j] + en[q][j] : 0;
+                o[q][j] = ns;
+                sum += ns;
+            }
+            if (l0 + 4 <= nl) {
+                *reinterpret_cast<int4*>(c.leave + l0) = make_int4(0, 0, 0, 0);
+                *reinterpret_cast<int4*>(c.enter + l0) = make_int4(0, 0, 0, 0);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (l0 + j < nl) { c.leave[l0 + j] = 0; c.enter[l0 + j] = 0; }
+            }
+            int incl = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, d);
+                if (ln >= d) incl += y;
+            }
+            pre[q] = run + incl - sum;
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (r == 0) {
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) grown += __shfl_xor_sync(0xffffffffu, grown, d);
+            if (ln == 0) s_g[w] = grown;
+        }
+        if (ln == 0) s_w[r & 1][w] = run;
+        __syncthreads();
+        int wb = 0, total = 0;
+#pragma unroll
+        for (int k = 0; k < TW; ++k) {
+            const int x = s_w[r & 1][k];
+            if (k < w) wb += x;
+            total += x;
+            if (r == 0) at += s_g[k];
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int l0 = r0 + 128 * q;
+            int on[5];
+            on[0] = at + wb + pre[q];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) on[j + 1] = on[j] + o[q][j];
+            if (l0 + 4 <= nl) {
+                *reinterpret_cast<int4*>(c.nxt.off + l0) = make_int4(on[0], on[1], on[2], on[3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (l0 + j < nl) c.nxt.off[l0 + j] = on[j];
+            }
+            if (l0 < nl && nl <= l0 + 4) {  // this thread holds the last lane (on[] stays at the end past it)
+                c.nxt.off[nl] = on[4];
+                c.cnt_next->n_cur = on[4];
+            }
+        }
+        at += total;
     }
-    int incl = sum;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, d);
-        if (ln >= d) incl += y;
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) grown += __shfl_xor_sync(0xffffffffu, grown, d);
-    if (ln == 31) { s_w[w] = incl; s_g[w] = grown; }
-    __syncthreads();
-    int at = first + incl - sum;
-#pragma unroll
-    for (int k = 0; k < TW; ++k) at += s_g[k] + (k < w ? s_w[k] : 0);
-    int on[5];
-    on[0] = at;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) on[j + 1] = on[j] + ns[j];
-    if (l0 + 4 <= nl) {
-        *reinterpret_cast<int4*>(c.nxt.off + l0) = make_int4(on[0], on[1], on[2], on[3]);
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (l0 + j < nl) c.nxt.off[l0 + j] = on[j];
-    }
-    if (l0 < nl && nl <= l0 + 4) {  // this thread holds the last lane (on[] stays at the end past it)
-        c.nxt.off[nl] = on[4];
-        c.cnt_next->n_cur = on[4];
-    }
+}
+
+// Block vb of the scan: close_step's, then the lane tiles.
+template <typename Real, int Q, bool Pdl>
+__device__ __forceinline__ void scan_block(const Ctx<Real>& c, int vb) {
+    const int tile = vb - c.n_junc_chunks - 1;
+    if (tile < 0) close_step<Real, Pdl, false>(c, vb);
+    else scan_tile<Real, Q, Pdl>(c, tile);
+}
+
+template <typename Real, int Q>
+__global__ void __launch_bounds__(TILE) k_lanescan(Ctx<Real> c) {
+    scan_block<Real, Q, true>(c, blockIdx.x);
 }
 
 // The next snapshot.  Stayer tiles (one per block iteration): a vehicle that

@@ -251,3 +251,45 @@ def test_single_launch(precision):
     b.set_step_mode(0)
     b.step(40)
     _same(a, b, scen.veh.n)
+
+
+def test_scan_tiles_of_several_rounds():
+    """A member behind more lanes than the scan has tiles for in single rounds
+    (4,194,304): its offsets are carried over the rounds and the tiles."""
+    net = sc.corridor_network(100, (60.0,) * 21_600)
+    assert net.n_lanes > 4_194_304
+    veh = sc.Vehicles(n=1, route_off=np.array([0, 1], np.int32), routes=np.array([21_599], np.int32),
+                      start_lane=np.array([2_159_999], np.int32), dep=np.array([3], np.int32), v0f=np.ones(1, np.float32))
+    scens = [sc.Scenario(net, veh, sc.Params(), "long"), sc.small_groups_scenario()]
+    scens[1].params.scenario = 1
+    batch = binding.Batch([scens[0], _large(scens[1])], precision=64)
+    assert batch.step_launches() == 3
+    alone = binding.Simulation(scens[1].net, scens[1].veh, scens[1].params, precision=64)
+    for n in (5, 75):
+        batch.step(n); alone.step(n)
+        _same_state(alone.state(), batch.state(1), scens[1].veh.n)
+    assert batch.state(0)["status"][0] == 2 and batch.metrics(0)["errors"] == 0
+
+
+def test_scan_of_spare_lanes_is_bound_by_memory():
+    """The scan of a pool with 1.6 million lanes, most of them spare, from cold
+    caches: within three times its 24 bytes per lane at 6.8 TB/s, and 5 us for
+    the launch and the events."""
+    import torch
+    scen = sc.small_scenario()
+    caps = dict(binding.slot_caps(scen), n_lanes=1_600_000, n_vehicles=ADDED)
+    slots = binding.Slots([caps], scen.params)
+    slots.load(0, scen)
+    slots.step(60)
+    cold = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    us = []
+    for _ in range(20):
+        cold.add_(1)
+        torch.cuda.synchronize()
+        slots.set_kernel_timing(True)
+        slots.step(1)
+        slots.synchronize()
+        ms, steps = slots.kernel_times()
+        us.append(1e3 * ms["lanescan"] / steps)
+    slots.set_kernel_timing(False)
+    assert np.median(us) < 3 * 24 * 1.6e6 / 6.8e6 + 5, us
