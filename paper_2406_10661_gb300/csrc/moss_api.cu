@@ -391,7 +391,7 @@ int place_shift(const MossHandle* h, int lane_w, int lsr) {
 // grid, 45.7 / 45.0 at 350,000 in 12 slots, 55.6 / 46.9 at 500,009 in a
 // district, 170 / 142 in the city.
 constexpr int FUSED_MAX_VEH = 200000;
-bool fused_place(const MossHandle* h) { return h->step_mode == 1 || h->n_veh <= FUSED_MAX_VEH; }
+bool fused_place(const MossHandle* h) { return h->n_veh <= FUSED_MAX_VEH; }
 
 // log2 of the lanes of a scan tile
 int scan_shift(const MossHandle* h) {
@@ -488,7 +488,8 @@ Grids grids(const MossHandle* h) {
 template <typename Real, bool Groups>
 cudaError_t launch_coop(MossHandle* h, Ctx<Real>& c) {
     int per_sm = 0;
-    const size_t smem = grids(h).place_smem;
+    const Grids g = grids(h);
+    const size_t smem = g.scan ? 0 : g.place_smem;
     // (its static part and a wide tile's lanes pass 48 KB together in FP64)
     cudaError_t e = cudaFuncSetAttribute(k_step_coop<Real, Groups>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)place_smem(1 << PLACE_LANES_LOG2));
@@ -497,9 +498,9 @@ cudaError_t launch_coop(MossHandle* h, Ctx<Real>& c) {
     if (e != cudaSuccess) return e;
     int grid = std::max(1, per_sm) * h->sm_count;
     int n_work = std::max(1, std::min((h->n_veh + 31) / 32, grid));
-    int n_ins = extra_blocks(h), n_place = grids(h).place;
+    int n_ins = g.decide_ins, n_scan = g.scan, n_place = g.place;
     unsigned* bar = h->d_bar;
-    void* args[] = {(void*)&c, (void*)&n_work, (void*)&n_ins, (void*)&n_place, (void*)&bar};
+    void* args[] = {(void*)&c, (void*)&n_work, (void*)&n_ins, (void*)&n_scan, (void*)&n_place, (void*)&bar};
     return cudaLaunchCooperativeKernel((const void*)k_step_coop<Real, Groups>, grid, TILE, args, smem,
                                        h->stream);
 }

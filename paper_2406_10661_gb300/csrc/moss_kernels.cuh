@@ -1401,13 +1401,9 @@ __global__ void __launch_bounds__(TILE) k_lanescan(Ctx<Real> c) {
 // kept its lane goes to off'[lane] + (stayers ahead of it in the lane) +
 // (entrants ahead of it), its stayers ahead counted in its tile (below).
 // Then the entrants: rank = stayers ahead + entrants ahead.  Block 0 advances
-// the clocks, which k_lanescan reads and this kernel does not.
+// the clocks, which k_lanescan reads and this does not.
 template <typename Real>
-__global__ void __launch_bounds__(TILE) k_place_slots(Ctx<Real> c) {
-    const int vb = blockIdx.x, nvb = gridDim.x;
-    grid_wait();
-    grid_release();
-    if (__syncthreads_or(threadIdx.x == 0 ? *c.err & ERR_POISON : 0)) return;
+__device__ __forceinline__ void place_slots(const Ctx<Real>& c, int vb, int nvb) {
     if (vb == 0) advance_clocks(c);
     __shared__ int s_warp[TILE / 32];
     const int n = c.cnt->n_cur;
@@ -1523,6 +1519,14 @@ __global__ void __launch_bounds__(TILE) k_place_slots(Ctx<Real> c) {
     }
 }
 
+template <typename Real>
+__global__ void __launch_bounds__(TILE) k_place_slots(Ctx<Real> c) {
+    grid_wait();
+    grid_release();
+    if (__syncthreads_or(threadIdx.x == 0 ? *c.err & ERR_POISON : 0)) return;
+    place_slots(c, blockIdx.x, gridDim.x);
+}
+
 // tile cuts of the current snapshot's offsets (after creation, a state reset
 // or a change of the tile size; one thread per lane)
 template <typename Real>
@@ -1537,10 +1541,12 @@ __global__ void k_tile_cuts(Ctx<Real> c) {
 
 // ---------------------------------------------------------------------------
 // The whole step as one cooperative launch (every block resident at once):
-// the work of k_decide and k_place as two phases separated by a grid-wide
-// barrier.  A barrier is a count of arrived blocks and a
+// the work of the kernels of the handle's form as phases separated by
+// grid-wide barriers (n_scan > 0: k_decide, k_lanescan and k_place_slots; else
+// k_decide and k_place).  A barrier is a count of arrived blocks and a
 // generation word; a wait that exceeds SPIN_LIMIT sets ERR_TIMEOUT and every
-// block leaves the step.
+// block leaves the step.  The city as one launch takes 192 us a step with the
+// placement by tiles, 162 in its own form.
 __device__ __forceinline__ bool grid_sync(unsigned* bar, int* err) {
     __shared__ int s_ok;
     __syncthreads();
@@ -1570,12 +1576,20 @@ __device__ __forceinline__ bool grid_sync(unsigned* bar, int* err) {
 #endif
 template <typename Real, bool Groups>
 __global__ void __launch_bounds__(TILE, MOSS_COOP_MIN_BLOCKS) k_step_coop(Ctx<Real> c, int n_work, int n_ins,
-                                                                          int n_place, unsigned* bar) {
+                                                                          int n_scan, int n_place, unsigned* bar) {
     if (*c.err & ERR_POISON) return;
     // decide: n_work tile runs, then n_ins insertion blocks, as virtual blocks
     for (int vb = blockIdx.x; vb < n_work + n_ins; vb += gridDim.x)
         decide_block<Real, Groups>(c, n_work, vb, n_work + n_ins);
     if (!grid_sync(bar, c.err)) return;
+    if (n_scan) {
+        for (int vb = blockIdx.x; vb < n_scan; vb += gridDim.x) {
+            scan_block<Real, SCAN_Q, false>(c, vb);
+            __syncthreads();  // shared memory serves the next one
+        }
+        if (grid_sync(bar, c.err)) place_slots(c, blockIdx.x, gridDim.x);
+        return;
+    }
     for (int vb = blockIdx.x; vb < n_place; vb += gridDim.x) {
         place_block<Real, false>(c, vb);
         __syncthreads();  // shared memory serves the next one

@@ -5,6 +5,7 @@ A vehicle's results depend on its own id and on the vehicles near it only, so
 they have to be what the handle without the added trips gives (the placement
 by tiles), bit for bit, and what the FP64 oracle gives."""
 import dataclasses
+import time
 
 import numpy as np
 import pytest
@@ -336,3 +337,26 @@ def test_a_burst_of_lane_changes_counts_little():
     assert a.metrics()["lane_changes"] > 15 * n // 10  # (15 steps of at least n / 10)
     _same(a, b, n)
     assert us[n + ADDED] < 1.25 * us[n], us
+
+
+def test_single_launch_keeps_the_form():
+    """The step as one launch scans and places by slots in a large handle too:
+    2,464,950 vehicles on the road take at most 1.3 times the three kernels
+    (the barriers and the lower occupancy; by tiles 1.4 times and more)."""
+    scen, (status, lane, s, v, rc) = sc.saturated_city()
+    sim = binding.Simulation(scen.net, scen.veh, scen.params)
+    sim.set_state(status, lane, s, v, rc, 0)
+    sim.step(8)
+    us = {}
+    for mode in (0, 1):
+        sim.set_step_mode(mode)
+        sim.step(8)
+        x = []
+        for _ in range(7):
+            sim.synchronize()
+            t = time.perf_counter()
+            sim.step(16)
+            sim.synchronize()
+            x.append((time.perf_counter() - t) / 16e-6)
+        us[mode] = np.median(x)
+    assert us[1] < 1.3 * us[0], us
