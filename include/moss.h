@@ -474,23 +474,24 @@ int moss_step_launches(moss_t h, int* out);
  * depend on the schedule) under candidate schedules, keeps the fastest by
  * coordinate search over, in this order: k_decide blocks per SM {3,4,5}; the
  * weight of a road-lane vehicle in the split of the snapshot into k_decide's
- * block runs {0,1,2} (a junction-lane vehicle weighs 1; 0: the weight fitted each step); the weight
- * of a lane in the tiles of k_place {1,2,4} (a slot weighs 2); those tiles at
- * full or half size {16,8}; k_place_slots blocks per SM {4,8,16}; the step
- * mode {0,1} (moss_set_step_mode).  Then it re-captures the step graphs.
- * chosen3 (may be NULL) receives the chosen decide blocks per SM, lane weight
- * and place blocks per SM; moss_get_schedule returns the whole schedule.
+ * block runs {0,1,2} (a junction-lane vehicle weighs 1; 0: the weight fitted
+ * each step); k_lanescan blocks per SM {1,2,4}; lanes per thread of a round of
+ * the lane scan {16,8}; k_place_slots blocks per SM {4,8,16}; the step mode
+ * {0,1} (moss_set_step_mode).  Then it re-captures the step graphs.  chosen3
+ * (may be NULL) receives the chosen decide/lanescan/place blocks per SM;
+ * moss_get_schedule returns the whole schedule.
  */
 int moss_autotune(moss_t h, int trial_steps, int* chosen3);
 
 /*
- * The launch schedule (no counterpart in the paper): out7 / in7 = k_decide
- * blocks per SM, the weight of a lane in k_place's tiles, k_place_slots blocks
- * per SM, the road-lane weight of k_decide's runs (0: fitted each step from
- * the previous step's run times, the default; 1..8: fixed), k_place's tiles at
- * half or full size (8 or 16), the step mode (0 or 1), as moss_autotune
- * describes, and the number of lane-change candidates that a k_decide block
- * lists in shared memory (0..256, default 256; the others in global memory).
+ * The launch schedule (no counterpart in the paper): out7 / in7 = k_decide,
+ * k_lanescan and k_place_slots blocks per SM, the road-lane weight of
+ * k_decide's runs (0: fitted each step from the previous step's run times, the
+ * default; 1..8: fixed), lanes per thread of a round of the lane scan (8 or
+ * 16), the step mode (0 or 1), as moss_autotune describes, and the number of
+ * lane-change candidates that a k_decide block lists in shared memory (0..256,
+ * default 256; the others in global memory).  The second, third and fifth value
+ * act where a step has those two kernels (moss_step_launches 3).
  * moss_set_schedule checks the ranges (1..16 for k_decide's blocks, 1..32 for
  * the next two; weight 0..8), waits for the handle's stream and
  * re-captures the step graphs; on an error the previous schedule stays.

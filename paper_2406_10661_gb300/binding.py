@@ -290,6 +290,8 @@ class _Handle:
         return self.schedule()
 
     def schedule(self) -> Dict[str, int]:
+        """The launch schedule: blocks per SM of the kernels, ... (moss_get_schedule;
+        ``lanescan``, ``place`` and ``lanes_per_thread`` act in steps of three kernels)."""
         out = np.zeros(7, dtype=np.int32)
         _check(self.lib.moss_get_schedule(self.h, _ptr(out, ctypes.c_int32)), self.h)
         return dict(zip(self.SCHEDULE_KEYS, out.tolist()))

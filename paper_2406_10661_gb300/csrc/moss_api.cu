@@ -150,10 +150,9 @@ struct MossHandle {
     bool rb_pending[MOSS_METRIC_SLOTS] = {};
 
     // launch configuration (blocks per SM) of the step kernels; moss_autotune picks them
-    int cfg_decide = MOSS_DECIDE_MIN_BLOCKS, cfg_place = 8;
-    int cfg_lanescan = 4;  // weight of a lane in k_place's tiles, in half-slots
+    int cfg_decide = MOSS_DECIDE_MIN_BLOCKS, cfg_lanescan = 4, cfg_place = 8;
     int cfg_runw = 0;    // weight of a road-lane slot in k_decide's runs (0: fitted each step)
-    int cfg_lsr = 4;     // k_place tiles of the full (4) or half (2) size
+    int cfg_lsr = 4;     // lanes per thread of a round of k_lanescan, over 4 (4 or 2)
     int cfg_ccap = 256;  // lane-change candidates a k_decide block lists in shared memory
 
     int parity = 0;  // snapshot buffer holding the current step
@@ -373,17 +372,17 @@ size_t reca_size(int precision) { return precision == 64 ? sizeof(RecA<double>) 
 size_t sv_size(int precision) { return precision == 64 ? sizeof(SV<double>) : sizeof(SV<float>); }
 
 // Tiles of k_place for these sizes: 1 << shift half-slots (a slot weighs 2, a
-// lane lane_w).  At least one slot per thread; above that about 4.5 tiles per
-// SM at most (the 30x30 grid of 100,000 trips: 23.0 us per step with 355
-// tiles, 23.8 with 711 and 23.4 with 178); at most 2^PLACE_LANES_LOG2 lanes a
-// tile (its shared memory).
-long long place_weight(const MossHandle* h, int lane_w) { return 2ll * h->n_veh + (long long)lane_w * h->n_lanes; }
+// lane PLACE_LANE_W).  At least one slot per thread; above that about 4.5
+// tiles per SM at most (the 30x30 grid of 100,000 trips: 23.0 us per step with
+// 355 tiles, 23.8 with 711 and 23.4 with 178); at most 2^PLACE_LANES_LOG2 lanes
+// a tile (its shared memory).
+long long place_weight(const MossHandle* h) { return 2ll * h->n_veh + (long long)PLACE_LANE_W * h->n_lanes; }
 
-int place_shift(const MossHandle* h, int lane_w, int lsr) {
+int place_shift(const MossHandle* h) {
     int shift = 9;
-    while (2 * (place_weight(h, lane_w) >> shift) > 9ll * h->sm_count && (2 << shift) <= (lane_w << PLACE_LANES_LOG2))
+    while (2 * (place_weight(h) >> shift) > 9ll * h->sm_count && (2 << shift) <= (PLACE_LANE_W << PLACE_LANES_LOG2))
         ++shift;
-    return lsr == 2 ? shift - 1 : shift;
+    return shift;
 }
 
 // The placement as one kernel (k_place), or as k_lanescan and k_place_slots
@@ -393,15 +392,15 @@ int place_shift(const MossHandle* h, int lane_w, int lsr) {
 constexpr int FUSED_MAX_VEH = 200000;
 bool fused_place(const MossHandle* h) { return h->n_veh <= FUSED_MAX_VEH; }
 
+// lanes per thread of a round of the scan, over 4 (the single launch has the
+// default's)
+int scan_q(const MossHandle* h) { return h->step_mode == 1 ? SCAN_Q : h->cfg_lsr; }
+
 // log2 of the lanes of a scan tile
 int scan_shift(const MossHandle* h) {
-    int shift = SCAN_ROUND_LOG2;
+    int shift = scan_round_log2(scan_q(h));
     while (((h->n_lanes - 1) >> shift) + 1 > SCAN_MAX_TILES) ++shift;
     return shift;
-}
-
-int place_tiles(const MossHandle* h, int lane_w, int lsr) {
-    return (int)(place_weight(h, lane_w) >> place_shift(h, lane_w, lsr)) + 1;
 }
 
 template <typename Real>
@@ -435,7 +434,7 @@ Ctx<Real> make_ctx(MossHandle* h, int cur) {
     c.tile_cur = h->d_tiles[cur]; c.tile_nxt = h->d_tiles[1 - cur];
     c.tile_shift = scan_shift(h); c.slot_w = 0; c.lane_w = 1;
     if (fused_place(h)) {
-        c.tile_shift = place_shift(h, h->cfg_lanescan, h->cfg_lsr); c.slot_w = 2; c.lane_w = h->cfg_lanescan;
+        c.tile_shift = place_shift(h); c.slot_w = 2; c.lane_w = PLACE_LANE_W;
     }
     c.cand_late = h->d_cand_late;
     c.cands = (Cand<Real>*)h->d_cands; c.gap_head = h->d_gap_head;
@@ -474,12 +473,12 @@ Grids grids(const MossHandle* h) {
     g.decide_work = std::max(1, std::min((h->n_veh + 31) / 32, h->sm_count * std::min(h->cfg_decide, resident)));
     g.decide_ins = extra_blocks(h);
     g.scan = 0;
-    g.place = place_tiles(h, h->cfg_lanescan, h->cfg_lsr) + h->n_junc_chunks + 1;
+    g.place = (int)(place_weight(h) >> place_shift(h)) + 1 + h->n_junc_chunks + 1;
     if (!fused_place(h)) {
         g.scan = ((h->n_lanes - 1) >> scan_shift(h)) + 1 + h->n_junc_chunks + 1;
         g.place = std::min(2 * (h->n_veh / TILE + 1), h->sm_count * h->cfg_place);
     }
-    g.place_smem = place_smem(place_lanes(place_shift(h, h->cfg_lanescan, h->cfg_lsr), h->cfg_lanescan));
+    g.place_smem = place_smem(place_lanes(place_shift(h)));
     return g;
 }
 
@@ -537,7 +536,9 @@ void enqueue_step(MossHandle* h, int cur, bool timed, bool first) {
     launch_chained(h, !first, g.decide_work + g.decide_ins, TILE, 0,
                    h->lane_groups ? k_decide<Real, true> : k_decide<Real, false>, c, g.decide_work);
     if (timed) cudaEventRecord(h->ev[1], s);
-    if (g.scan) launch_chained(h, !timed, g.scan, TILE, 0, k_lanescan<Real, SCAN_Q>, c);
+    if (g.scan)
+        launch_chained(h, !timed, std::min(g.scan, h->sm_count * h->cfg_lanescan), TILE, 0,
+                       scan_q(h) == 2 ? k_lanescan<Real, 2> : k_lanescan<Real, SCAN_Q>, c, g.scan);
     if (timed) cudaEventRecord(h->ev[2], s);
     if (g.scan) launch_chained(h, !timed, g.place, TILE, 0, k_place_slots<Real>, c);
     else launch_chained(h, !timed, g.place, TILE, g.place_smem, k_place<Real>, c);
@@ -873,9 +874,8 @@ int device_setup(MossHandle* h, void* stream) {
     TRY(upload(h, &h->d_head, std::vector<unsigned long long>(NL, 0ull)));
     TRY(upload(h, &h->d_enter, std::vector<int32_t>(NL, 0)));
     TRY(upload(h, &h->d_leave, std::vector<int32_t>(NL, 0)));
-    // tiles under any schedule: place_shift leaves at most 2 x 4.5 per SM, or
-    // tiles of at least the weight of 2^(PLACE_LANES_LOG2 - 2) lanes
-    h->max_tiles = 10 * (size_t)h->sm_count + ((2 * (size_t)NV + NL) >> (PLACE_LANES_LOG2 - 2)) + 4;
+    // tiles under any schedule
+    h->max_tiles = std::max<size_t>(SCAN_MAX_TILES, (size_t)(place_weight(h) >> place_shift(h)) + 1);
     for (int k = 0; k < 2; ++k) {
         TRY(dalloc(h, &h->d_tiles[k], h->max_tiles + 1));
         TRY(dalloc(h, &h->d_delta[k], h->max_tiles));
@@ -2124,8 +2124,8 @@ int moss_autotune(moss_t h, int trial_steps, int* chosen3) {
     if (trial_steps < 1) return fail(h, MOSS_EINVAL, "trial_steps must be >= 1");
     CK(cudaStreamSynchronize(h->stream));
     // coordinate search over the schedule: blocks per SM of each kernel, the
-    // road-lane weight of k_decide's runs, the lane weight and size of
-    // k_place's tiles and the step mode; results do not depend on the schedule, only the time does
+    // road-lane weight of k_decide's runs, the lanes per thread of the scan and
+    // the step mode; results do not depend on the schedule, only the time does
     int coop = 0;
     CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
     struct Knob { int* v; int n; int c[3]; };

@@ -910,12 +910,13 @@ __device__ __forceinline__ int entrants_ahead(const Ctx<Real>& c, int q, Real s,
 constexpr int TW = TILE / 32;           // warps per block
 constexpr int PLACE_ROUNDS = 16;        // slot rounds whose leaver masks are held at a time
 constexpr int PLACE_LANES_LOG2 = 11;    // a tile holds at most 2^11 lanes
+constexpr int PLACE_LANE_W = 4;         // weight of a lane in the tiles, in half-slots
 // shared memory of a tile with up to `lanes` lanes: next offset (one more),
 // shift, entrants and their list per lane
 __host__ __device__ constexpr size_t place_smem(int lanes) { return sizeof(int) * (4 * (size_t)lanes + 1); }
-// lanes of the widest tile: each one adds at least lane_w
-__host__ __device__ constexpr int place_lanes(int tile_shift, int lane_w) {
-    return ((1 << tile_shift) + lane_w - 1) / lane_w;
+// lanes of the widest tile: each one adds at least PLACE_LANE_W
+__host__ __device__ constexpr int place_lanes(int tile_shift) {
+    return ((1 << tile_shift) + PLACE_LANE_W - 1) / PLACE_LANE_W;
 }
 
 // the clocks of every scenario, one step on (a frozen or retiring one stands
@@ -938,7 +939,7 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
     __shared__ int s_lp[PLACE_ROUNDS * TW];         // leavers of the tile before them
     __shared__ int s_sum[TW];
     __shared__ int s_nel;                           // lanes with entrants
-    const int cap = place_lanes(c.tile_shift, c.lane_w);
+    const int cap = place_lanes(c.tile_shift);
     int* const s_nx = s_lanes;            // [cap + 1] next offset of a lane
     int* const s_sh = s_lanes + cap + 1;  // [cap] next slot - slot of a lane's first vehicle, + leavers before the lane
     int* const s_hd = s_sh + cap;         // [cap] entrants of a lane: -1 none; >= 0 list; <= -2: one, ahead of the last
@@ -1244,13 +1245,15 @@ __global__ void __launch_bounds__(TILE, MOSS_PLACE_MIN_BLOCKS) k_place(Ctx<Real>
 // its latencies: the offsets in a kernel of their own (k_lanescan), then one
 // thread per slot and one warp per entrant, whatever their lanes
 // (k_place_slots).  Here a tile is 1 << tile_shift consecutive lanes (slot_w
-// is 0): one round of SCAN_ROUND lanes, more rounds where the handle has so
+// is 0): one round of 8 or 16 lanes per thread, more rounds where the handle has so
 // many lanes that there would be more than SCAN_MAX_TILES tiles, each of
 // which adds up the growth of those before it.
-constexpr int SCAN_Q = 4;                          // a thread takes 4 consecutive lanes SCAN_Q times per round
-constexpr int SCAN_ROUND_LOG2 = 12;
+constexpr int SCAN_Q = 4;  // a thread takes 4 consecutive lanes Q times per round: SCAN_Q, or 2 by schedule
 constexpr int SCAN_MAX_TILES = 1024;
-static_assert((1 << SCAN_ROUND_LOG2) == 4 * SCAN_Q * TILE, "the threads cover a round");
+// log2 of the lanes of a round
+__host__ __device__ constexpr int scan_round_log2(int q) { return q == 4 ? 12 : 11; }
+static_assert((1 << scan_round_log2(4)) == 16 * TILE && (1 << scan_round_log2(2)) == 8 * TILE,
+              "the threads cover a round");
 
 // One lane tile: newsize(l) = size(l) - leave(l) + enter(l), its prefix sum
 // within the tile, and the growth of the tiles before it (tile_delta).  A warp
@@ -1267,7 +1270,7 @@ static_assert((1 << SCAN_ROUND_LOG2) == 4 * SCAN_Q * TILE, "the threads cover a 
 // 14 / 12, 16 lanes that clear first: 17.  The city's step 139.3 -> 136.2 us.
 template <typename Real, int Q, bool Pdl>
 __device__ __forceinline__ void scan_tile(const Ctx<Real>& c, int tile) {
-    constexpr int ROUND = 4 * TILE * Q;
+    constexpr int ROUND = 1 << scan_round_log2(Q);
     __shared__ int s_w[2][TW], s_g[TW];
     const int ln = threadIdx.x & 31, w = threadIdx.x >> 5, nl = c.n_lanes;
     const int t0 = tile << c.tile_shift;
@@ -1384,7 +1387,7 @@ __device__ __forceinline__ void scan_tile(const Ctx<Real>& c, int tile) {
     }
 }
 
-// Block vb of the scan: close_step's, then the lane tiles.
+// Virtual block vb of the scan: close_step's, then the lane tiles.
 template <typename Real, int Q, bool Pdl>
 __device__ __forceinline__ void scan_block(const Ctx<Real>& c, int vb) {
     const int tile = vb - c.n_junc_chunks - 1;
@@ -1393,8 +1396,11 @@ __device__ __forceinline__ void scan_block(const Ctx<Real>& c, int vb) {
 }
 
 template <typename Real, int Q>
-__global__ void __launch_bounds__(TILE) k_lanescan(Ctx<Real> c) {
-    scan_block<Real, Q, true>(c, blockIdx.x);
+__global__ void __launch_bounds__(TILE) k_lanescan(Ctx<Real> c, int n_scan) {
+    for (int vb = blockIdx.x; vb < n_scan; vb += gridDim.x) {
+        scan_block<Real, Q, true>(c, vb);
+        __syncthreads();  // shared memory serves the next one
+    }
 }
 
 // The next snapshot.  Stayer tiles (one per block iteration): a vehicle that

@@ -360,3 +360,31 @@ def test_single_launch_keeps_the_form():
             x.append((time.perf_counter() - t) / 16e-6)
         us[mode] = np.median(x)
     assert us[1] < 1.3 * us[0], us
+
+
+@pytest.mark.parametrize("lanescan,lanes_per_thread", [(1, 8), (1, 16), (32, 8), (32, 16)])
+@pytest.mark.parametrize("roads", [1023, 1025, 4097, 160_000])
+def test_scan_schedules(roads, lanescan, lanes_per_thread):
+    """The scan's blocks per SM and lanes per thread, as documented: every
+    choice gives the same result, with fewer blocks than tiles too, and from
+    one step to the next."""
+    net = sc.corridor_network(1, (60.0,) * roads)
+    at = np.linspace(0, roads - 1, 500).astype(np.int64)
+    veh = sc.Vehicles(n=500, route_off=np.concatenate([[0], np.cumsum(np.minimum(roads - at, 9))]).astype(np.int32),
+                      routes=np.concatenate([np.arange(x, min(x + 9, roads)) for x in at]).astype(np.int32),
+                      start_lane=at.astype(np.int32), dep=(np.arange(500) % 5).astype(np.int32),
+                      v0f=np.ones(500, np.float32))
+    a = binding.Simulation(net, _more(veh), sc.Params())
+    b = binding.Simulation(net, _more(veh), sc.Params())
+    assert b.step_launches() == 3
+    a.step(33)
+    b.step(7)
+    default = b.schedule()
+    sched = dict(default, lanescan=lanescan, lanes_per_thread=lanes_per_thread)
+    b.set_schedule(**sched)
+    assert b.schedule() == sched
+    b.step(17)
+    b.set_schedule(**default)
+    b.step(9)
+    _same(a, b, 500, waiting=0)
+    assert a.metrics()["n_arrived"] + a.metrics()["n_active"] == 500
