@@ -371,26 +371,17 @@ bool same_model(const MossParams& a, const MossParams& b) {
 size_t reca_size(int precision) { return precision == 64 ? sizeof(RecA<double>) : sizeof(RecA<float>); }
 size_t sv_size(int precision) { return precision == 64 ? sizeof(SV<double>) : sizeof(SV<float>); }
 
-// Tiles of k_place for these sizes: 1 << shift half-slots (a slot weighs 2, a
-// lane PLACE_LANE_W).  At least one slot per thread; above that about 4.5
-// tiles per SM at most (the 30x30 grid of 100,000 trips: 23.0 us per step with
-// 355 tiles, 23.8 with 711 and 23.4 with 178); at most 2^PLACE_LANES_LOG2 lanes
-// a tile (its shared memory).
-long long place_weight(const MossHandle* h) { return 2ll * h->n_veh + (long long)PLACE_LANE_W * h->n_lanes; }
-
-int place_shift(const MossHandle* h) {
-    int shift = 9;
-    while (2 * (place_weight(h) >> shift) > 9ll * h->sm_count && (2 << shift) <= (PLACE_LANE_W << PLACE_LANES_LOG2))
-        ++shift;
-    return shift;
-}
-
 // The placement as one kernel (k_place), or as k_lanescan and k_place_slots
-// for large networks: us per step 23.2 / 24.7 at 100,000 trips on the 30x30
-// grid, 45.7 / 45.0 at 350,000 in 12 slots, 55.6 / 46.9 at 500,009 in a
-// district, 170 / 142 in the city.
-constexpr int FUSED_MAX_VEH = 200000;
-bool fused_place(const MossHandle* h) { return h->n_veh <= FUSED_MAX_VEH; }
+// for handles of more weight (half-slots: a vehicle 2, a lane PLACE_LANE_W).
+// us per step, one kernel / two, trips and lanes:
+//   36,000 on 14,064:  23.6 / 25.1     75,000 on  30,288: 27.4 / 26.3
+//   50,000 on 19,428:  24.8 / 25.0    100,000 on  40,704: 27.9 / 27.1
+//   20,000 on 40,704:  22.8 / 24.1     50,000 on  72,660: 27.0 / 26.3
+//    4,000 on  2,424:  18.9 / 21.1     20,000 on 361,802: 25.4 / 24.7
+// (FP64 alike: 38.0 / 38.8 at 36,000 trips, 57.0 / 55.7 at 100,000).
+constexpr long long PLACE_MAX_WEIGHT = 240000;
+long long place_weight(const MossHandle* h) { return 2ll * h->n_veh + (long long)PLACE_LANE_W * h->n_lanes; }
+bool fused_place(const MossHandle* h) { return place_weight(h) <= PLACE_MAX_WEIGHT; }
 
 // lanes per thread of a round of the scan, over 4 (the single launch has the
 // default's)
@@ -434,7 +425,7 @@ Ctx<Real> make_ctx(MossHandle* h, int cur) {
     c.tile_cur = h->d_tiles[cur]; c.tile_nxt = h->d_tiles[1 - cur];
     c.tile_shift = scan_shift(h); c.slot_w = 0; c.lane_w = 1;
     if (fused_place(h)) {
-        c.tile_shift = place_shift(h); c.slot_w = 2; c.lane_w = PLACE_LANE_W;
+        c.tile_shift = PLACE_SHIFT; c.slot_w = 2; c.lane_w = PLACE_LANE_W;
     }
     c.cand_late = h->d_cand_late;
     c.cands = (Cand<Real>*)h->d_cands; c.gap_head = h->d_gap_head;
@@ -456,7 +447,6 @@ Ctx<Real> make_ctx(MossHandle* h, int cur) {
 
 struct Grids {
     int decide_work, decide_ins, scan, place;
-    size_t place_smem;
 };
 
 // blocks of k_decide past its work blocks: one start lane per thread, and
@@ -473,12 +463,11 @@ Grids grids(const MossHandle* h) {
     g.decide_work = std::max(1, std::min((h->n_veh + 31) / 32, h->sm_count * std::min(h->cfg_decide, resident)));
     g.decide_ins = extra_blocks(h);
     g.scan = 0;
-    g.place = (int)(place_weight(h) >> place_shift(h)) + 1 + h->n_junc_chunks + 1;
+    g.place = (int)(place_weight(h) >> PLACE_SHIFT) + 1 + h->n_junc_chunks + 1;
     if (!fused_place(h)) {
         g.scan = ((h->n_lanes - 1) >> scan_shift(h)) + 1 + h->n_junc_chunks + 1;
         g.place = std::min(2 * (h->n_veh / TILE + 1), h->sm_count * h->cfg_place);
     }
-    g.place_smem = place_smem(place_lanes(place_shift(h)));
     return g;
 }
 
@@ -488,10 +477,10 @@ template <typename Real, bool Groups>
 cudaError_t launch_coop(MossHandle* h, Ctx<Real>& c) {
     int per_sm = 0;
     const Grids g = grids(h);
-    const size_t smem = g.scan ? 0 : g.place_smem;
-    // (its static part and a wide tile's lanes pass 48 KB together in FP64)
+    const size_t smem = g.scan ? 0 : PLACE_SMEM;
+    // (with its static part past 48 KB in FP64)
     cudaError_t e = cudaFuncSetAttribute(k_step_coop<Real, Groups>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)place_smem(1 << PLACE_LANES_LOG2));
+                                         (int)PLACE_SMEM);
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_coop<Real, Groups>, TILE, smem);
     if (e != cudaSuccess) return e;
@@ -500,8 +489,7 @@ cudaError_t launch_coop(MossHandle* h, Ctx<Real>& c) {
     int n_ins = g.decide_ins, n_scan = g.scan, n_place = g.place;
     unsigned* bar = h->d_bar;
     void* args[] = {(void*)&c, (void*)&n_work, (void*)&n_ins, (void*)&n_scan, (void*)&n_place, (void*)&bar};
-    return cudaLaunchCooperativeKernel((const void*)k_step_coop<Real, Groups>, grid, TILE, args, smem,
-                                       h->stream);
+    return cudaLaunchCooperativeKernel((const void*)k_step_coop<Real, Groups>, grid, TILE, args, smem, h->stream);
 }
 
 // one launch; chained: it may start while the kernel before it in the stream
@@ -541,7 +529,7 @@ void enqueue_step(MossHandle* h, int cur, bool timed, bool first) {
                        scan_q(h) == 2 ? k_lanescan<Real, 2> : k_lanescan<Real, SCAN_Q>, c, g.scan);
     if (timed) cudaEventRecord(h->ev[2], s);
     if (g.scan) launch_chained(h, !timed, g.place, TILE, 0, k_place_slots<Real>, c);
-    else launch_chained(h, !timed, g.place, TILE, g.place_smem, k_place<Real>, c);
+    else launch_chained(h, !timed, g.place, TILE, PLACE_SMEM, k_place<Real>, c);
     if (timed) cudaEventRecord(h->ev[3], s);
 }
 
@@ -875,7 +863,7 @@ int device_setup(MossHandle* h, void* stream) {
     TRY(upload(h, &h->d_enter, std::vector<int32_t>(NL, 0)));
     TRY(upload(h, &h->d_leave, std::vector<int32_t>(NL, 0)));
     // tiles under any schedule
-    h->max_tiles = std::max<size_t>(SCAN_MAX_TILES, (size_t)(place_weight(h) >> place_shift(h)) + 1);
+    h->max_tiles = std::max<size_t>(SCAN_MAX_TILES, (PLACE_MAX_WEIGHT >> PLACE_SHIFT) + 1);
     for (int k = 0; k < 2; ++k) {
         TRY(dalloc(h, &h->d_tiles[k], h->max_tiles + 1));
         TRY(dalloc(h, &h->d_delta[k], h->max_tiles));

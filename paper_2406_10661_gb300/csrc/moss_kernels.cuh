@@ -877,11 +877,10 @@ __device__ void run_fit(const Ctx<Real>& c) {
 // k_place: the lane offsets of the next snapshot, then the snapshot itself.
 //
 // A tile is a run of whole lanes [tile_cur[t], tile_cur[t+1]) with their
-// vehicles, cut where slot_w * off[l] + lane_w * l passes a multiple of
-// 1 << tile_shift
-// (the previous step's tiles wrote the cuts).  newsize(l) = size(l) - leave(l)
-// + enter(l).  k_decide also counts how each tile grows (tile_delta), so the
-// next offset of a tile's first lane is its offset now plus the growth of the
+// vehicles, cut where 2 off[l] + PLACE_LANE_W l passes a multiple of
+// 1 << PLACE_SHIFT (the previous step's tiles wrote the cuts).  newsize(l) =
+// size(l) - leave(l) + enter(l).  k_decide also counts how each tile grows
+// (tile_delta), so the next offset of a tile's first lane is its offset now plus the growth of the
 // tiles before it: every tile adds those words up for itself and no tile
 // waits for another.  The vehicles of a lane lie in the tile, so a stayer's
 // next slot is its own slot plus a per-lane shift, minus the leavers before it
@@ -890,7 +889,9 @@ __device__ void run_fit(const Ctx<Real>& c) {
 // Bound by latency: about six dependent memory rounds and four barriers, 6 us
 // on the 12x12 grid and 10 on the 30x30 grid of 70,000 vehicles, where the
 // scan with look-back and the placement as two kernels took 16 and 15.5.  The
-// tile size follows the network (place_shift on the host).  Everything the
+// tiles are small (a slot per thread and 1.3 us less a step than twice the size
+// on the 30x30 grid); handles of more than about three per SM take the two
+// kernels below (PLACE_MAX_WEIGHT on the host).  Everything the
 // step before wrote (cuts, offsets, records) is loaded before grid_wait, past
 // L1: the tail of k_decide covers it.
 
@@ -909,15 +910,11 @@ __device__ __forceinline__ int entrants_ahead(const Ctx<Real>& c, int q, Real s,
 
 constexpr int TW = TILE / 32;           // warps per block
 constexpr int PLACE_ROUNDS = 16;        // slot rounds whose leaver masks are held at a time
-constexpr int PLACE_LANES_LOG2 = 11;    // a tile holds at most 2^11 lanes
-constexpr int PLACE_LANE_W = 4;         // weight of a lane in the tiles, in half-slots
-// shared memory of a tile with up to `lanes` lanes: next offset (one more),
-// shift, entrants and their list per lane
-__host__ __device__ constexpr size_t place_smem(int lanes) { return sizeof(int) * (4 * (size_t)lanes + 1); }
-// lanes of the widest tile: each one adds at least PLACE_LANE_W
-__host__ __device__ constexpr int place_lanes(int tile_shift) {
-    return ((1 << tile_shift) + PLACE_LANE_W - 1) / PLACE_LANE_W;
-}
+constexpr int PLACE_SHIFT = 9;          // a tile takes 1 << PLACE_SHIFT half-slots: a vehicle 2, a lane PLACE_LANE_W
+constexpr int PLACE_LANE_W = 4;
+constexpr int PLACE_LANES = (1 << PLACE_SHIFT) / PLACE_LANE_W;  // lanes of the widest tile
+static_assert(PLACE_LANES <= TILE, "a thread per lane");
+constexpr size_t PLACE_SMEM = sizeof(int) * (4 * PLACE_LANES + 1);
 
 // the clocks of every scenario, one step on (a frozen or retiring one stands
 // still; one that reaches its horizon freezes)
@@ -933,29 +930,31 @@ __device__ __forceinline__ void advance_clocks(const Ctx<Real>& c) {
 
 template <typename Real, bool Pdl>
 __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
-    extern __shared__ int s_lanes[];
     __shared__ unsigned long long s_wsum[TW];       // per warp: leavers << 32 | next size of its lanes
     __shared__ unsigned s_ball[PLACE_ROUNDS * TW];  // leaver mask of each 32 slots
     __shared__ int s_lp[PLACE_ROUNDS * TW];         // leavers of the tile before them
     __shared__ int s_sum[TW];
     __shared__ int s_nel;                           // lanes with entrants
-    const int cap = place_lanes(c.tile_shift);
-    int* const s_nx = s_lanes;            // [cap + 1] next offset of a lane
-    int* const s_sh = s_lanes + cap + 1;  // [cap] next slot - slot of a lane's first vehicle, + leavers before the lane
-    int* const s_hd = s_sh + cap;         // [cap] entrants of a lane: -1 none; >= 0 list; <= -2: one, ahead of the last
-                                          // -2 - s_hd stayers
-    int* const s_el = s_hd + cap;         // [cap] lanes with entrants
+    extern __shared__ int s_lanes[];      // (PLACE_SMEM: with the decision's FP64 queue past what a kernel may declare)
+    int* const s_nx = s_lanes;            // [PLACE_LANES + 1] next offset of a lane
+    int* const s_sh = s_nx + PLACE_LANES + 1;  // [PLACE_LANES] next slot - slot of a lane's first vehicle, + leavers before
+                                               // the lane
+    int* const s_hd = s_sh + PLACE_LANES;  // [PLACE_LANES] entrants of a lane: -1 none; >= 0 list; <= -2: one, ahead of
+                                           // the last -2 - s_hd stayers
+    int* const s_el = s_hd + PLACE_LANES;  // [PLACE_LANES] lanes with entrants
     const int tid = threadIdx.x, ln = tid & 31, w = tid >> 5;
     // ---- what the previous step wrote
     const int tag = __ldcg(&c.cnt->tag);
-    const int L0 = __ldcg(&c.tile_cur[tile]), L1 = __ldcg(&c.tile_cur[tile + 1]), m = L1 - L0;
+    const int L0 = __ldcg(&c.tile_cur[tile]), L1 = __ldcg(&c.tile_cur[tile + 1]);
     const int S0 = __ldcg(&c.cur.off[L0]), S1 = __ldcg(&c.cur.off[L1]);
-    const int K = (m + TILE - 1) / TILE;  // lane rounds of a warp
-    const int kw = w * 32 * K + ln;       // the thread's first lane of the tile
+    // (a step that reported ERR_RANGE may have left cuts of two steps: this
+    // one ends below, past the writes to the arrays above)
+    const int m = min(L1 - L0, PLACE_LANES);
+    const int l = L0 + tid;  // the thread's lane of the tile (tid < m)
     int o0 = 0, o1 = 0;
-    if (kw < m) {
-        o0 = __ldcg(&c.cur.off[L0 + kw]);
-        o1 = __ldcg(&c.cur.off[L0 + kw + 1]);
+    if (tid < m) {
+        o0 = __ldcg(&c.cur.off[l]);
+        o1 = __ldcg(&c.cur.off[l + 1]);
     }
     int2 al = make_int2(-1, -1);  // id, lane of the first round's record
     int4 ab = make_int4(0, 0, 0, 0);
@@ -979,37 +978,26 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
     }
     int grown = 0;
     for (int p = tid; p < tile; p += TILE) grown += c.tile_delta[p];
-    unsigned long long run = 0;
-    for (int r = 0; r < K; ++r) {
-        const int k = kw + 32 * r, l = L0 + k;
-        unsigned long long x = 0;
-        if (k < m) {
-            if (r) { o0 = c.cur.off[l]; o1 = c.cur.off[l + 1]; }
-            const int lv = c.leave[l], en = c.enter[l];
-            const unsigned long long h = c.head[l];
-            if (lv) c.leave[l] = 0;
-            s_hd[k] = -1;
-            if (en) {
-                c.enter[l] = 0;
-                if ((int)(h >> 32) == tag) s_hd[k] = (int)(unsigned)(h & 0xffffffffull);
-                s_el[atomicAdd(&s_nel, 1)] = k;
-            }
-            x = ((unsigned long long)(unsigned)lv << 32) | (unsigned)(o1 - o0 - lv + en);
+    unsigned long long x = 0;
+    if (tid < m) {
+        const int lv = c.leave[l], en = c.enter[l];
+        const unsigned long long h = c.head[l];
+        if (lv) c.leave[l] = 0;
+        s_hd[tid] = -1;
+        if (en) {
+            c.enter[l] = 0;
+            if ((int)(h >> 32) == tag) s_hd[tid] = (int)(unsigned)(h & 0xffffffffull);
+            s_el[atomicAdd(&s_nel, 1)] = tid;
         }
-        unsigned long long incl = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (ln >= o) incl += y;
-        }
-        const unsigned long long ex = run + incl - x;
-        if (k < m) {
-            s_nx[k] = (int)(unsigned)(ex & 0xffffffffull);
-            s_sh[k] = (int)(ex >> 32) - o0;
-        }
-        run += __shfl_sync(0xffffffffu, incl, 31);
+        x = ((unsigned long long)(unsigned)lv << 32) | (unsigned)(o1 - o0 - lv + en);
     }
-    if (ln == 0) s_wsum[w] = run;
+    unsigned long long incl = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (ln >= o) incl += y;
+    }
+    if (ln == 31) s_wsum[w] = incl;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) grown += __shfl_xor_sync(0xffffffffu, grown, o);
     if (ln == 0) s_sum[w] = grown;
@@ -1045,26 +1033,22 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
             carry += __shfl_sync(0xffffffffu, incl, 31);
         }
     }
-    const int nb = prefix + (int)(unsigned)(wb & 0xffffffffull), lb = (int)(wb >> 32);
-    for (int r = 0; r < K; ++r) {
-        const int k = kw + 32 * r;
-        if (k < m) {
-            const int nx = nb + s_nx[k];
-            c.nxt.off[L0 + k] = nx;
-            s_nx[k] = nx;
-            s_sh[k] += nx + lb;
-        }
+    const unsigned long long ex = wb + incl - x;  // leavers << 32 | next size of the lanes before the thread's
+    if (tid < m) {
+        const int nx = prefix + (int)(unsigned)(ex & 0xffffffffull);
+        c.nxt.off[l] = nx;
+        s_nx[tid] = nx;
+        s_sh[tid] = nx + (int)(ex >> 32) - o0;
     }
     if (tid == 0) s_nx[m] = prefix + (int)(unsigned)(tot & 0xffffffffull);
     __syncthreads();
     // ---- the next step's tile cuts and the ends of the snapshot
-    for (int k = tid; k < m; k += TILE) {
-        const int l = L0 + k;
-        const int q0 = tile_key(c, s_nx[k], l), q1 = tile_key(c, s_nx[k + 1], l + 1);
+    if (tid < m) {
+        const int q0 = tile_key(c, s_nx[tid], l), q1 = tile_key(c, s_nx[tid + 1], l + 1);
         for (int q = q0 + 1; q <= q1; ++q) c.tile_nxt[q] = l + 1;
         if (l + 1 == c.n_lanes) {
-            c.nxt.off[l + 1] = s_nx[k + 1];
-            c.cnt_next->n_cur = s_nx[k + 1];
+            c.nxt.off[l + 1] = s_nx[tid + 1];
+            c.cnt_next->n_cur = s_nx[tid + 1];
             c.tile_nxt[q1 + 1] = l + 1;
         }
     }

@@ -388,3 +388,40 @@ def test_scan_schedules(roads, lanescan, lanes_per_thread):
     b.step(9)
     _same(a, b, 500, waiting=0)
     assert a.metrics()["n_arrived"] + a.metrics()["n_active"] == 500
+
+
+@pytest.mark.parametrize("side,trips,launches", [(4, 1000, 2), (12, 12007, 2), (30, 15000, 2), (30, 100_000, 3),
+                                                 (100, 1000, 3)])
+def test_form_follows_vehicles_and_lanes(side, trips, launches):
+    """The form whose step was measured faster: three-lane grids, by trips and
+    by lanes (471,624 at the last), and the same results next to the line."""
+    net = sc.grid_network(side, 200.0, 3, 13.89)
+    veh = sc.random_demand(net, trips, 60, seed=1, dest_pool=64)
+    sim = binding.Simulation(net, veh, sc.Params())
+    assert sim.step_launches() == launches
+    if trips == 1000 and side == 100:
+        large = binding.Simulation(net, _more(veh), sc.Params())
+        sim.step(90); large.step(90)
+        _same(sim, large, trips)
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("past", [0, 1])
+def test_both_sides_of_the_line(past, precision):
+    """The heaviest handle that takes the placement by tiles and the next one:
+    the same rollout, FP64 as the oracle's."""
+    scen = sc.small_scenario()
+    k = (240_000 - 4 * scen.net.n_lanes) // 2 + past
+    veh = _more(scen.veh)
+    end = int(veh.route_off[k])
+    veh = sc.Vehicles(n=k, route_off=veh.route_off[:k + 1], routes=veh.routes[:end], start_lane=veh.start_lane[:k],
+                      dep=veh.dep[:k], v0f=veh.v0f[:k])
+    sim = binding.Simulation(scen.net, veh, scen.params, precision=precision)
+    assert sim.step_launches() == 2 + past
+    a = binding.Simulation(scen.net, scen.veh, scen.params, precision=precision)
+    sim.step(150); a.step(150)
+    _same(a, sim, scen.veh.n, waiting=k - scen.veh.n)
+    if precision == 64:
+        ora = oracle.Oracle(scen.net, scen.veh, scen.params)
+        ora.step(150)
+        _as_oracle(sim, ora, scen.veh.n)
