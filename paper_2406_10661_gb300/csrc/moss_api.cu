@@ -150,7 +150,7 @@ struct MossHandle {
     bool rb_pending[MOSS_METRIC_SLOTS] = {};
 
     // launch configuration (blocks per SM) of the step kernels; moss_autotune picks them
-    int cfg_decide = MOSS_DECIDE_MIN_BLOCKS, cfg_lanescan = 4, cfg_place = 8;
+    int cfg_decide = 0, cfg_lanescan = 4, cfg_place = 8;  // (cfg_decide: as many as an SM holds at once)
     int cfg_runw = 0;    // weight of a road-lane slot in k_decide's runs (0: fitted each step)
     int cfg_lsr = 4;     // lanes per thread of a round of k_lanescan, over 4 (4 or 2)
     int cfg_ccap = 256;  // lane-change candidates a k_decide block lists in shared memory
@@ -458,9 +458,8 @@ int extra_blocks(const MossHandle* h) {
 
 Grids grids(const MossHandle* h) {
     Grids g;
-    // runs of at least a warp of vehicles, as many as the chip holds at once
-    const int resident = h->precision == 64 ? decide_min_blocks<double>() : decide_min_blocks<float>();
-    g.decide_work = std::max(1, std::min((h->n_veh + 31) / 32, h->sm_count * std::min(h->cfg_decide, resident)));
+    // runs of at least a warp of vehicles
+    g.decide_work = std::max(1, std::min((h->n_veh + 31) / 32, h->sm_count * h->cfg_decide));
     g.decide_ins = extra_blocks(h);
     g.scan = 0;
     g.place = (int)(place_weight(h) >> PLACE_SHIFT) + 1 + h->n_junc_chunks + 1;
@@ -778,6 +777,7 @@ int device_setup(MossHandle* h, void* stream) {
     }
     CK(cudaGetDevice(&h->device));
     CK(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device));
+    h->cfg_decide = h->precision == 64 ? decide_min_blocks<double>() : decide_min_blocks<float>();
     TRY(upload(h, &h->d_lane, h->lanes));
     std::vector<JuncInfo> junc(NJ);
     for (int j = 0; j < NJ; ++j) {

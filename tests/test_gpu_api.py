@@ -206,3 +206,22 @@ def test_lane_and_road_getters_match_the_state(G):
     want = np.where(cnt > 0, total / np.maximum(cnt, 1), limit / np.diff(net.road_lane_off))
     assert np.allclose(sim.road_speed(), want, rtol=1e-12, atol=0)
     assert stopped.any()
+
+
+@pytest.mark.parametrize("precision,default", [(32, 5), (64, 3)])
+def test_decide_blocks_are_what_the_schedule_says(precision, default):
+    """The default is the number of k_decide blocks that an SM holds at once in this precision; more, which run one
+    after the other, are taken as asked and give the same result."""
+    scen = sc.small_groups_scenario()
+    ref = binding.Simulation(scen.net, scen.veh, scen.params, precision=precision)
+    assert ref.schedule()["decide"] == default
+    ref.step(120)
+    for decide in (1, default + 1, 16):
+        sim = binding.Simulation(scen.net, scen.veh, scen.params, precision=precision)
+        sim.set_schedule(decide=decide)
+        assert sim.schedule()["decide"] == decide
+        sim.step(120)
+        a, b = ref.state(), sim.state()
+        for k in a:
+            assert np.array_equal(a[k], b[k]), k
+        assert ref.metrics() == sim.metrics()
