@@ -469,7 +469,7 @@ int moss_step_launches(moss_t h, int* out);
 
 /*
  * Autotuner of the launch schedule (no counterpart in the paper): times the
- * next steps of the simulation (16 x trial_steps of them, 14 without
+ * next steps of the simulation (16 x trial_steps of them, 15 without
  * cooperative launch; they are simulated normally, and the results do not
  * depend on the schedule) under candidate schedules, keeps the fastest by
  * coordinate search over, in this order: k_decide blocks per SM {3,4,5}; the
@@ -477,9 +477,13 @@ int moss_step_launches(moss_t h, int* out);
  * block runs {0,1,2} (a junction-lane vehicle weighs 1; 0: the weight fitted
  * each step); k_lanescan blocks per SM {1,2,4}; lanes per thread of a round of
  * the lane scan {16,8}; k_place_slots blocks per SM {4,8,16}; the step mode
- * {0,1} (moss_set_step_mode).  Then it re-captures the step graphs.  chosen3
- * (may be NULL) receives the chosen decide/lanescan/place blocks per SM;
- * moss_get_schedule returns the whole schedule.
+ * {0,1} (moss_set_step_mode).  The trial steps are replayed from graphs as
+ * moss_step replays them.  A value that the handle's steps do not read stays
+ * (the scan's and the slots' up to two kernels per step, the road-lane weight
+ * in small handles), and so does one that no other beats by 2%.  Then it
+ * re-captures the step graphs.  chosen3 (may be NULL) receives the chosen
+ * decide/lanescan/place blocks per SM; moss_get_schedule returns the whole
+ * schedule.
  */
 int moss_autotune(moss_t h, int trial_steps, int* chosen3);
 

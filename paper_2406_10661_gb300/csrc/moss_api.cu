@@ -579,25 +579,38 @@ void destroy_graphs(MossHandle* h) {
         }
 }
 
-int build_graphs(MossHandle* h) {
-    for (int p = 0; p < 2; ++p) {
-        for (int q = 0; q < N_GRAPHS; ++q) {
-            cudaGraph_t g = nullptr;
-            CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-            h->launch_err = cudaSuccess;
-            for (int k = 0; k < GRAPH_STEPS[q]; ++k) enqueue(h, (p + k) & 1, false, k == 0);
-            CK(cudaStreamEndCapture(h->stream, &g));
-            if (h->launch_err != cudaSuccess) {
-                cudaGraphDestroy(g);
-                return cuda_fail(h, h->launch_err, "step launch");
-            }
-            cudaGraphExec_t ex = nullptr;
-            cudaError_t e = cudaGraphInstantiate(&ex, g, 0);
-            cudaGraphDestroy(g);
-            if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphInstantiate");
-            h->graph[q][p] = ex;
-        }
+// graph q (GRAPH_STEPS[q] steps) from parity p
+int build_graph(MossHandle* h, int q, int p) {
+    cudaGraph_t g = nullptr;
+    CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+    h->launch_err = cudaSuccess;
+    for (int k = 0; k < GRAPH_STEPS[q]; ++k) enqueue(h, (p + k) & 1, false, k == 0);
+    CK(cudaStreamEndCapture(h->stream, &g));
+    if (h->launch_err != cudaSuccess) {
+        cudaGraphDestroy(g);
+        return cuda_fail(h, h->launch_err, "step launch");
     }
+    cudaGraphExec_t ex = nullptr;
+    cudaError_t e = cudaGraphInstantiate(&ex, g, 0);
+    cudaGraphDestroy(g);
+    if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphInstantiate");
+    h->graph[q][p] = ex;
+    return MOSS_OK;
+}
+
+int build_graphs(MossHandle* h) {
+    for (int p = 0; p < 2; ++p)
+        for (int q = 0; q < N_GRAPHS; ++q) TRY(build_graph(h, q, p));
+    return MOSS_OK;
+}
+
+// n steps by graph replay
+int replay_steps(MossHandle* h, int n) {
+    for (int q = 0; q < N_GRAPHS; ++q)
+        for (; n >= GRAPH_STEPS[q]; n -= GRAPH_STEPS[q]) {
+            CK(cudaGraphLaunch(h->graph[q][h->parity], h->stream));
+            h->parity ^= GRAPH_STEPS[q] & 1;
+        }
     return MOSS_OK;
 }
 
@@ -1646,12 +1659,7 @@ int moss_step(moss_t h, int n) {
         CK(cudaGetLastError());
         return MOSS_OK;
     }
-    for (int q = 0; q < N_GRAPHS; ++q)
-        for (; n >= GRAPH_STEPS[q]; n -= GRAPH_STEPS[q]) {
-            CK(cudaGraphLaunch(h->graph[q][h->parity], h->stream));
-            h->parity ^= GRAPH_STEPS[q] & 1;
-        }
-    return MOSS_OK;
+    return replay_steps(h, n);
 }
 
 int moss_set_signal_phase(moss_t h, int n, const int32_t* junction_ids, const int32_t* phase_idx) {
@@ -2090,20 +2098,22 @@ int moss_set_kernel_timing(moss_t h, int enable) {
     return MOSS_OK;
 }
 
-// time `steps` steps (the simulation advances normally) with the current
-// launch configuration; returns the summed kernel milliseconds
+// milliseconds of `steps` steps under the current schedule as moss_step runs
+// them, by graph replay (the simulation advances normally)
 static int time_steps(MossHandle* h, int steps, double* ms) {
-    double tot = 0;
-    for (int k = 0; k < steps; ++k) {
-        enqueue(h, h->parity, true, true);
-        h->parity ^= 1;
-        CK(cudaEventSynchronize(h->ev[N_STEP_KERNELS]));
-        float x = 0;
-        CK(cudaEventElapsedTime(&x, h->ev[0], h->ev[N_STEP_KERNELS]));
-        tot += x;
+    destroy_graphs(h);
+    for (int q = 0, n = steps; q < N_GRAPHS; n %= GRAPH_STEPS[q], ++q) {
+        if (n < GRAPH_STEPS[q]) continue;
+        TRY(build_graph(h, q, h->parity));  // (only the last graph, one step at most, changes the parity)
+        CK(cudaGraphUpload(h->graph[q][h->parity], h->stream));
     }
-    CK(cudaGetLastError());
-    *ms = tot;
+    CK(cudaEventRecord(h->ev[0], h->stream));
+    TRY(replay_steps(h, steps));
+    CK(cudaEventRecord(h->ev[1], h->stream));
+    CK(cudaEventSynchronize(h->ev[1]));
+    float x = 0;
+    CK(cudaEventElapsedTime(&x, h->ev[0], h->ev[1]));
+    *ms = x;
     return MOSS_OK;
 }
 
@@ -2113,34 +2123,55 @@ int moss_autotune(moss_t h, int trial_steps, int* chosen3) {
     CK(cudaStreamSynchronize(h->stream));
     // coordinate search over the schedule: blocks per SM of each kernel, the
     // road-lane weight of k_decide's runs, the lanes per thread of the scan and
-    // the step mode; results do not depend on the schedule, only the time does
+    // the step mode; results do not depend on the schedule, only the time does.
+    // A value that the handle's step does not read keeps what it is (its trial
+    // steps follow under the chosen schedule), and so does one that no other
+    // beats by TUNE_MARGIN, what the steps of one schedule differ by.
+    constexpr double TUNE_MARGIN = 0.98;
     int coop = 0;
     CK(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device));
-    struct Knob { int* v; int n; int c[3]; };
+    const bool two = !fused_place(h);  // k_lanescan and k_place_slots
+    // k_decide's runs go by weight when its blocks take four tiles or more
+    const bool weighted = (h->n_veh + TILE - 1) / TILE >= 4 * h->sm_count * 3;
+    struct Knob { int* v; int n; int c[3]; bool read; };
     const Knob knobs[] = {
-        {&h->cfg_decide, 3, {3, 4, 5}},   {&h->cfg_runw, 3, {0, 1, 2}}, {&h->cfg_lanescan, 3, {1, 2, 4}},
-        {&h->cfg_lsr, 2, {4, 2, 0}},      {&h->cfg_place, 3, {4, 8, 16}}, {&h->step_mode, coop ? 2 : 1, {0, 1, 0}},
+        {&h->cfg_decide, 3, {3, 4, 5}, true}, {&h->cfg_runw, 3, {0, 1, 2}, weighted}, {&h->cfg_lanescan, 3, {1, 2, 4}, two},
+        {&h->cfg_lsr, 2, {4, 2, 0}, two}, {&h->cfg_place, 3, {4, 8, 16}, two},
+        {&h->step_mode, coop ? 2 : 1, {0, 1, 0}, coop != 0},
     };
+    const int mode = h->step_mode;
+    h->step_mode = 0;  // (the single launch reads the run weight alone)
+    int left = 0, rc = MOSS_OK;
     for (const Knob& kb : knobs) {
-        int best = *kb.v;
-        double best_ms = 1e300;
-        for (int k = 0; k < kb.n; ++k) {
+        if (!kb.read) {
+            left += kb.n * trial_steps;
+            continue;
+        }
+        const int was = kb.v == &h->step_mode ? mode : *kb.v;
+        int best = was;
+        double best_ms = 1e300, was_ms = 1e300;
+        for (int k = 0; k < kb.n && rc == MOSS_OK; ++k) {
             *kb.v = kb.c[k];
-            h->launch_err = cudaSuccess;
-            TRY(tile_cuts(h));
             double ms = 0;
-            TRY(time_steps(h, trial_steps, &ms));
-            if (h->launch_err != cudaSuccess) {  // a mode this device cannot launch
+            rc = tile_cuts(h);
+            if (rc == MOSS_OK) rc = time_steps(h, trial_steps, &ms);
+            if (rc != MOSS_OK && h->launch_err != cudaSuccess) {  // a mode this device cannot launch
                 h->launch_err = cudaSuccess;
+                rc = MOSS_OK;
+                left += trial_steps;
                 continue;
             }
             if (ms < best_ms) { best_ms = ms; best = kb.c[k]; }
+            if (kb.c[k] == was) was_ms = ms;
         }
-        *kb.v = best;
+        *kb.v = was_ms * TUNE_MARGIN <= best_ms ? was : best;
     }
-    TRY(tile_cuts(h));
+    if (rc != MOSS_OK) h->step_mode = mode;
     destroy_graphs(h);
+    TRY(tile_cuts(h));
     TRY(build_graphs(h));
+    if (rc != MOSS_OK) return rc;
+    TRY(replay_steps(h, left));
     if (chosen3) { chosen3[0] = h->cfg_decide; chosen3[1] = h->cfg_lanescan; chosen3[2] = h->cfg_place; }
     return check_device(h);
 }

@@ -225,3 +225,26 @@ def test_decide_blocks_are_what_the_schedule_says(precision, default):
         for k in a:
             assert np.array_equal(a[k], b[k]), k
         assert ref.metrics() == sim.metrics()
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("trial", [1, 11])
+def test_autotune_leaves_what_the_step_does_not_read(trial, precision):
+    """A small handle's steps have no lane scan, no placement by slots and no weighted runs: those values stay, and the
+    steps are the announced number, replayed in every length of graph (11 = 8 + 2 + 1), with unchanged results."""
+    scen = sc.small_scenario()
+    sim = binding.Simulation(scen.net, scen.veh, scen.params, precision=precision)
+    assert sim.step_launches() == 2
+    sim.step(21)
+    before = sim.schedule()
+    chosen = sim.autotune(trial)
+    for k in ("lanescan", "place", "lanes_per_thread", "road_weight", "candidates_per_block"):
+        assert chosen[k] == before[k], (k, before, chosen)
+    assert sim.metrics()["step"] == 21 + 16 * trial
+    ref = binding.Simulation(scen.net, scen.veh, scen.params, precision=precision)
+    ref.step(21 + 16 * trial + 7)
+    sim.step(7)
+    a, b = ref.state(), sim.state()
+    for k in a:
+        assert np.array_equal(a[k], b[k]), k
+    assert ref.metrics() == sim.metrics()
