@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -1248,14 +1249,24 @@ int enqueue_readback(MossHandle* h, int s, int slot) {
 }
 
 // waits until the slot's last readback has arrived; an error of the stream
-// ends the wait, and so does the end of its work
+// ends the wait, and so does the end of its work.  Past the first looks (some
+// 10 us) it waits as the process has asked CUDA to wait: it sleeps between the
+// looks under cudaDeviceScheduleBlockingSync, else it spins or yields.
 int wait_readback(MossHandle* h, int slot) {
     const long long* word = h->h_rb + (size_t)slot * RB_WORDS + M_NFIELDS + 2;
     const long long ticket = h->rb_ticket[slot];
+    unsigned how = ~0u;
     for (unsigned spins = 1; __atomic_load_n(word, __ATOMIC_ACQUIRE) != ticket; ++spins) {
-        if (spins % 4096) continue;
+        if (spins % 4096 && (how & cudaDeviceScheduleMask) != cudaDeviceScheduleBlockingSync) continue;
         const cudaError_t e = cudaStreamQuery(h->stream);
-        if (e == cudaErrorNotReady) continue;
+        if (e == cudaErrorNotReady) {
+            if (how == ~0u) CK(cudaGetDeviceFlags(&how));
+            if ((how & cudaDeviceScheduleMask) == cudaDeviceScheduleBlockingSync)
+                std::this_thread::sleep_for(std::chrono::microseconds(50));
+            else if ((how & cudaDeviceScheduleMask) == cudaDeviceScheduleYield)
+                std::this_thread::yield();
+            continue;
+        }
         CK(e);
         CK(cudaStreamSynchronize(h->stream));
         if (__atomic_load_n(word, __ATOMIC_ACQUIRE) != ticket) return fail(h, MOSS_ECUDA, "a metric readback is missing");

@@ -1,6 +1,8 @@
 """Metrics read without waiting for the stream (moss_metrics_enqueue /
 moss_metrics_read): a slot holds the metrics as they were when it was
 enqueued, later steps do not change it, and misuse is refused."""
+import os
+
 import numpy as np
 import pytest
 
@@ -248,3 +250,36 @@ def test_autotune_leaves_what_the_step_does_not_read(trial, precision):
     for k in a:
         assert np.array_equal(a[k], b[k]), k
     assert ref.metrics() == sim.metrics()
+
+
+_BLOCKING = """
+import ctypes, sys, time
+cuda = ctypes.CDLL("libcuda.so.1")
+assert cuda.cuInit(0) == 0
+dev = ctypes.c_int()
+assert cuda.cuDeviceGet(ctypes.byref(dev), 0) == 0
+assert cuda.cuDevicePrimaryCtxSetFlags_v2(dev, 4) == 0  # CU_CTX_SCHED_BLOCKING_SYNC
+from paper_2406_10661_gb300 import binding, scenario as sc
+scen = sc.city_scenario(n=600_000, G=50, dest_pool=64)
+sim = binding.Simulation(scen.net, scen.veh, scen.params)
+sim.step(8)
+sim.metrics()
+for read in (sim.metrics, sim.lane_queue, lambda: (sim.metrics_enqueue(0), sim.metrics_read(0))):
+    sim.step(4000)
+    wall, cpu = time.perf_counter(), time.thread_time()
+    read()
+    print(time.perf_counter() - wall, time.thread_time() - cpu)
+"""
+
+
+def test_readers_sleep_where_the_process_asked_for_it():
+    """Under blocking synchronisation a reader behind queued steps leaves its core idle (10 looks of a few us per ms and
+    the first ones: a quarter at most) and still returns."""
+    import subprocess
+    import sys
+    out = subprocess.run([sys.executable, "-c", _BLOCKING], capture_output=True, text=True, timeout=300,
+                         cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert out.returncode == 0, out.stderr
+    waits = np.array([line.split() for line in out.stdout.splitlines()], dtype=np.float64)
+    assert len(waits) == 3 and (waits[:, 0] > 0.02).all(), waits
+    assert (waits[:, 1] < 0.25 * waits[:, 0]).all(), waits
