@@ -52,3 +52,12 @@ def test_committed_profiles_have_traffic_lines():
         with open(os.path.join(prof, f)) as fh:
             kernels = [m.group(1) for m in (pat.match(line.strip()) for line in fh) if m]
         assert sorted(kernels) == ["k_decide", "k_lanescan", "k_place"], f
+
+
+def test_lane_bytes_follow_the_form_of_the_step():
+    """24 B per lane (offset, leave and enter read, next offset written, both counts cleared), charged to the lane scan,
+    or to the placement where the step has no scan of its own."""
+    two = bench.launch_bytes({"decide": 1.0, "lanescan": 0.0, "place": 1.0}, 1000.0, 100)
+    three = bench.launch_bytes({"decide": 1.0, "lanescan": 0.1, "place": 1.0}, 1000.0, 100)
+    assert three == {"decide": 41e3, "lanescan": 2400.0, "place": 73e3}
+    assert two == {"decide": 41e3, "lanescan": 0.0, "place": 73e3 + 2400.0}
