@@ -381,6 +381,7 @@ size_t sv_size(int precision) { return precision == 64 ? sizeof(SV<double>) : si
 //    4,000 on  2,424:  18.9 / 21.1     20,000 on 361,802: 25.4 / 24.7
 // (FP64 alike: 38.0 / 38.8 at 36,000 trips, 57.0 / 55.7 at 100,000).
 constexpr long long PLACE_MAX_WEIGHT = 240000;
+constexpr int PLACE_SHIFT = 9;
 long long place_weight(const MossHandle* h) { return 2ll * h->n_veh + (long long)PLACE_LANE_W * h->n_lanes; }
 bool fused_place(const MossHandle* h) { return place_weight(h) <= PLACE_MAX_WEIGHT; }
 
@@ -477,10 +478,10 @@ template <typename Real, bool Groups>
 cudaError_t launch_coop(MossHandle* h, Ctx<Real>& c) {
     int per_sm = 0;
     const Grids g = grids(h);
-    const size_t smem = g.scan ? 0 : PLACE_SMEM;
+    const size_t smem = g.scan ? 0 : place_smem<Real>();
     // (with its static part past 48 KB in FP64)
     cudaError_t e = cudaFuncSetAttribute(k_step_coop<Real, Groups>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)PLACE_SMEM);
+                                         (int)place_smem<Real>());
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_coop<Real, Groups>, TILE, smem);
     if (e != cudaSuccess) return e;
@@ -529,7 +530,7 @@ void enqueue_step(MossHandle* h, int cur, bool timed, bool first) {
                        scan_q(h) == 2 ? k_lanescan<Real, 2> : k_lanescan<Real, SCAN_Q>, c, g.scan);
     if (timed) cudaEventRecord(h->ev[2], s);
     if (g.scan) launch_chained(h, !timed, g.place, TILE, 0, k_place_slots<Real>, c);
-    else launch_chained(h, !timed, g.place, TILE, PLACE_SMEM, k_place<Real>, c);
+    else launch_chained(h, !timed, g.place, TILE, place_smem<Real>(), k_place<Real>, c);
     if (timed) cudaEventRecord(h->ev[3], s);
 }
 

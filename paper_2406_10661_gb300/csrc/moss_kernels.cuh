@@ -878,7 +878,7 @@ __device__ void run_fit(const Ctx<Real>& c) {
 //
 // A tile is a run of whole lanes [tile_cur[t], tile_cur[t+1]) with their
 // vehicles, cut where 2 off[l] + PLACE_LANE_W l passes a multiple of
-// 1 << PLACE_SHIFT (the previous step's tiles wrote the cuts).  newsize(l) =
+// 1 << tile_shift (the previous step's tiles wrote the cuts).  newsize(l) =
 // size(l) - leave(l) + enter(l).  k_decide also counts how each tile grows
 // (tile_delta), so the next offset of a tile's first lane is its offset now plus the growth of the
 // tiles before it: every tile adds those words up for itself and no tile
@@ -886,14 +886,20 @@ __device__ void run_fit(const Ctx<Real>& c) {
 // next slot is its own slot plus a per-lane shift, minus the leavers before it
 // in the tile, plus the entrants ahead of it.
 //
+// The entrants of the tile are gathered in shared memory (a lane's list is
+// walked once, by the lane's thread), ranked there and counted against the
+// stayers eight threads each, side by side: in the flowing traffic of a city
+// some lane takes several every step, and every step waits for the worst lane.
+// One entrant of a lane after the other, each walking the list again, the
+// kernel took 17 to 21 us between its events on cities of 50,000 to 150,000
+// trips, so 10 to 12 (a step 29.5 -> 23.5 and 40.8 -> 28.8 us; by slots 26.3
+// and 30.8).
+//
 // Bound by latency: about six dependent memory rounds and four barriers, 6 us
-// on the 12x12 grid and 10 on the 30x30 grid of 70,000 vehicles, where the
-// scan with look-back and the placement as two kernels took 16 and 15.5.  The
-// tiles are small (a slot per thread and 1.3 us less a step than twice the size
-// on the 30x30 grid); handles of more than about three per SM take the two
-// kernels below (PLACE_MAX_WEIGHT on the host).  Everything the
-// step before wrote (cuts, offsets, records) is loaded before grid_wait, past
-// L1: the tail of k_decide covers it.
+// on the 12x12 grid and 9 on the 30x30 grid of 70,000 vehicles, where the
+// scan with look-back and the placement as two kernels took 16 and 15.5.
+// Everything the step before wrote (cuts, offsets, records) is loaded before
+// grid_wait, past L1: the tail of k_decide covers it.
 
 // entrants of a list (from q on) that are ahead of (s, id); n_in: its length
 template <typename Real>
@@ -910,11 +916,15 @@ __device__ __forceinline__ int entrants_ahead(const Ctx<Real>& c, int q, Real s,
 
 constexpr int TW = TILE / 32;           // warps per block
 constexpr int PLACE_ROUNDS = 16;        // slot rounds whose leaver masks are held at a time
-constexpr int PLACE_SHIFT = 9;          // a tile takes 1 << PLACE_SHIFT half-slots: a vehicle 2, a lane PLACE_LANE_W
-constexpr int PLACE_LANE_W = 4;
-constexpr int PLACE_LANES = (1 << PLACE_SHIFT) / PLACE_LANE_W;  // lanes of the widest tile
+constexpr int PLACE_LANE_W = 4;         // weight of a lane in the tiles, in half-slots (a vehicle: 2)
+constexpr int PLACE_SHIFT_MAX = 10;     // a tile takes 1 << 9 or 1 << 10 half-slots
+constexpr int PLACE_LANES = (1 << PLACE_SHIFT_MAX) / PLACE_LANE_W;  // lanes of the widest tile
 static_assert(PLACE_LANES <= TILE, "a thread per lane");
-constexpr size_t PLACE_SMEM = sizeof(int) * (4 * PLACE_LANES + 1);
+constexpr int PLACE_ENT = 128;          // entrants that a tile holds in shared memory
+template <typename Real>
+__host__ __device__ constexpr size_t place_smem() {
+    return PLACE_ENT * (sizeof(Real) + 4 * sizeof(int)) + sizeof(int) * (5 * PLACE_LANES + 2);
+}
 
 // the clocks of every scenario, one step on (a frozen or retiring one stands
 // still; one that reaches its horizon freezes)
@@ -934,14 +944,21 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
     __shared__ unsigned s_ball[PLACE_ROUNDS * TW];  // leaver mask of each 32 slots
     __shared__ int s_lp[PLACE_ROUNDS * TW];         // leavers of the tile before them
     __shared__ int s_sum[TW];
-    __shared__ int s_nel;                           // lanes with entrants
-    extern __shared__ int s_lanes[];      // (PLACE_SMEM: with the decision's FP64 queue past what a kernel may declare)
-    int* const s_nx = s_lanes;            // [PLACE_LANES + 1] next offset of a lane
-    int* const s_sh = s_nx + PLACE_LANES + 1;  // [PLACE_LANES] next slot - slot of a lane's first vehicle, + leavers before
+    __shared__ int s_ne, s_nel;                     // entrants held here, lanes whose entrants are not
+    // (dynamic: with the decision's FP64 queue past what a kernel may declare)
+    extern __shared__ __align__(16) unsigned char s_mem[];
+    Real* const s_es = reinterpret_cast<Real*>(s_mem);               // [PLACE_ENT] entrants: position,
+    int* const s_eid = reinterpret_cast<int*>(s_es + PLACE_ENT);     // id,
+    int* const s_eq = s_eid + PLACE_ENT;                             // record (-1: none),
+    int* const s_ek = s_eq + PLACE_ENT;                              // lane of the tile,
+    int* const s_bh = s_ek + PLACE_ENT;                              // stayers of the lane behind it
+    int* const s_nx = s_bh + PLACE_ENT;     // [PLACE_LANES + 1] next offset of a lane
+    int* const s_ob = s_nx + PLACE_LANES + 1;  // [PLACE_LANES + 1] its offset
+    int* const s_sh = s_ob + PLACE_LANES + 1;  // [PLACE_LANES] next slot - slot of a lane's first vehicle, + leavers before
                                                // the lane
-    int* const s_hd = s_sh + PLACE_LANES;  // [PLACE_LANES] entrants of a lane: -1 none; >= 0 list; <= -2: one, ahead of
-                                           // the last -2 - s_hd stayers
-    int* const s_el = s_hd + PLACE_LANES;  // [PLACE_LANES] lanes with entrants
+    int* const s_hd = s_sh + PLACE_LANES;   // [PLACE_LANES] entrants of a lane: 0 none; > 0: 1 + (first of them here | how
+                                            // many << 9); < 0: ~(their list)
+    int* const s_el = s_hd + PLACE_LANES;   // [PLACE_LANES] lanes with a list
     const int tid = threadIdx.x, ln = tid & 31, w = tid >> 5;
     // ---- what the previous step wrote
     const int tag = __ldcg(&c.cnt->tag);
@@ -962,7 +979,8 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
         al = __ldcg(reinterpret_cast<const int2*>(&c.cur.a[S0 + tid].id));
         ab = __ldcg(reinterpret_cast<const int4*>(&c.cur.b[S0 + tid]));
     }
-    if (tid == 0) s_nel = 0;
+    if (tid == 0) s_ne = s_nel = 0;
+    if (tid < PLACE_ENT) s_eq[tid] = -1;
     __syncthreads();
     if (Pdl) {
         grid_wait();
@@ -983,12 +1001,28 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
         const int lv = c.leave[l], en = c.enter[l];
         const unsigned long long h = c.head[l];
         if (lv) c.leave[l] = 0;
-        s_hd[tid] = -1;
+        int hd = 0;
         if (en) {
             c.enter[l] = 0;
-            if ((int)(h >> 32) == tag) s_hd[tid] = (int)(unsigned)(h & 0xffffffffull);
-            s_el[atomicAdd(&s_nel, 1)] = tid;
+            if ((int)(h >> 32) == tag) {
+                int q = (int)(unsigned)(h & 0xffffffffull);
+                const int j = atomicAdd(&s_ne, en);
+                if (j + en <= PLACE_ENT) {
+                    hd = 1 + (j | en << 9);
+                    for (int t = 0; t < en; ++t) {
+                        s_eq[j + t] = q;
+                        s_ek[j + t] = tid;
+                        if (t + 1 < en && (q = c.enext[q]) < 0) { atomicOr(c.err, ERR_RANGE); break; }
+                    }
+                } else {
+                    hd = ~q;
+                    s_el[atomicAdd(&s_nel, 1)] = tid;
+                }
+            }
         }
+        s_hd[tid] = hd;
+        s_ob[tid] = o0;
+        s_ob[tid + 1] = o1;
         x = ((unsigned long long)(unsigned)lv << 32) | (unsigned)(o1 - o0 - lv + en);
     }
     unsigned long long incl = x;
@@ -1041,6 +1075,11 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
         s_sh[tid] = nx + (int)(ex >> 32) - o0;
     }
     if (tid == 0) s_nx[m] = prefix + (int)(unsigned)(tot & 0xffffffffull);
+    if (tid < PLACE_ENT && s_eq[tid] >= 0) {
+        const RecA<Real> Q = c.ea[s_eq[tid]];
+        s_es[tid] = Q.s;
+        s_eid[tid] = Q.id;
+    }
     __syncthreads();
     // ---- the next step's tile cuts and the ends of the snapshot
     if (tid < m) {
@@ -1052,65 +1091,87 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
             c.tile_nxt[q1 + 1] = l + 1;
         }
     }
-    // ---- entrants: eight threads per lane that has any, four lanes at a time
-    // in a warp.  The stayers of a lane keep their order (nobody overtakes
-    // within a lane, R13), so the stayers behind an entrant form the rear of
-    // the lane's old segment: they are counted from the segment's end, 8
-    // slots per round, up to the first round that holds a stayer ahead of the
-    // entrant (entrants join mostly at the rear of a lane: one round).
-    // Stayers ahead = the lane's stayers (its next size minus its entrants)
-    // minus those behind.
-    const int sub = ln >> 3, sl = ln & 7, nel = s_nel;
+    // ---- entrants: eight threads each, four at a time in a warp.  The stayers
+    // of a lane keep their order (nobody overtakes within a lane, R13), so the
+    // stayers behind an entrant form the rear of the lane's old segment: they
+    // are counted from the segment's end, 8 slots per round, up to the first
+    // round that holds a stayer ahead of the entrant (entrants join mostly at
+    // the rear of a lane: one round).  Stayers ahead = the lane's stayers (its
+    // next size minus its entrants) minus those behind.
+    const int sub = ln >> 3, sl = ln & 7, ne = min(s_ne, PLACE_ENT), nel = s_nel;
+    const auto stayers_behind = [&](bool open, int b, int e, Real s, int id) {
+        int bh = 0;
+        for (int x0 = e - 1; __any_sync(0xffffffffu, open); x0 -= 8) {
+            const int x = x0 - sl;
+            bool st = false, ah = false;
+            if (open && x >= b) {
+                st = c.code[x] == C_STAY;  // (the other loads go out with this one)
+                ah = ahead(c.stay[x].s, c.cur.a[x].id, s, id) && st;
+            }
+            const unsigned mb = (__ballot_sync(0xffffffffu, st && !ah) >> (8 * sub)) & 0xffu;
+            const unsigned ma = (__ballot_sync(0xffffffffu, ah) >> (8 * sub)) & 0xffu;
+            if (open) bh += __popc(mb);
+            if (ma || x0 - 8 < b) open = false;
+        }
+        return bh;
+    };
+    for (int j0 = 4 * w; j0 < ne; j0 += 4 * TW) {
+        const int j = j0 + sub, q = j < ne ? s_eq[j] : -1;
+        int k = 0, id = 0;
+        Real s = Real(0);
+        RecA<Real> Q;
+        RecB QB;
+        if (q >= 0) {
+            k = s_ek[j]; s = s_es[j]; id = s_eid[j];
+            if (sl == 0) { Q = c.ea[q]; QB = c.eb[q]; }
+        }
+        const int bh = stayers_behind(q >= 0, s_ob[k], s_ob[k + 1], s, id);
+        if (q < 0 || sl) continue;
+        s_bh[j] = bh;
+        const int n = (s_hd[k] - 1) >> 9, f = (s_hd[k] - 1) & 511;
+        int pos = s_nx[k + 1] - n - bh;
+        for (int t = f; t < f + n; ++t) pos += ahead(s_es[t], s_eid[t], s, id);
+        if (pos < s_nx[k] || pos >= s_nx[k + 1] || pos >= c.n_veh) {
+            atomicOr(c.err, ERR_RANGE);
+        } else {
+            c.nxt.a[pos] = Q;
+            c.nxt.b[pos] = QB;
+        }
+    }
+    // the lanes whose entrants did not fit, one entrant of a lane after the other
     for (int j0 = 4 * w; j0 < nel; j0 += 4 * TW) {
-        int q = -1, k = 0, b = 0, e = 0;
+        int q = -1, k = 0;
         if (j0 + sub < nel) {
             k = s_el[j0 + sub];
-            q = s_hd[k];
-            b = c.cur.off[L0 + k];
-            e = c.cur.off[L0 + k + 1];
+            q = ~s_hd[k];
         }
         const int q0 = q;
-        int n_in = 0, bh = 0;
+        int n_in = 0;
         while (__any_sync(0xffffffffu, q >= 0)) {
             RecA<Real> Q;
-            RecB QB;
+            Q.s = Real(0); Q.id = 0;
             int nq = -1;
             if (q >= 0) {
                 Q = c.ea[q];
                 nq = c.enext[q];
-                if (sl == 0) QB = c.eb[q];
             }
-            if (q >= 0) bh = 0;  // (a lane that is through keeps its count while others go on)
-            bool open = q >= 0;
-            for (int x0 = e - 1; __any_sync(0xffffffffu, open); x0 -= 8) {
-                const int x = x0 - sl;
-                bool st = false, ah = false;
-                if (open && x >= b && c.code[x] == C_STAY) {
-                    st = true;
-                    ah = ahead(c.stay[x].s, c.cur.a[x].id, Q.s, Q.id);
-                }
-                const unsigned mb = (__ballot_sync(0xffffffffu, st && !ah) >> (8 * sub)) & 0xffu;
-                const unsigned ma = (__ballot_sync(0xffffffffu, ah) >> (8 * sub)) & 0xffu;
-                bh += __popc(mb);
-                if (ma || x0 - 8 < b) open = false;
-            }
+            const int bh = stayers_behind(q >= 0, s_ob[k], s_ob[k + 1], Q.s, Q.id);
             if (q >= 0) {
                 if (sl == 0) {
-                    int len = 1, ent = 0;
-                    if (nq >= 0 || q != q0) ent = entrants_ahead(c, q0, Q.s, Q.id, &len);
+                    int len = 0;
+                    const int ent = entrants_ahead(c, q0, Q.s, Q.id, &len);
                     const int pos = s_nx[k + 1] - len - bh + ent;
                     if (pos < s_nx[k] || pos >= s_nx[k + 1] || pos >= c.n_veh) {
                         atomicOr(c.err, ERR_RANGE);
                     } else {
                         c.nxt.a[pos] = Q;
-                        c.nxt.b[pos] = QB;
+                        c.nxt.b[pos] = c.eb[q];
                     }
                 }
                 q = nq;
                 if (++n_in > c.n_veh) { atomicOr(c.err, ERR_RANGE); q = -1; }
             }
         }
-        if (n_in == 1 && sl == 0) s_hd[k] = -2 - bh;
     }
     __syncthreads();
     // ---- stayers
@@ -1148,8 +1209,12 @@ __device__ __forceinline__ void place_tile(const Ctx<Real>& c, int tile) {
             const int lane = al.y, k = lane - L0;
             const int o = s_nx[k], end = s_nx[k + 1], h = s_hd[k];
             int pos = s_sh[k] + i - (lcarry + s_lp[r * TW + w] + __popc(ball & ((1u << ln) - 1u)));
-            if (h >= 0) pos += entrants_ahead(c, h, sv.s, al.x);
-            else if (h != -1) pos += end - 2 - pos < -2 - h;  // stayers behind it: end - 2 - pos
+            if (h > 0) {  // an entrant is ahead of the stayers behind it
+                const int n = (h - 1) >> 9, f = (h - 1) & 511, behind = end - n - 1 - pos;
+                for (int t = f; t < f + n; ++t) pos += s_bh[t] > behind;
+            } else if (h < 0) {
+                pos += entrants_ahead(c, ~h, sv.s, al.x);
+            }
             if (pos < o || pos >= end || pos >= c.n_veh) {
                 atomicOr(c.err, ERR_RANGE);
             } else {

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import oracle
+import test_gpu_large_form as large
 from paper_2406_10661_gb300 import binding, scenario as sc
 
 pytestmark = pytest.mark.gpu
@@ -91,3 +92,59 @@ def test_attempt_draw(precision, p_attempt):
         o.step(1)
     assert sim.metrics()["mobil_evals"] == ora.metrics()["mobil_evals"]
     assert (p_attempt > 0) == (sim.metrics()["mobil_evals"] > 0)
+
+
+# 40 .. 520 entrants of one lane in one step: some held in shared memory (up to 128 per tile), some listed, and the
+# tiles' lanes mixed; (1, 40): the lanes of a whole tile with one or two each
+@pytest.mark.parametrize("precision", [32, 64])
+@pytest.mark.parametrize("n,lanes", [(40, 2), (127, 2), (128, 2), (129, 2), (257, 3), (520, 2), (1040, 4)])
+def test_many_entrants_of_a_lane(n, lanes, precision):
+    """Everyone attempts a change and gains by any: bursts from the full lane into the others, each step."""
+    rng = np.random.RandomState(n)
+    net = sc.corridor_network(lanes, (14.0 * n + 100.0, 400.0))
+    lane = np.full(n, lanes - 1)
+    lane[::5] = rng.randint(0, lanes, len(lane[::5]))
+    s = net.lane_length[0].astype(np.float64) - 20.0 - 14.0 * np.arange(n) - rng.uniform(0, 2.0, n)
+    veh = sc.corridor_vehicles(net, lane, np.zeros(n), v0f=rng.uniform(0.8, 1.2, n))
+    st = {"status": np.ones(n, np.int32), "lane": lane.astype(np.int32), "s": s, "v": rng.uniform(4.0, 12.0, n),
+          "rc": np.zeros(n, np.int32)}
+    if precision == 32:
+        st["s"] = st["s"].astype(np.float32).astype(np.float64)
+        st["v"] = st["v"].astype(np.float32).astype(np.float64)
+    prm = sc.Params(seed=7, p_attempt=1.0, a_th=-3.0)
+    sim = binding.Simulation(net, veh, prm, precision=precision)
+    assert sim.step_launches() == 2
+    ora = oracle.Oracle(net, veh, prm)
+    for o in (sim, ora):
+        o.set_state(st["status"], st["lane"], st["s"], st["v"], st["rc"], 0)
+    if precision == 32:  # (against the placement by slots, bit for bit)
+        other = binding.Simulation(net, large._more(veh), prm)
+        assert other.step_launches() == 3
+        large._set(other, st, n + large.ADDED)
+        for _ in range(12):
+            sim.step(1); other.step(1)
+            large._same(sim, other, n)
+        return
+    for _ in range(12):
+        sim.step(1); ora.step(1)
+        _check(sim, ora)
+    assert sim.metrics()["lane_changes"] > n // 4
+
+
+def test_flowing_city_does_not_wait_for_entrants():
+    """Some lane of a city in flowing traffic takes several entrants in every step: the placement, at 0.47 of the
+    decision's time (0.80 with a lane's entrants one after the other), stays below 0.62 of it."""
+    from perf import cases
+    sim = cases.prepare({"kind": "sim", "net": "city", "side": 30, "lanes": 3, "length": 300.0, "trips": 50000,
+                         "steps": 10, "read": "observe", "precision": 32, "groups": False, "policy": "fixed"}, 7)["sim"]
+    assert sim.step_launches() == 2
+    sim.step(2000)
+    share = []
+    for _ in range(9):
+        sim.set_kernel_timing(True)
+        sim.step(16)
+        sim.synchronize()
+        ms, _ = sim.kernel_times()
+        share.append(ms["place"] / ms["decide"])
+        sim.set_kernel_timing(False)
+    assert np.median(share) < 0.62, share
