@@ -374,16 +374,22 @@ size_t sv_size(int precision) { return precision == 64 ? sizeof(SV<double>) : si
 
 // The placement as one kernel (k_place), or as k_lanescan and k_place_slots
 // for handles of more weight (half-slots: a vehicle 2, a lane PLACE_LANE_W).
-// us per step, one kernel / two, trips and lanes:
-//   36,000 on 14,064:  23.6 / 25.1     75,000 on  30,288: 27.4 / 26.3
-//   50,000 on 19,428:  24.8 / 25.0    100,000 on  40,704: 27.9 / 27.1
-//   20,000 on 40,704:  22.8 / 24.1     50,000 on  72,660: 27.0 / 26.3
-//    4,000 on  2,424:  18.9 / 21.1     20,000 on 361,802: 25.4 / 24.7
-// (FP64 alike: 38.0 / 38.8 at 36,000 trips, 57.0 / 55.7 at 100,000).
-constexpr long long PLACE_MAX_WEIGHT = 240000;
-constexpr int PLACE_SHIFT = 9;
+// us per step, one kernel / two, in queued and in flowing traffic (trips on
+// lanes, weight):
+//    50,000 on  19,428, 178,000: 19.6 / 21.9     100,000 on  40,704,   363,000: 22.8 / 25.0, 27.5 / 28.6
+//   100,000 on  72,806, 491,000: 26.9 / 28.9     200,000 on  81,168,   725,000: 31.8 / 34.3
+//   250,000 on  72,806, 791,000: 36.0 / 37.5     350,000 on  88,305, 1,053,000: 37.5 / 39.7, 39.8 / 42.1
+//   500,009 on  72,806, 1,291,000: 46.2 / 47.7   200,000 on 362,353, 1,849,000: 39.6 / 34.7
+//   500,000 on 209,868, 1,839,000: 49.6 / 47.9   2.1 million in 64 scenarios: 130 / 119
+// and 12 slots of 350,000 trips, about 1,250,000: 41.3 / 40.9.  FP64 alike.
+constexpr long long PLACE_MAX_WEIGHT = 1200000;
 long long place_weight(const MossHandle* h) { return 2ll * h->n_veh + (long long)PLACE_LANE_W * h->n_lanes; }
 bool fused_place(const MossHandle* h) { return place_weight(h) <= PLACE_MAX_WEIGHT; }
+
+// log2 of the half-slots of a tile: at least one slot per thread; twice that
+// past 4.5 tiles per SM (200,000 trips on 81,168 lanes: 34.3 -> 31.8 us)
+int place_shift(const MossHandle* h) { return 2 * (place_weight(h) >> 9) <= 9ll * h->sm_count ? 9 : PLACE_SHIFT_MAX; }
+int place_tiles(const MossHandle* h) { return (int)(place_weight(h) >> place_shift(h)) + 1; }
 
 // lanes per thread of a round of the scan, over 4 (the single launch has the
 // default's)
@@ -427,7 +433,7 @@ Ctx<Real> make_ctx(MossHandle* h, int cur) {
     c.tile_cur = h->d_tiles[cur]; c.tile_nxt = h->d_tiles[1 - cur];
     c.tile_shift = scan_shift(h); c.slot_w = 0; c.lane_w = 1;
     if (fused_place(h)) {
-        c.tile_shift = PLACE_SHIFT; c.slot_w = 2; c.lane_w = PLACE_LANE_W;
+        c.tile_shift = place_shift(h); c.slot_w = 2; c.lane_w = PLACE_LANE_W;
     }
     c.cand_late = h->d_cand_late;
     c.cands = (Cand<Real>*)h->d_cands; c.gap_head = h->d_gap_head;
@@ -464,7 +470,7 @@ Grids grids(const MossHandle* h) {
     g.decide_work = std::max(1, std::min((h->n_veh + 31) / 32, h->sm_count * h->cfg_decide));
     g.decide_ins = extra_blocks(h);
     g.scan = 0;
-    g.place = (int)(place_weight(h) >> PLACE_SHIFT) + 1 + h->n_junc_chunks + 1;
+    g.place = place_tiles(h) + h->n_junc_chunks + 1;
     if (!fused_place(h)) {
         g.scan = ((h->n_lanes - 1) >> scan_shift(h)) + 1 + h->n_junc_chunks + 1;
         g.place = std::min(2 * (h->n_veh / TILE + 1), h->sm_count * h->cfg_place);
@@ -878,7 +884,7 @@ int device_setup(MossHandle* h, void* stream) {
     TRY(upload(h, &h->d_enter, std::vector<int32_t>(NL, 0)));
     TRY(upload(h, &h->d_leave, std::vector<int32_t>(NL, 0)));
     // tiles under any schedule
-    h->max_tiles = std::max<size_t>(SCAN_MAX_TILES, (PLACE_MAX_WEIGHT >> PLACE_SHIFT) + 1);
+    h->max_tiles = std::max(SCAN_MAX_TILES, fused_place(h) ? place_tiles(h) : 0);
     for (int k = 0; k < 2; ++k) {
         TRY(dalloc(h, &h->d_tiles[k], h->max_tiles + 1));
         TRY(dalloc(h, &h->d_delta[k], h->max_tiles));
