@@ -443,8 +443,8 @@ int moss_slot_set_horizon(moss_t h, int slot, int64_t stop_at);
  * while enabled).  moss_kernel_times returns the summed milliseconds per
  * kernel since enabling, in the order (decide, lanescan, place, resolve), and
  * the number of timed steps.  The resolution of lane-change candidates is
- * part of decide (resolve stays 0), and up to 200,000 vehicles the lane scan
- * is part of place (lanescan stays 0).
+ * part of decide (resolve stays 0), and where a step has two kernels
+ * (moss_step_launches) the lane scan is part of place (lanescan stays 0).
  */
 int moss_set_kernel_timing(moss_t h, int enable);
 int moss_kernel_times(moss_t h, double* ms4, int64_t* steps);
@@ -452,8 +452,8 @@ int moss_kernel_times(moss_t h, double* ms4, int64_t* steps);
 /*
  * Launch form of a step (no counterpart in the paper, whose step is a
  * sequence of kernels on several streams, App. B.2): mode 0 (the default)
- * replays two or three kernels per step from a captured CUDA graph; mode 1 runs the
- * whole step as one cooperative launch (every block resident at once, the
+ * replays two or three kernels per step (moss_step_launches) from captured CUDA
+ * graphs; mode 1 runs the whole step as one cooperative launch (every block resident at once, the
  * kernels' work as phases separated by grid-wide barriers whose waits are
  * bounded: MOSS_ETIMEOUT), also graph-replayed.  Results do not depend on
  * the mode.  Waits for the handle's stream and re-captures the graphs.
@@ -462,9 +462,9 @@ int moss_kernel_times(moss_t h, double* ms4, int64_t* steps);
  */
 int moss_set_step_mode(moss_t h, int mode);
 
-/* Kernel launches of the library per step in the current mode (mode 0: 2 up to
- * 200,000 vehicles, decide and place; 3 above: decide, lane scan, place; mode
- * 1: 1). */
+/* Kernel launches of the library per step in the current mode.  Mode 0: 2
+ * (decide, place) up to 2 x vehicles + 4 x lanes of 1,200,000, capacities in
+ * slot batches; 3 above (decide, lane scan, place by slots).  Mode 1: 1. */
 int moss_step_launches(moss_t h, int* out);
 
 /*

@@ -12,13 +12,16 @@
 // search in the adjacent lane's segment (adjacent lanes of a road are
 // adjacent in memory).
 //
-// One step = two kernels:
+// One step = k_decide, then the placement as one kernel (k_place) or, in
+// handles of many vehicles or lanes (PLACE_MAX_WEIGHT on the host), as two
+// (k_lanescan, k_place_slots):
 //   k_decide    per vehicle: sensing, IDM (App. B.3 eqs. (1)-(2)), the
-//               randomized MOBIL decision (App. B.3; run from a per-warp
-//               shared-memory queue of the vehicles whose attempt draw
-//               passed), ballistic integration with clamps, transfer at lane
-//               ends and arrival (App. B.2 update stream 1); each block
-//               takes a run of whole roads and at its end resolves the
+//               randomized MOBIL decision (App. B.3; the vehicles whose
+//               attempt draw passed are packed in shared memory: FP32 a queue
+//               per warp, one thread per vehicle; FP64 a queue per block, a
+//               thread per side), ballistic integration with clamps, transfer
+//               at lane ends and arrival (App. B.2 update stream 1); each
+//               block takes a run of whole roads and at its end resolves the
 //               lane-change candidates of its run (deterministic conflict
 //               rule between candidates entering the same gap from both
 //               sides); extra blocks run the departure insertion (App. B.2
@@ -29,8 +32,12 @@
 //               their lane keep their relative order (no overtaking within a
 //               lane), vehicles that entered a lane are merged by (s, id);
 //               other blocks: signal states of the next step (§3.2 policies),
-//               scenario clocks, the fit of the next step's run weight.
-// (k_step_coop runs the same two as phases of one cooperative launch.)
+//               scenario clocks, the fit of the next step's run weight;
+//   k_lanescan  the offsets of the next snapshot alone, tiles of lanes; other
+//               blocks: signal states, the fit;
+//   k_place_slots  the next snapshot by slots and entrants; the clocks.
+// (k_step_coop runs the kernels of the handle's form as phases of one
+// cooperative launch.)
 #pragma once
 
 #include <cuda/atomic>
@@ -66,8 +73,8 @@ enum : int { ERR_TIMEOUT = 1, ERR_ROUTE = 2, ERR_TRANSFER = 4, ERR_RANGE = 8 };
 // of the handle returns at once and the host reports the error
 constexpr int ERR_POISON = ERR_TIMEOUT | ERR_RANGE;
 
-constexpr int TILE = 256;           // slots per tile of k_decide / k_place (= threads)
-constexpr int JUNC_CHUNK = 256;     // junctions per k_place block (one per thread)
+constexpr int TILE = 256;           // threads per block of the step's kernels, slots per pass
+constexpr int JUNC_CHUNK = 256;     // junctions per block of the kernel after k_decide (one per thread)
 constexpr int RUNSTAT_MAX = 4096;  // k_decide work blocks whose run statistics are kept
 constexpr long long SPIN_LIMIT = 1ll << 22;  // bounded waits (~0.5 s with backoff)
 
@@ -210,17 +217,18 @@ struct Ctx {
     RecB* eb;
     int32_t* enext;       // per-lane singly linked list of entrants
     unsigned long long* head;  // [n_lanes] (tag << 32 | entrant) or stale
-    int32_t* enter;       // [n_lanes], zeroed by k_place after use
-    int32_t* leave;       // [n_lanes], zeroed by k_place after use
+    int32_t* enter;       // [n_lanes], zeroed after use by the kernel that writes the offsets (k_place or k_lanescan)
+    int32_t* leave;       // [n_lanes], likewise
     Cand<Real>* cands;    // this step's lane-change candidates (cnt->n_cand of them)
     int32_t* cand_late;   // [n_veh] candidates of a run past its block's own list, from the run's first slot on
     unsigned long long* gap_head;  // [n_veh + n_lanes + 1] (tag << 32 | candidate) or stale
-    int32_t* tile_delta;  // vehicles that enter minus vehicles that leave the lanes of a k_place tile this step
-    int32_t* delta_nxt;   // the next step's, cleared by k_place
+    int32_t* tile_delta;  // vehicles that enter minus vehicles that leave the lanes of a tile (k_place's or k_lanescan's)
+                          // this step
+    int32_t* delta_nxt;   // the next step's, cleared by the same kernel
     int32_t* tile_cur;    // k_place tiles of this step: tile t holds the lanes [tile_cur[t], tile_cur[t+1])
     int32_t* tile_nxt;    // the next step's, written by k_place
     int tile_shift;       // a tile ends where slot_w * off[l] + lane_w * l passes a multiple of 1 << tile_shift
-    int slot_w, lane_w;   // weights of a slot and of a lane in the tiles
+    int slot_w, lane_w;   // weights of a slot and of a lane in the tiles (k_lanescan's: 0 and 1)
     int n_junc_chunks;
     int run_w;           // weight of a road-lane slot in k_decide's runs (junction-lane slot: 1); 0: fitted
     int4* runstat;       // [RUNSTAT_MAX] per k_decide work block: duration (ns, lo/hi), road-lane and junction-lane slots

@@ -30,7 +30,8 @@ __device__ __forceinline__ void list_push(unsigned long long* head, int32_t* ene
 }
 
 // ---------------------------------------------------------------------------
-// k_place's tile that holds lane l, whose segment starts at off
+// the tile (k_place's or k_lanescan's) that holds lane l, whose segment starts
+// at off
 template <typename Real>
 __device__ __forceinline__ int tile_key(const Ctx<Real>& c, int off, int l) {
     return (int)(((long long)off * c.slot_w + (long long)c.lane_w * l) >> c.tile_shift);
@@ -63,7 +64,7 @@ __device__ __forceinline__ void count_move(const Ctx<Real>& c, int l, int m) {
     }
 }
 
-// A k_decide block's lane-change candidates: their candidates: their indices in the candidate
+// A k_decide block's lane-change candidates: their indices in the candidate
 // list, resolved by the block once its run is done.  The first cand_cap of
 // them (a schedule value, at most CAND_LOCAL) are listed in shared memory,
 // the rest in the run's own part of cand_late, which starts at the run's
@@ -377,10 +378,11 @@ __device__ __forceinline__ void mobil_finish(const Ctx<Real>& c, const MobilQueu
 // warp is active or all are, so what counts is the number of warps that run
 // each part: against a queue per warp and one thread for the whole of a
 // vehicle's MOBIL, the vehicles of all warps are packed and the second side
-// costs only those that have one.  30x30 grid in FP64: k_decide 132 -> 62 us
-// a step.  In FP32, where latency or instruction issue bounds the kernel, the
-// exchange and the three barriers cost more than that saves (30x30 grid under
-// an agent's phases 32.0 -> 33.5 us a step, city 110 -> 165 us): the form above.
+// costs only those that have one.  30x30 grid of 100,000 trips in FP64:
+// k_decide 157 -> 61 us a step between its events.  In FP32, where latency
+// bounds the kernel, the exchange and the three barriers cost more than that
+// saves (4x4 to 30x30 grids 0 to 8% slower, 350,000 trips in 12 slots 46 -> 54
+// us a step): the form above.
 template <typename Real>
 struct WideQueue {
     Real a[TILE], gap[TILE], sgap[TILE];          // own-lane kinematics (LaneAcc)
@@ -531,11 +533,13 @@ __device__ __forceinline__ void wide_finish(const Ctx<Real>& c, WideQueue<Real>&
 }
 
 // ---------------------------------------------------------------------------
-// k_decide: blocks [0, n_work) take 256-slot tiles of the current snapshot
-// (one vehicle per thread); blocks [n_work, gridDim) run the insertion.
+// k_decide: blocks [0, n_work) take runs of slots of the current snapshot, 256
+// at a time (one vehicle per thread); blocks [n_work, gridDim) run the
+// insertion and add up the phase pressures of the max-pressure junctions.
 // Per vehicle: the own-lane acceleration and the attempt draw, MOBIL if the
-// draw passed (from the warp's queue, above), then the update; lane-change
-// candidates are finished at the end of the block's run.
+// draw passed (from the warp's queue in FP32, the block's in FP64), then the
+// update; lane-change candidates are finished at the end of the block's run,
+// or with the queue where one round of it holds the run (FP64).
 // Groups: the network has lane groups (some road has a turn that not all of
 // its lanes serve), so the mandatory changes of R27 can occur; without them
 // that path is not compiled in.
@@ -555,7 +559,7 @@ __host__ __device__ constexpr int decide_min_blocks() {
 // The run of slots [*sb, *se) of work block vb of n_work.  A vehicle on a
 // road lane costs about twice one on a junction lane (MOBIL, longer
 // neighbour searches), so the runs split the snapshot by weight: run_w (a
-// schedule choice, 2 by default) per road-lane slot, 1 per junction-lane
+// schedule choice, fitted by default) per road-lane slot, 1 per junction-lane
 // slot, from the current lane offsets at the lane ranges of each scenario
 // (road lanes first, then junction lanes), when blocks take four tiles or
 // more each; then each end moves back to the start of its road.  The runs
@@ -655,7 +659,7 @@ __device__ __forceinline__ void decide_run(const Ctx<Real>& c, int n, int n_work
 // The work of block vb of nvb (k_decide's grid, or a virtual block of the
 // single-launch step): vb < n_work takes a run of slot tiles, the others run
 // the insertion and add up the phase pressures of the max-pressure junctions
-// (k_place advances those).
+// (the kernel after it advances those).
 template <typename Real, bool Groups>
 __device__ __forceinline__ void decide_block(const Ctx<Real>& c, int n_work, int vb, int nvb) {
     constexpr bool Wide = wide_form<Real>();
