@@ -49,15 +49,21 @@ __device__ __forceinline__ void count_enter(const Ctx<Real>& c, int l) {
     atomicAdd(&c.tile_delta[tile_key(c, c.slot_w ? c.cur.off[l] : 0, l)], 1);
 }
 
-// a vehicle goes from lane l to lane m.  Within a tile nothing grows: nearly
-// all lane changes, whose atomics on a few words would otherwise queue up when
-// many vehicles change at once (18,098 of 67,769 in a step, 7 scan tiles:
-// k_decide 49.4 -> 32.6 us)
+// a vehicle goes from lane l to lane m.  Within a scan tile nothing grows:
+// nearly all lane changes, whose atomics on a few words would otherwise queue
+// up when many vehicles change at once (18,098 of 67,769 in a step, 7 scan
+// tiles: k_decide 49.4 -> 32.6 us).  The tiles of k_place are many, and the
+// comparison would wait there for both lanes' offsets.
 template <typename Real>
 __device__ __forceinline__ void count_move(const Ctx<Real>& c, int l, int m) {
+    if (c.slot_w) {
+        count_leave(c, l);
+        count_enter(c, m);
+        return;
+    }
     atomicAdd(&c.leave[l], 1);
     atomicAdd(&c.enter[m], 1);
-    const int from = tile_key(c, c.slot_w ? c.cur.off[l] : 0, l), to = tile_key(c, c.slot_w ? c.cur.off[m] : 0, m);
+    const int from = l >> c.tile_shift, to = m >> c.tile_shift;
     if (from != to) {
         atomicAdd(&c.tile_delta[from], -1);
         atomicAdd(&c.tile_delta[to], 1);
